@@ -4,16 +4,20 @@
 // name from those three macros and includes this file; every wrapper checks
 // that the (dim, prec) it is asked for is its own.
 #pragma once
+#include <cmath>
 #include <type_traits>
 
 #include "kernels.cuh"
 #include "kernels_def.cuh"
+#include "kernels_patch.cuh"
 
 namespace pmg {
 namespace PMG_KNS {
 
-using TP = std::conditional_t<PMG_PREC == 0, double, float>;
 constexpr int DP = PMG_DIM;
+// the Cartesian patches of this part are solved by the dense sector products
+// (K = 1: pointwise) instead of sum factorisation
+constexpr bool kDense = K == 1 || Dense<DP, TP>::ok();
 
 static bool mine(int dim, int prec) { return dim == DP && prec == PMG_PREC; }
 
@@ -144,11 +148,50 @@ static unsigned persistent_grid(const void* kern, int threads, int smem, int64_t
 }
 
 template <int DIM, typename T>
+static DenseJob<T> dense_job(const T* r, T* dst, int n, const PatchParamsHost& H) {
+  DenseJob<T> J{};
+  J.r = r;
+  J.dst = dst;
+  J.table = (const uint4*)H.table;
+  J.n = n;
+  J.colour = H.colour;
+  const double c = (H.colour < 0 ? H.omega_as : 1.0) * (K == 1 ? H.inv_a0 : 1.0 / H.scale);
+  J.c = (T)c;
+  int e = 0;
+  const bool finite = std::isfinite(c);
+  J.cmul = finite ? (unsigned long long)std::ldexp(std::frexp(c, &e), 64) : 0;
+  // the operands are scaled by 2^(1080 - SH - e_patch), the products by 2^-52 (dense_body)
+  constexpr int SH = Sectors<DIM>::SPLIT ? DIM + 3 : 3;
+  J.vexp = finite ? e - 64 + 52 - (1080 - SH) : 0;
+  J.npatch = (uint32_t)patch_count(DIM, n, H.colour);
+  J.d0 = FastDiv(std::max(1, patch_count_1d(n, H.colour, 0)));
+  J.d1 = FastDiv(DIM == 3 ? std::max(1, patch_count_1d(n, H.colour, 1)) : 1);
+  return J;
+}
+
+// patches per block of the dense kernels
+template <int DIM, typename T>
+constexpr uint32_t dense_batch() { return K == 1 ? 256 : Dense<DIM, T>::P; }
+
+template <int DIM, typename T>
+static cudaError_t patch_dense_t(const T* r, T* dst, int n, const PatchParamsHost& H, cudaStream_t st) {
+  if (patch_count(DIM, n, H.colour) > 0xFFFFFFFFll - 256) return cudaErrorInvalidConfiguration;
+  const DenseJob<T> J = dense_job<DIM, T>(r, dst, n, H);
+  const unsigned grid = (J.npatch + dense_batch<DIM, T>() - 1) / dense_batch<DIM, T>();
+  if constexpr (K == 1) patch_point_kernel<DIM, T><<<grid, 256, 0, st>>>(J);
+  else patch_dense_kernel<DIM, T><<<grid, 32 * Dense<DIM, T>::NW, Dense<DIM, T>::SMEM, st>>>(J);
+  g_launches += 1;
+  return cudaGetLastError();
+}
+
+template <int DIM, typename T>
 static cudaError_t patch_cart_t(const T* r, T* dst, int n, int ppc, int n_iter, const T* dinv,
                                 const PatchParamsHost& H, int* counter, cudaStream_t st) {
   using S = PatchShape<DIM>;
   const int64_t np = patch_count(DIM, n, H.colour);
   if (np == 0) return cudaSuccess;  // no interior vertex (of this colour), no patch
+  if constexpr (kDense) return patch_dense_t<DIM, T>(r, dst, n, H, st);
+  else {
   if (ppc < 1 || ppc > kMaxPatchesPerBlock) return cudaErrorInvalidValue;
   const int64_t nbatch = (np + ppc - 1) / ppc;
   // more patch lines than threads is fine: every step loops over its lines
@@ -171,6 +214,7 @@ static cudaError_t patch_cart_t(const T* r, T* dst, int n, int ppc, int n_iter, 
                                                          counter, nbatch);
   g_launches += 1;
   return cudaGetLastError();
+  }
 }
 
 static cudaError_t patch_cart(int dim, int prec, const void* r, void* dst, int n, int ppc, int n_iter,
@@ -194,6 +238,8 @@ static cudaError_t patch_cart_il_t(const T* r, T* dst, int n, int threads, int n
                                    const PatchParamsHost& H, int* counter, cudaStream_t st) {
   const int64_t np = patch_count(DIM, n, H.colour);
   if (np == 0) return cudaSuccess;
+  if constexpr (kDense) return patch_dense_t<DIM, T>(r, dst, n, H, st);
+  else {
   const int prec = sizeof(T) == 8 ? 0 : 1;
   const int il = patch_il_of(DIM, prec, n_iter);
   if (il == 0 || threads < 32 || threads > 1024 || threads % 32) return cudaErrorInvalidValue;
@@ -214,6 +260,7 @@ static cudaError_t patch_cart_il_t(const T* r, T* dst, int n, int threads, int n
                                                             counter, nbatch);
   g_launches += 1;
   return cudaGetLastError();
+  }
 }
 
 static cudaError_t patch_cart_il(int dim, int prec, const void* r, void* dst, int n, int threads, int n_iter,
@@ -390,6 +437,26 @@ static cudaError_t cart_apply_ff_group(int dim, int count, const ApplyJob* jobs,
 template <int DIM, typename T>
 static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int ppc, int n_iter, const T* dinv,
                                       int* counter, cudaStream_t st) {
+  if constexpr (kDense) {
+    GroupOf<DenseJob<T>> G;
+    G.count = 0;
+    G.start[0] = 0;
+    int64_t grid = 0;
+    for (int j = 0; j < count; ++j) {
+      const int64_t np = patch_count(DIM, jobs[j].n, jobs[j].P.colour);
+      if (np == 0) continue;  // no patch (of this colour) on this job's level
+      if (np > 0xFFFFFFFFll - 256) return cudaErrorInvalidConfiguration;
+      G.job[G.count++] = dense_job<DIM, T>((const T*)jobs[j].r, (T*)jobs[j].dst, jobs[j].n, jobs[j].P);
+      grid += (np + dense_batch<DIM, T>() - 1) / dense_batch<DIM, T>();
+      G.start[G.count] = grid;
+    }
+    if (G.count == 0) return cudaSuccess;
+    if (grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
+    if constexpr (K == 1) patch_point_group_kernel<DIM, T><<<(unsigned)grid, 256, 0, st>>>(G);
+    else patch_dense_group_kernel<DIM, T><<<(unsigned)grid, 32 * Dense<DIM, T>::NW, Dense<DIM, T>::SMEM, st>>>(G);
+    g_launches += 1;
+    return cudaGetLastError();
+  } else {
   using S = PatchShape<DIM>;
   if (ppc < 1 || ppc > kMaxPatchesPerBlock) return cudaErrorInvalidValue;
   GroupOf<PatchJob<T>> G;
@@ -426,6 +493,89 @@ static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int 
   patch_cart_group_kernel<DIM, T><<<grid, threads, smem, st>>>(ppc, n_iter, dinv, dinv_len(DIM), counter, nbatch, G);
   g_launches += 1;
   return cudaGetLastError();
+  }
+}
+
+// ---------------------------------------------------------------- dense patch operator
+// Device bytes of the part's table of sector matrices (0: not a dense part)
+// and of the FP64 scratch its set-up needs: columns, entries, statistics.
+static int64_t patch_table_bytes(int dim, int prec) {
+  if (!mine(dim, prec) || !kDense || K == 1) return 0;
+  return Dense<DP, TP>::TABLE_BYTES;
+}
+
+static int64_t patch_scratch_bytes(int dim) {
+  using S = Sectors<DP>;
+  return dim == DP ? 8 * ((int64_t)S::ORBITS * S::NODES + S::ENTRIES) + 4 * (S::ROWS + 4) : 0;
+}
+
+// FP64 part: sector matrices of the local solver (unit scale; dinv: its
+// inverse diagonals) into the scratch: entries, columns, the classes' least
+// row exponents (4) and the row exponents
+template <int DIM>
+static int64_t scratch_ints() { return (int64_t)Sectors<DIM>::ORBITS * Sectors<DIM>::NODES + Sectors<DIM>::ENTRIES; }
+
+template <int DIM, typename V>
+static cudaError_t patch_columns(const PatchParamsHost& H, int n_iter, const double* dinv, double* columns,
+                                 cudaStream_t st) {
+  const int np = std::max(1, 32 / PatchShape<DIM>::TPP);  // few: a block's FP64 work is its latency
+  const int threads = std::min(256, (np * PatchShape<DIM>::TPP + 31) / 32 * 32);
+  const int smem = np * PatchShape<DIM>::ELEMS * (int)sizeof(V);
+  if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
+  for (int it = 0; it < n_iter; ++it)
+    patch_columns_kernel<DIM, V><<<(Sectors<DIM>::ORBITS + np - 1) / np, threads, smem, st>>>(
+        columns, np, it == 0, dinv, to_params<double>(H));
+  g_launches += n_iter;
+  return cudaGetLastError();
+}
+
+// the patches of K = 8 in 3D do not fit a block in pairs of doubles
+template <int DIM>
+constexpr bool columns_dd() { return PatchShape<DIM>::ELEMS * 16 <= kMaxDynSmem; }
+
+template <int DIM, typename T>
+static cudaError_t patch_entries_t(const PatchParamsHost& H, int n_iter, bool fp64, const double* dinv,
+                                   double* scratch, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8 && K > 1) {
+    using S = Sectors<DIM>;
+    double* columns = scratch + S::ENTRIES;
+    int* minexp = (int*)(scratch + scratch_ints<DIM>());
+    cudaError_t e = cudaMemsetAsync(minexp, 0x7F, 16, st);
+    if (e != cudaSuccess) return e;
+    if constexpr (columns_dd<DIM>())
+      e = fp64 ? patch_columns<DIM, dd>(H, n_iter, dinv, columns, st)
+               : patch_columns<DIM, double>(H, n_iter, dinv, columns, st);
+    else e = patch_columns<DIM, double>(H, n_iter, dinv, columns, st);
+    if (e != cudaSuccess) return e;
+    patch_entries_kernel<DIM><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, scratch, minexp + 4, minexp);
+    g_launches += 1;
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
+static cudaError_t patch_entries(int dim, const PatchParamsHost& H, int n_iter, int prec, const double* dinv,
+                                 double* scratch, cudaStream_t st) {
+  if (dim != DP) return cudaErrorInvalidValue;
+  return patch_entries_t<DP, TP>(H, n_iter, prec == 0, dinv, scratch, st);
+}
+
+// the part's table from the scratch
+template <int DIM, typename T>
+static cudaError_t patch_table_t(const double* scratch, void* table, cudaStream_t st) {
+  if constexpr (kDense && K > 1) {
+    const int* minexp = (const int*)(scratch + scratch_ints<DIM>());
+    const int64_t work = (int64_t)Sectors<DIM>::TILES * 128;
+    patch_table_kernel<DIM, T><<<(unsigned)((work + 255) / 256), 256, 0, st>>>(scratch, minexp + 4, minexp, (uint32_t*)table);
+    g_launches += 1;
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
+static cudaError_t patch_table(int dim, int prec, const double* scratch, void* table, cudaStream_t st) {
+  if (!mine(dim, prec)) return cudaErrorInvalidValue;
+  return patch_table_t<DP, TP>(scratch, table, st);
 }
 
 static cudaError_t patch_cart_group(int dim, int prec, int count, const PatchSolveJob* jobs, int ppc, int n_iter,
@@ -575,16 +725,40 @@ static int max_threads_of(const void* k) {
   return a.maxThreadsPerBlock;
 }
 
+template <int DIM, typename T>
+static int cart_max_threads(bool interleaved) {
+  if constexpr (kDense) return !interleaved ? kPatchMaxThreads : (sizeof(T) == 8 ? 768 : 1024);  // no effect
+  else if (!interleaved) return max_threads_of((const void*)patch_cart_kernel<DIM, T>);
+  else return max_threads_of((const void*)patch_cart_il_kernel<DIM, T>);
+}
+
 static int patch_max_threads(int dim, int prec, int deformed) {
   if (!mine(dim, prec)) return 0;
-  return deformed ? std::min(max_threads_of((const void*)patch_def_kernel<DP, TP, float>),
-                             max_threads_of((const void*)patch_def_kernel<DP, TP, double>))
-                  : max_threads_of((const void*)patch_cart_kernel<DP, TP>);
+  if (deformed)
+    return std::min(max_threads_of((const void*)patch_def_kernel<DP, TP, float>),
+                    max_threads_of((const void*)patch_def_kernel<DP, TP, double>));
+  return cart_max_threads<DP, TP>(false);
 }
 
 static int patch_il_max_threads(int dim, int prec) {
   if (!mine(dim, prec) || patch_il<DP, TP>() == 0) return 0;
-  return max_threads_of((const void*)patch_cart_il_kernel<DP, TP>);
+  return cart_max_threads<DP, TP>(true);
+}
+
+template <int DIM, typename T, class Acc>
+static void prepare_cart(int optin, const Acc& acc) {
+  if constexpr (!kDense) {
+    acc(allow_smem(patch_cart_kernel<DIM, T>, optin));
+    acc(allow_smem(patch_cart_group_kernel<DIM, T>, optin));
+    if (patch_il<DIM, T>() > 0) acc(allow_smem(patch_cart_il_kernel<DIM, T>, optin));
+  } else if constexpr (K > 1) {
+    acc(allow_smem(patch_dense_kernel<DIM, T>, optin));
+    acc(allow_smem(patch_dense_group_kernel<DIM, T>, optin));
+  }
+  if constexpr (sizeof(T) == 8 && K > 1) {
+    acc(allow_smem(patch_columns_kernel<DIM, double>, optin));
+    if constexpr (columns_dd<DIM>()) acc(allow_smem(patch_columns_kernel<DIM, dd>, optin));
+  }
 }
 
 static cudaError_t prepare() {
@@ -594,9 +768,7 @@ static cudaError_t prepare() {
   if (e != cudaSuccess) return e;
   cudaError_t r = cudaSuccess;
   auto acc = [&](cudaError_t x) { if (x != cudaSuccess && r == cudaSuccess) r = x; };
-  acc(allow_smem(patch_cart_kernel<DP, TP>, optin));
-  acc(allow_smem(patch_cart_group_kernel<DP, TP>, optin));
-  if (patch_il<DP, TP>() > 0) acc(allow_smem(patch_cart_il_kernel<DP, TP>, optin));
+  prepare_cart<DP, TP>(optin, acc);
   acc(allow_smem(patch_def_kernel<DP, TP, float>, optin));
   acc(allow_smem(patch_def_kernel<DP, TP, double>, optin));
   acc(allow_smem(def_cell_kernel<DP, TP, float>, optin));
@@ -638,6 +810,10 @@ const KernelTable* PMG_TABLE_FN() {
       PMG_KNS::patch_gather_group,
       PMG_KNS::h_prolong_add_group,
       PMG_KNS::h_restrict_group,
+      PMG_KNS::patch_table_bytes,
+      PMG_KNS::patch_scratch_bytes,
+      PMG_KNS::patch_entries,
+      PMG_KNS::patch_table,
   };
   return &t;
 }

@@ -58,6 +58,43 @@ __device__ __forceinline__ const double* ctab<double>() { return c_tab64; }
 template <>
 __device__ __forceinline__ const float* ctab<float>() { return c_tab32; }
 
+// Pair of doubles for the set-up of the patch matrices: hi + lo, products and
+// sums with their rounding errors kept (Knuth's TwoSum, the FMA TwoProduct;
+// lo is not renormalised between operations).
+struct dd {
+  double hi, lo;
+  __device__ __forceinline__ dd() {}
+  __device__ __forceinline__ dd(double h, double l = 0.0) : hi(h), lo(l) {}
+  __device__ __forceinline__ dd& operator+=(const dd& o) {
+    const double s = __dadd_rn(hi, o.hi), b = __dsub_rn(s, hi);
+    lo += (__dsub_rn(hi, __dsub_rn(s, b)) + __dsub_rn(o.hi, b)) + o.lo;
+    hi = s;
+    return *this;
+  }
+};
+__device__ __forceinline__ dd operator+(dd a, const dd& b) { return a += b; }
+__device__ __forceinline__ dd operator-(dd a, const dd& b) { return a += dd(-b.hi, -b.lo); }
+__device__ __forceinline__ dd operator*(const dd& a, const dd& b) {
+  const double p = __dmul_rn(a.hi, b.hi);  // not fused into a later sum
+  return dd(p, fma(a.hi, b.lo, fma(a.lo, b.hi, fma(a.hi, b.hi, -p))));
+}
+__device__ __forceinline__ dd operator*(double a, const dd& b) {
+  const double p = __dmul_rn(a, b.hi);
+  return dd(p, fma(a, b.lo, fma(a, b.hi, -p)));
+}
+__device__ __forceinline__ double value_of(const dd& a) { return a.hi + a.lo; }
+__device__ __forceinline__ double value_of(double a) { return a; }
+
+// type of the 1D tables that a line pass on T reads
+template <typename T>
+struct TableOf {
+  using type = T;
+};
+template <>
+struct TableOf<dd> {
+  using type = double;
+};
+
 // ===========================================================================
 // Cartesian operator A = s * sum_dir (K on dir, M elsewhere), applied by one
 // pass per direction over the global grid (the 1D matrices are the
@@ -702,8 +739,8 @@ __device__ __forceinline__ void pfor(const PB& pb, F&& f) {
 
 // y = C x for a patch matrix of degree p (m x m, row-major), skipping the
 // structural zeros between the two cells of the patch.
-template <int p, typename T>
-__device__ __forceinline__ void pmv(const T* C, const T* x, T* y) {
+template <int p, typename TC, typename T>
+__device__ __forceinline__ void pmv(const TC* C, const T* x, T* y) {
   constexpr int m = mp(p);
 #pragma unroll
   for (int i = 0; i < m; ++i) {
@@ -719,7 +756,7 @@ __device__ __forceinline__ void pmv(const T* C, const T* x, T* y) {
 // inverse diagonal from a table shared by all patches (scale-free).
 template <int DIM, typename T>
 struct CartGeo {
-  const T* dinv;  // concatenated per-level tables, level l at dinv_off(l)
+  const typename TableOf<T>::type* dinv;  // concatenated per-level tables, level l at dinv_off(l)
   T scale;
   T inv_scale;
   T inv_a0;
@@ -729,7 +766,7 @@ struct CartGeo {
     for (int j = 1; j < l; ++j) o += ipow(mp(plev(K, j)), DIM);
     return o;
   }
-  __device__ __forceinline__ T dinv_at(int, int l, int i) const { return dinv[dinv_off(l) + i] * inv_scale; }
+  __device__ __forceinline__ T dinv_at(int, int l, int i) const { return inv_scale * dinv[dinv_off(l) + i]; }
   __device__ __forceinline__ T a0inv(int) const { return inv_a0; }
 
   // The Jacobi steps of Algorithm 3 fold into the line passes of the
@@ -746,8 +783,9 @@ struct CartGeo {
     constexpr int p = plev(K, l);
     constexpr int m = mp(p);
     constexpr int SZT = PatchShape<DIM>::SZT;
-    const T* MP = ctab<T>() + LAY.MP[l];
-    const T* KP = ctab<T>() + LAY.KP[l];
+    using TC = typename TableOf<T>::type;
+    const TC* MP = ctab<TC>() + LAY.MP[l];
+    const TC* KP = ctab<TC>() + LAY.KP[l];
     const T s = scale;
     // first pass, along x: x = d (MODE 1: computed from r and stored)
     auto first = [&](auto sm, int b, T* x) {
@@ -841,7 +879,8 @@ __device__ __forceinline__ void restrict_p(const PB& pb, int dst) {
   constexpr int m = mp(pf), mc = mp(pc);
   constexpr int SZT = PatchShape<DIM>::SZT;
   constexpr int EZ = DIM == 3 ? m : 1;
-  const T* Tr = ctab<T>() + LAY.Tr[l];  // m x mc, row-major
+  using TC = typename TableOf<T>::type;
+  const TC* Tr = ctab<TC>() + LAY.Tr[l];  // m x mc, row-major
   // x: (m, m, EZ) in t0 -> (mc, m, EZ) in t1
   pfor<m * EZ>(pb, [&](int g, int L) {
     auto sm = pb.at(g);
@@ -906,7 +945,8 @@ __device__ __forceinline__ void prolong_p(const PB& pb, int src, int dst) {
   constexpr int m = mp(pf), mc = mp(pc);
   constexpr int SZT = PatchShape<DIM>::SZT;
   constexpr int EZC = DIM == 3 ? mc : 1;
-  const T* Tr = ctab<T>() + LAY.Tr[l];
+  using TC = typename TableOf<T>::type;
+  const TC* Tr = ctab<TC>() + LAY.Tr[l];
   // x: (mc, mc, EZC) -> (m, mc, EZC) in t0
   pfor<mc * EZC>(pb, [&](int g, int L) {
     auto sm = pb.at(g);

@@ -1,0 +1,861 @@
+// Cartesian vertex-patch smoother as one matrix product per patch (included
+// by inst_k.cuh after kernels.cuh).
+//
+// On a Cartesian mesh the local solver of every patch -- Algorithm 2 around
+// the p-multigrid V-cycle of Algorithm 3, full or half -- is the same linear
+// map, up to the factor 1 / h^{d-2}: d_j = B r_j / h^{d-2}.  B is formed once
+// per method (patch_columns_kernel: the local solver applied to unit
+// vectors) and applied here to a block of patches at a time on the tensor
+// cores.  The solver commutes with the reflections of the patch in every
+// direction, so in the basis of even and odd combinations of mirrored nodes
+// B falls into 2^d independent blocks ("sectors") of K or K - 1 rows per
+// direction: (K^2 + (K-1)^2)^d products per patch in place of (2K-1)^{2d}.
+//
+// Why: sum factorisation spends seven short contractions per vmult and moves
+// every intermediate through shared memory; in FP64 it is bound by GB300's
+// FP64 pipe (1.25 TFLOP/s, two multiply-adds per clock and SM), in FP32 by
+// shared-memory traffic and the barriers between the line passes.
+//
+// FP64 arithmetic: operands in fixed point (one exponent per matrix row and per
+// patch), split into 7 signed digits of 8 bits that are exact in FP16;
+// products of digits are summed exactly by the tensor cores (integers in the
+// FP32 accumulator) and across digit pairs in 64-bit integers, keeping the 34
+// digit pairs i + j <= 7 (0-based; without i + j = 7 the error is 100 times
+// larger).  No FP64 instruction is executed.  Error of one local solve
+// against extended precision, N(0,1) residuals, before (sum factorisation)
+// and now: K = 3 3.3e-16, 3.3e-16; K = 4 3.9e-16, 3.7e-16; K = 5 3.6e-16,
+// 3.7e-16; 2D K = 7 4.1e-16, 3.1e-16.  FP32: three BF16 parts of each value
+// (8 bits each, exact), the six products of weight 2^-16 and above.
+//
+// Patch launch of one sweep, before and now (GB300): FP64 K = 4 at 32^3 cells
+// 2.344 and 0.210 ms (tensor pipe 40% of its cycles, issue slots 45%: the
+// digit conversions and the 64-bit gather and scatter); FP64 K = 5 at 24^3
+// 2.12 and 0.38 ms; FP32 K = 4 at 32^3 0.135 and 0.055 ms (shared-memory and
+// L1 wavefronts: 80% of their rate), K = 5 at 40^3 0.473 and 0.319 ms, K = 3
+// at 67^3 0.328 and 0.203 ms, K = 2 at 100^3 0.283 and 0.162 ms.
+#pragma once
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
+
+namespace pmg {
+namespace PMG_KNS {
+
+using TP = std::conditional_t<PMG_PREC == 0, double, float>;  // this part's precision
+
+// Sectors of the patch operator: sector s is odd in direction d where bit d
+// of s is set.  Even coefficients 0..K-1 (K-1: the centre node), odd ones
+// 0..K-2.  Patches of at most 32 nodes are not split: their single matrix
+// fits the same number of 16 x 16 tiles.
+template <int DIM>
+struct Sectors {
+  static constexpr int M = mp(K);
+  static constexpr int NODES = ipow(M, DIM);
+  static constexpr bool SPLIT = NODES > 32;
+  static constexpr int NS = SPLIT ? 1 << DIM : 1;
+  static constexpr int E = SPLIT ? K : M;          // coefficients per direction of an even sector
+  static constexpr int ORBITS = ipow(E, DIM);      // nodes up to reflection
+  static constexpr int IMAGES = SPLIT ? 1 << DIM : 1;
+  __host__ __device__ static constexpr int ext(int s, int d) { return d >= DIM ? 1 : ((s >> d) & 1) ? E - 1 : E; }
+  __host__ __device__ static constexpr int size(int s) { return ext(s, 0) * ext(s, 1) * ext(s, 2); }
+  __host__ __device__ static constexpr int tiles(int s) { return (size(s) + 15) / 16; }  // 16-row tiles per side
+  // offsets of sector s: padded rows, rows, 16 x 16 tiles, matrix entries
+  __host__ __device__ static constexpr int prow(int s) { int o = 0; for (int t = 0; t < s; ++t) o += 16 * tiles(t); return o; }
+  __host__ __device__ static constexpr int row(int s) { int o = 0; for (int t = 0; t < s; ++t) o += size(t); return o; }
+  __host__ __device__ static constexpr int tile(int s) { int o = 0; for (int t = 0; t < s; ++t) o += tiles(t) * tiles(t); return o; }
+  __host__ __device__ static constexpr int entry(int s) { int o = 0; for (int t = 0; t < s; ++t) o += size(t) * size(t); return o; }
+  static constexpr int PROWS = prow(NS), ROWS = row(NS), TILES = tile(NS), ENTRIES = entry(NS);
+  static_assert(ROWS == NODES, "the sectors hold every node once");
+};
+
+// An orbit: a node of the first orthant (coordinates 0..E-1) and its mirror
+// images; image b is mirrored in the directions of b's bits.
+template <int DIM>
+struct Orbit {
+  using S = Sectors<DIM>;
+  int c[3];
+  __device__ __forceinline__ explicit Orbit(int o) {
+    c[0] = o % S::E;
+    c[1] = (o / S::E) % S::E;
+    c[2] = DIM == 3 ? o / (S::E * S::E) : 0;
+  }
+  // image b is a node of its own (the centre has no mirror image); likewise
+  // the orbit has a coefficient in sector b
+  __device__ __forceinline__ bool has(int b) const {
+    bool h = true;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) h = h && !(((b >> d) & 1) && c[d] == S::E - 1);
+    return h;
+  }
+  __device__ __forceinline__ int at(int d, int b) const { return ((b >> d) & 1) ? S::M - 1 - c[d] : c[d]; }
+  __device__ __forceinline__ int node(int b) const {
+    return at(0, b) + S::M * (at(1, b) + S::M * (DIM == 3 ? at(2, b) : 0));
+  }
+  // directions in which the node is central
+  __device__ __forceinline__ int centres() const {
+    int n = 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) n += S::SPLIT && c[d] == S::E - 1;
+    return n;
+  }
+};
+
+// Lines of a patch along x up to reflection in the other directions: line L
+// holds the nodes (0..M-1, c_1, c_2), c_d < E; image b is mirrored in
+// direction d where bit d - 1 of b is set.  A thread takes all images of a
+// line, so the offsets of its nodes and coefficients along x are immediates.
+template <int DIM>
+struct Lines {
+  using S = Sectors<DIM>;
+  static constexpr int N = ipow(S::E, DIM - 1);
+  static constexpr int IMAGES = S::SPLIT ? 1 << (DIM - 1) : 1;
+  int c[2];
+  __device__ __forceinline__ explicit Lines(int L) {
+    c[0] = L % S::E;
+    c[1] = DIM == 3 ? L / S::E : 0;
+  }
+  __device__ __forceinline__ bool has(int b) const {
+    bool h = true;
+#pragma unroll
+    for (int d = 0; d < DIM - 1; ++d) h = h && !(((b >> d) & 1) && c[d] == S::E - 1);
+    return h;
+  }
+  // directions in which the line passes through the centre
+  __device__ __forceinline__ int centres() const {
+    return S::SPLIT ? (c[0] == S::E - 1) + (DIM == 3 && c[1] == S::E - 1) : 0;
+  }
+  // offset of image b's first node on a grid of N1 nodes per direction
+  __device__ __forceinline__ int node(int b, int N1) const {
+    const int y = (b & 1) ? S::M - 1 - c[0] : c[0], z = (b & 2) ? S::M - 1 - c[1] : c[1];
+    return N1 * (y + (DIM == 3 ? N1 * z : 0));
+  }
+  // first coefficient of the line in sector s
+  __device__ __forceinline__ int coef(int s) const { return S::ext(s, 0) * (c[0] + S::ext(s, 1) * c[1]); }
+};
+
+// even / odd combinations of a line's images in every direction: entry i of
+// image b becomes the coefficient of parity b in the other directions and,
+// along x, even coefficient i for i < K, odd coefficient M - 1 - i beyond.
+// (Its own inverse up to the factor 2 per direction, which the matrix absorbs.)
+template <int DIM, typename V>
+__device__ __forceinline__ void reflect(V (&v)[Lines<DIM>::IMAGES][Sectors<DIM>::M]) {
+  using S = Sectors<DIM>;
+  if constexpr (S::SPLIT) {
+#pragma unroll
+    for (int b = 0; b < Lines<DIM>::IMAGES; ++b)
+#pragma unroll
+      for (int i = 0; i < K - 1; ++i) {
+        const V e = v[b][i] + v[b][S::M - 1 - i], o = v[b][i] - v[b][S::M - 1 - i];
+        v[b][i] = e;
+        v[b][S::M - 1 - i] = o;
+      }
+#pragma unroll
+    for (int d = 0; d < DIM - 1; ++d)
+#pragma unroll
+      for (int b = 0; b < Lines<DIM>::IMAGES; ++b)
+        if (!((b >> d) & 1))
+#pragma unroll
+          for (int i = 0; i < S::M; ++i) {
+            const V e = v[b][i] + v[b | (1 << d)][i], o = v[b][i] - v[b | (1 << d)][i];
+            v[b][i] = e;
+            v[b | (1 << d)][i] = o;
+          }
+  }
+}
+
+// f(entry, sector, coefficient along x) for the entries of image b after reflect
+template <int DIM, class F>
+__device__ __forceinline__ void for_coefs(int b, F&& f) {
+  using S = Sectors<DIM>;
+#pragma unroll
+  for (int i = 0; i < S::M; ++i) {
+    if (!S::SPLIT || i < K) f(i, 2 * b, i);
+    else f(i, 2 * b + 1, S::M - 1 - i);
+  }
+}
+
+// ---------------------------------------------------------------- block shape
+// P patches per block (the n extent of the products), NW warps.  3D patches of
+// K >= 6 keep the sum-factorised kernel: their operands fill an SM's shared
+// memory with 8-16 patches, and the matrix is streamed from L2 for so few
+// columns (K = 6 FP32 at 33^3 cells: 0.67 ms against 0.49 ms).
+template <int DIM, typename T>
+struct Dense {
+  using S = Sectors<DIM>;
+  static constexpr bool F64 = sizeof(T) == 8;
+  static constexpr int SL = F64 ? 7 : 3;                        // parts per value
+  static constexpr int P = 16;
+  static constexpr int NT = P / 8;                              // 8-column tiles
+  static constexpr int NSUB = 32 / P;                           // lines a warp handles at once
+  static constexpr int UNITS = S::PROWS / 16;                   // 16-row tiles of the result
+  static constexpr int NW = UNITS >= 8 ? 8 : (UNITS > 2 ? 4 : 2);
+  static constexpr int UPW = (UNITS + NW - 1) / NW;             // units per warp
+  // Operands: FP64 fixed-point values [row][XP], FP32 the three parts as
+  // planes of BF16 [part][row][XP]; the pitch spreads the rows over the banks.
+  static constexpr int XP = F64 ? P + 4 : P + 8;
+  static constexpr int XBYTES = F64 ? S::PROWS * XP * 8 : SL * S::PROWS * XP * 2;
+  // Results [row][YP], nodal results [patch][ZP].  FP64: the results follow
+  // the operands (they first hold the gathered values), the nodal results
+  // take the operands' place; FP32: both take the operands' place.
+  static constexpr int YP = F64 ? P : P + 4;
+  static constexpr int YBYTES = (S::ROWS * YP * (int)sizeof(T) + 15) / 16 * 16;
+  static constexpr int ZP = S::NODES | 1;
+  static constexpr int ZBYTES = P * ZP * (int)sizeof(T);
+  static constexpr int max2(int a, int b) { return a > b ? a : b; }
+  static constexpr int YOFF = F64 ? (max2(XBYTES, ZBYTES) + 15) / 16 * 16 : 0;
+  static constexpr int ZOFF = F64 ? 0 : YBYTES;
+  static constexpr int SMEM = F64 ? YOFF + YBYTES : max2(XBYTES, YBYTES + ZBYTES);
+  // blocks per SM that the shared memory and 64 K registers (at least 128 a
+  // thread in FP64: 7 accumulators and 7 fragments per column tile) allow
+  static constexpr int MINB() {
+    const int bs = 227 * 1024 / (SMEM + 1536), br = 65536 / (32 * NW * (F64 ? 128 : 64)), b = bs < br ? bs : br;
+    return b < 1 ? 1 : (b > 8 ? 8 : b);
+  }
+  static constexpr bool ok() { return K >= 2 && (DIM == 2 || K <= 5) && SMEM <= kMaxDynSmem; }
+  // table: 16-byte fragments, then (FP64) per row its exponent above its
+  // class's, and the exponents of the four classes (Orbit::centres)
+  static constexpr int FRAGS = S::TILES * SL * 32;
+  static constexpr int TABLE_BYTES = FRAGS * 16 + (F64 ? S::ROWS * 4 + 16 : 0);
+};
+
+// One 16-row tile of the result: a warp's unit of work.
+struct DenseUnit {
+  short prow;   // first operand row of the sector
+  short kt;     // 16-column tiles
+  short row;    // result row of the tile
+  short valid;  // its rows that exist
+  int frag;     // first fragment (in units of 32 lanes)
+};
+template <int N>
+struct DenseUnits {
+  DenseUnit u[N];
+};
+template <int DIM, typename T>
+constexpr DenseUnits<Dense<DIM, T>::UNITS> dense_units() {
+  using S = Sectors<DIM>;
+  DenseUnits<Dense<DIM, T>::UNITS> r{};
+  int n = 0;
+  for (int s = 0; s < S::NS; ++s)
+    for (int m = 0; m < S::tiles(s); ++m) {
+      DenseUnit& u = r.u[n++];
+      u.prow = (short)S::prow(s);
+      u.kt = (short)S::tiles(s);
+      u.row = (short)(S::row(s) + 16 * m);
+      u.valid = (short)(S::size(s) - 16 * m < 16 ? S::size(s) - 16 * m : 16);
+      u.frag = (S::tile(s) + m * S::tiles(s)) * Dense<DIM, T>::SL;
+    }
+  return r;
+}
+
+// Parameters of one level's launch.  FP64: a result is its integer x cmul x
+// 2^(vexp + the patch's exponent - its class's exponent), cmul in [2^63, 2^64).
+template <typename T>
+struct DenseJob {
+  const T* r;
+  T* dst;
+  const uint4* table;
+  int n, colour;
+  T c;                       // FP32: omega_AS / scale (additive) or 1 / scale
+  unsigned long long cmul;   // FP64: the same as a normalised integer (0: not finite)
+  int vexp;                  // and its binary exponent
+  uint32_t npatch;
+  FastDiv d0, d1;            // patches per direction
+};
+
+// ---------------------------------------------------------------- FP64 <-> fixed point
+// v 2^(58 - e + 1022) truncated, for |v| < 2^(e - 1022) (e: biased exponent + 1 bound)
+__device__ __forceinline__ long long fixed_of(double v, int e) {
+  const int hi = __double2hiint(v);
+  const unsigned lo = (unsigned)__double2loint(v);
+  const int ex = (hi >> 20) & 0x7FF;
+  const unsigned mh = ((unsigned)hi & 0xFFFFFu) | (ex ? 0x100000u : 0u);
+  const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 5;
+  const int sh = min(e - (ex ? ex : 1), 63);
+  const long long x = (long long)(m >> sh);
+  const long long sg = (long long)(hi >> 31);
+  return (x ^ sg) - sg;
+}
+
+// y cmul 2^(ve + 64) rounded to nearest (ties away), in integer arithmetic
+__device__ __forceinline__ double double_of(long long y, unsigned long long cmul, int ve) {
+  const unsigned long long sg = (unsigned long long)(y >> 63);
+  const unsigned long long a = ((unsigned long long)y ^ sg) - sg;
+  if (a == 0) return 0.0;
+  const int z = __clzll((long long)a);
+  unsigned long long p = __umul64hi(a << z, cmul);  // >= 2^62
+  int ex = ve - z + 64 + 63 + 1023;                 // biased exponent of 2^63 2^(ve + 64 - z)
+  if (!(p >> 63)) {
+    p <<= 1;
+    --ex;
+  }
+  p += 0x400;                // round at bit 11
+  if (p < 0x400) {           // carried out of the top bit
+    p = 0x8000000000000000ull;
+    ++ex;
+  }
+  if (ex >= 1 && ex <= 2046) {
+    const unsigned long long m = (p >> 11) & 0xFFFFFFFFFFFFFull;
+    return __longlong_as_double((long long)(m | ((unsigned long long)ex << 52) | (sg & 0x8000000000000000ull)));
+  }
+  // overflow or a subnormal result
+  const double d = ldexp((double)(p >> 11), ex - 1023 - 52);
+  return sg ? -d : d;
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm_t(uint32_t (&b)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+               : "r"(addr));
+}
+
+constexpr int kNoExp = -(1 << 30);          // class exponent of a matrix that is not finite
+constexpr float kMagic = 12582912.0f;       // 1.5 2^23: the accumulator's bits count integers from here
+constexpr int kMagicBits = 0x4B400000;
+
+// FP64 products of one unit: result rows of sector coefficients times the
+// operand rows, in units of 2^-52 of (table integer x operand integer) at the
+// exponent of the row's class.  Two k tiles add at most 14 products of 2^18 to an
+// accumulator (below its exact range of 2^22 around kMagic) before it is
+// emptied into y.
+template <int DIM>
+__device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table, const long long* X,
+                                          long long* Y, int lane) {
+  using D = Dense<DIM, double>;
+  constexpr int SL = D::SL, NT = D::NT, ND = SL + 1;  // ND: digit sums kept, i + j < ND
+  const int g = lane >> 2, q = lane & 3;
+  const int* shift = reinterpret_cast<const int*>(table + D::FRAGS) + u.row + g;  // row exponent - its class's
+  long long y[NT][4] = {};
+  float acc[ND][NT][4];
+  auto reset = [&]() {
+#pragma unroll
+    for (int d = 0; d < ND; ++d)
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[d][t][i] = kMagic;
+  };
+  auto empty = [&]() {
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        auto pair = [&](int d) {
+          return (__float_as_int(acc[d][t][i]) - kMagicBits) * 256 + (__float_as_int(acc[d + 1][t][i]) - kMagicBits);
+        };
+        y[t][i] += ((long long)pair(0) << 36) + ((long long)pair(2) << 20) + ((long long)pair(4) << 4) +
+                   ((pair(6) + 2048) >> 12);  // rounded: a bias would add up over the mirror images
+      }
+  };
+  reset();
+  const uint4* tp = table + (int64_t)u.frag * 32 + lane;
+  for (int k = 0; k < u.kt; ++k) {
+    // digits of the operand values of rows 2q, 2q+1, 2q+8, 2q+9 of the tile
+    uint32_t b[SL][NT][2];
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long* x = X + (u.prow + 16 * k + 2 * q + 8 * h) * D::XP + 8 * t + g;
+        // biased so that byte SL - 1 - j holds digit j + 128
+        const long long w0 = x[0] + 0x0080808080808080ll, w1 = x[D::XP] + 0x0080808080808080ll;
+#pragma unroll
+        for (int j = 0; j < SL; ++j) {
+          const int byte = SL - 1 - j, bb = byte & 3;
+          const uint32_t v0 = (uint32_t)(byte < 4 ? w0 : w0 >> 32), v1 = (uint32_t)(byte < 4 ? w1 : w1 >> 32);
+          const uint32_t pr = __byte_perm(v0, v1, bb | (bb << 4) | ((4 + bb) << 8) | ((4 + bb) << 12));
+          const uint32_t hb = (pr & 0x00FF00FFu) | 0x64006400u;  // 1024 + digit + 128 as halves
+          const __half2 dg = __hsub2(*reinterpret_cast<const __half2*>(&hb), __half2half2(__ushort_as_half(0x6480)));
+          b[j][t][h] = *reinterpret_cast<const uint32_t*>(&dg);
+        }
+      }
+#pragma unroll
+    for (int i = 0; i < SL; ++i) {
+      const uint4 a = __ldg(tp + (k * SL + i) * 32);
+#pragma unroll
+      for (int j = 0; j < SL; ++j)
+        if (i + j < ND) {
+#pragma unroll
+          for (int t = 0; t < NT; ++t) mma_f16(acc[i + j][t], a, b[j][t][0], b[j][t][1]);
+        }
+    }
+    if ((k & 1) && k + 1 < u.kt) {
+      empty();
+      reset();
+    }
+  }
+  empty();
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (g + 8 * h < u.valid) {
+      const int sh = __ldg(shift + 8 * h);
+      const long long half = (1ll << sh) >> 1;
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) Y[(u.row + g + 8 * h) * D::YP + 8 * t + 2 * q + i] = (y[t][2 * h + i] + half) >> sh;
+    }
+}
+
+// FP32 products of one unit into y.  The leading products are taken out of
+// the accumulator after every k tile and summed with rounding (the tensor
+// cores truncate their sums); the five small products share an accumulator.
+template <int DIM>
+__device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table, const uint16_t* X,
+                                          float (&y)[Dense<DIM, float>::NT][4], int lane) {
+  using D = Dense<DIM, float>;
+  using S = Sectors<DIM>;
+  constexpr int SL = D::SL, NT = D::NT;
+  float lo[NT][4] = {};
+#pragma unroll
+  for (int t = 0; t < NT; ++t)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y[t][i] = 0.f;
+  const uint4* tp = table + (int64_t)u.frag * 32 + lane;
+  // ldmatrix source row of this lane: (k 0-7 | 8-15) x (n 0-7 | 8-15)
+  const uint32_t xa = (uint32_t)__cvta_generic_to_shared(X) +
+                      2 * ((u.prow + 8 * ((lane >> 3) & 1) + (lane & 7)) * D::XP + 8 * (lane >> 4));
+  for (int k = 0; k < u.kt; ++k) {
+    uint4 a[SL];
+#pragma unroll
+    for (int i = 0; i < SL; ++i) a[i] = __ldg(tp + (k * SL + i) * 32);
+#pragma unroll
+    for (int t = 0; t < NT; t += 2) {
+      uint32_t b[SL][4];
+#pragma unroll
+      for (int j = 0; j < SL; ++j) ldsm_t(b[j], xa + 2 * ((j * S::PROWS + 16 * k) * D::XP + 8 * t));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float hi[4] = {};
+        mma_bf16(hi, a[0], b[0][2 * h], b[0][2 * h + 1]);
+#pragma unroll
+        for (int j = 0; j < SL; ++j)
+#pragma unroll
+          for (int i = 0; i + j < SL; ++i)
+            if (i + j > 0) mma_bf16(lo[t + h], a[i], b[j][2 * h], b[j][2 * h + 1]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[t + h][i] += hi[i];
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < NT; ++t)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) y[t][i] += lo[t][i];
+}
+
+static __constant__ const DenseUnits<Dense<PMG_DIM, TP>::UNITS> c_units = dense_units<PMG_DIM, TP>();
+
+// The patches of batch `batch` of a level: gather r_j, even / odd
+// combinations, products, and back; omega_AS d_j to the colour's vector
+// (additive) or d_j added to u (multiplicative).  A lane holds one patch (P
+// lanes) and the warps share the nodes, so index arithmetic is uniform and
+// shared-memory accesses fall on consecutive patches.
+template <int DIM, typename T>
+__device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch) {
+  using S = Sectors<DIM>;
+  using D = Dense<DIM, T>;
+  constexpr int P = D::P, NSUB = D::NSUB, NW = D::NW;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int64_t s_base[P];
+  __shared__ int s_colour[P];
+  __shared__ unsigned s_max[P];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pn = lane % P, item0 = warp * NSUB + lane / P;
+  constexpr int STEP = NW * NSUB;
+  const int N1 = K * J.n + 1;
+  // this lane's patch (patch_meta_init's order)
+  const uint32_t pid = batch * P + pn;
+  const bool active = pid < J.npatch;
+  int64_t base;
+  {
+    const uint32_t t = active ? pid : 0, r1 = J.d0.div(t), r2 = J.d1.div(r1);
+    const int i[3] = {(int)(t - r1 * J.d0.d), (int)(DIM == 3 ? r1 - r2 * J.d1.d : r1), (int)(DIM == 3 ? r2 : 0)};
+    int v[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      v[d] = J.colour < 0 ? i[d] + 1 : 2 * i[d] + (((J.colour >> d) & 1) ? 1 : 2);
+    base = (int64_t)(K * (v[0] - 1) + 1) + (int64_t)N1 * (K * (v[1] - 1) + 1);
+    if (DIM == 3) base += (int64_t)N1 * N1 * (K * (v[2] - 1) + 1);
+    if (threadIdx.x < P) {
+      s_base[pn] = active ? base : -1;
+      s_colour[pn] = J.colour < 0 ? (v[0] & 1) | ((v[1] & 1) << 1) | (DIM == 3 ? (v[2] & 1) << 2 : 0) : 0;
+      s_max[pn] = 0;
+    }
+  }
+  const T* rp = J.r + base;
+  using L = Lines<DIM>;
+  using XT = std::conditional_t<D::F64, long long, uint16_t>;
+  using YT = std::conditional_t<D::F64, long long, float>;
+  XT* X = reinterpret_cast<XT*>(smraw);
+  YT* Y = reinterpret_cast<YT*>(smraw + D::YOFF);
+  T* Z = reinterpret_cast<T*>(smraw + D::ZOFF);
+  // padding rows of the operand: zero
+  if constexpr (S::PROWS != S::ROWS) {
+#pragma unroll
+    for (int s = 0; s < S::NS; ++s) {
+      constexpr int PARTS = D::F64 ? 1 : D::SL;
+      const int z0 = S::prow(s) + S::size(s), nz = S::prow(s) + 16 * S::tiles(s) - z0;
+      if (nz > 0)
+        for (int i = threadIdx.x; i < PARTS * nz * P; i += 32 * NW) {
+          const int pt = i / (nz > 0 ? nz * P : 1), w = i - pt * nz * P;
+          X[(pt * S::PROWS + z0 + w / P) * D::XP + w % P] = 0;
+        }
+    }
+  }
+  int e = 0;         // FP64: biased exponent bound of the patch's values
+  bool bad = false;  // FP64: an infinity or NaN among them
+  bool tiny = false;
+  const int* classexp = reinterpret_cast<const int*>(J.table + D::FRAGS) + S::ROWS;
+  if constexpr (D::F64) {
+    __syncthreads();  // s_max
+    double* R = reinterpret_cast<double*>(Y);
+    unsigned mx = 0;
+    for (int l = item0; l < S::NODES / S::M; l += STEP) {
+      const double* q = rp + N1 * (DIM == 3 ? l % S::M + N1 * (l / S::M) : l);
+      double v[S::M];
+#pragma unroll
+      for (int i = 0; i < S::M; ++i) v[i] = active ? q[i] : 0.0;
+#pragma unroll
+      for (int i = 0; i < S::M; ++i) {
+        R[(l * S::M + i) * P + pn] = v[i];
+        mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu);
+      }
+    }
+#pragma unroll
+    for (int o = P; o < 32; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane < P) atomicMax(&s_max[pn], mx);
+    __syncthreads();
+    mx = s_max[pn];
+    bad = mx >= 0x7FF00000u || J.cmul == 0 || classexp[0] == kNoExp;
+    // the bound leaves 0.8% to the top digit's range; subnormal patches are
+    // scaled by 2^100 and bounded by the high word's leading bit
+    tiny = mx < 0x00100000u;
+    e = tiny ? 113 - __clz((int)mx) : (int)((mx + 0x4000u) >> 20);
+  }
+  // even / odd combinations, stored as operands
+  for (int l = item0; l < L::N; l += STEP) {
+    const L ln(l);
+    if constexpr (D::F64) {
+      const double* R = reinterpret_cast<const double*>(Y);
+      long long v[L::IMAGES][S::M];
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b) {
+        const double* q = R + ln.node(b, S::M) * P + pn;
+#pragma unroll
+        for (int i = 0; i < S::M; ++i)
+          v[b][i] = ln.has(b) || !S::SPLIT ? fixed_of(tiny ? q[i * P] * 0x1p100 : q[i * P], e) : 0;
+      }
+      reflect<DIM>(v);
+      const int sh0 = (S::SPLIT ? DIM + 3 : 3) - ln.centres();  // to 55 bits and sign: 2^(d-c) images were summed
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b)
+        if (ln.has(b) || !S::SPLIT)
+          for_coefs<DIM>(b, [&](int i, int s, int ox) {
+            const int sh = S::SPLIT && i == K - 1 ? sh0 - 1 : sh0;
+            X[(S::prow(s) + ox + ln.coef(s)) * D::XP + pn] = (v[b][i] + (1ll << (sh - 1))) >> sh;
+          });
+    } else {
+      float v[L::IMAGES][S::M];
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b) {
+        const float* q = rp + ln.node(b, N1);
+        const bool in = active && (ln.has(b) || !S::SPLIT);
+#pragma unroll
+        for (int i = 0; i < S::M; ++i) v[b][i] = in ? q[i] : 0.f;
+      }
+      reflect<DIM>(v);
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b)
+        if (ln.has(b) || !S::SPLIT)
+          for_coefs<DIM>(b, [&](int i, int s, int ox) {
+            XT* x = X + (S::prow(s) + ox + ln.coef(s)) * D::XP + pn;
+            const uint32_t b1 = __float_as_uint(v[b][i]);
+            const float f2 = v[b][i] - __uint_as_float(b1 & 0xFFFF0000u);
+            const uint32_t b2 = __float_as_uint(f2);
+            const float f3 = f2 - __uint_as_float(b2 & 0xFFFF0000u);
+            x[0] = (uint16_t)(b1 >> 16);
+            x[S::PROWS * D::XP] = (uint16_t)(b2 >> 16);
+            x[2 * S::PROWS * D::XP] = (uint16_t)(__float_as_uint(f3) >> 16);
+          });
+    }
+  }
+  __syncthreads();
+  if constexpr (D::F64) {
+    for (int u = warp; u < D::UNITS; u += NW) dense_mma<DIM>(c_units.u[u], J.table, X, Y, lane);
+  } else {
+    float y[D::UPW][D::NT][4];
+#pragma unroll
+    for (int i = 0; i < D::UPW; ++i)
+      if (warp + i * NW < D::UNITS) dense_mma<DIM>(c_units.u[warp + i * NW], J.table, X, y[i], lane);
+    __syncthreads();  // the results take the operands' place
+#pragma unroll
+    for (int i = 0; i < D::UPW; ++i)
+      if (warp + i * NW < D::UNITS) {
+        const DenseUnit& u = c_units.u[warp + i * NW];
+#pragma unroll
+        for (int t = 0; t < D::NT; ++t)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int rr = (lane >> 2) + 8 * h;
+            if (rr < u.valid)
+              *reinterpret_cast<float2*>(Y + (u.row + rr) * D::YP + 8 * t + 2 * (lane & 3)) =
+                  make_float2(y[i][t][2 * h], y[i][t][2 * h + 1]);
+          }
+      }
+  }
+  __syncthreads();
+  // back to the nodes
+  for (int l = item0; l < L::N; l += STEP) {
+    const L ln(l);
+    YT v[L::IMAGES][S::M];
+#pragma unroll
+    for (int b = 0; b < L::IMAGES; ++b) {
+      const bool in = ln.has(b) || !S::SPLIT;
+      for_coefs<DIM>(b, [&](int i, int s, int ox) {
+        v[b][i] = in ? Y[(S::row(s) + ox + ln.coef(s)) * D::YP + pn] : YT(0);
+      });
+    }
+    reflect<DIM>(v);
+#pragma unroll
+    for (int b = 0; b < L::IMAGES; ++b)
+      if (ln.has(b) || !S::SPLIT) {
+        T* z = Z + pn * D::ZP + ln.node(b, S::M);
+        const int ve = J.vexp + e - (tiny ? 100 : 0), nc = ln.centres();
+        const int ve0 = D::F64 ? ve - __ldg(classexp + nc) : 0, ve1 = D::F64 ? ve - __ldg(classexp + nc + 1) : 0;
+#pragma unroll
+        for (int i = 0; i < S::M; ++i) {
+          if constexpr (D::F64)
+            z[i] = bad ? __longlong_as_double(0x7FF8000000000000ll) : double_of(v[b][i], J.cmul, S::SPLIT && i == K - 1 ? ve1 : ve0);
+          else
+            z[i] = J.c * v[b][i];
+        }
+      }
+  }
+  __syncthreads();
+  // a warp writes a patch; each lane keeps the offsets of its nodes
+  constexpr int NO = (S::NODES + 31) / 32;
+  int off[NO];
+#pragma unroll
+  for (int j = 0; j < NO; ++j) {
+    const int i = lane + 32 * j, r = i / S::M;
+    off[j] = i - r * S::M + N1 * (DIM == 3 ? r % S::M + N1 * (r / S::M) : r);
+  }
+  const int64_t N = (int64_t)N1 * N1 * (DIM == 3 ? N1 : 1);
+  for (int gp = warp; gp < P; gp += NW) {
+    if (s_base[gp] < 0) break;  // past the last patch
+    T* o = J.dst + s_colour[gp] * N + s_base[gp];
+    const T* z = Z + gp * D::ZP + lane;
+    if (J.colour < 0) {
+#pragma unroll
+      for (int j = 0; j < NO; ++j)
+        if (lane + 32 * j < S::NODES) o[off[j]] = z[32 * j];
+    } else {  // one patch of the colour per node
+#pragma unroll
+      for (int j = 0; j < NO; ++j)
+        if (lane + 32 * j < S::NODES) o[off[j]] += z[32 * j];
+    }
+  }
+}
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(32 * Dense<DIM, T>::NW, Dense<DIM, T>::MINB()) patch_dense_kernel(const __grid_constant__ DenseJob<T> J) {
+  dense_body<DIM, T>(J, blockIdx.x);
+}
+
+// Grouped launch: the batches of all jobs, job after job
+template <int DIM, typename T>
+__global__ void __launch_bounds__(32 * Dense<DIM, T>::NW, Dense<DIM, T>::MINB())
+    patch_dense_group_kernel(const __grid_constant__ GroupOf<DenseJob<T>> G) {
+  const int j = group_find(G, blockIdx.x);
+  dense_body<DIM, T>(G.job[j], blockIdx.x - (uint32_t)G.start[j]);
+}
+
+// K = 1: the patch is its vertex, the local solve one multiplication by
+// c = omega_AS / A_{j,1} (additive) or 1 / A_{j,1}.
+template <int DIM, typename T>
+__device__ __forceinline__ void point_body(const DenseJob<T>& J, uint32_t pid) {
+  const uint32_t r1 = J.d0.div(pid), r2 = J.d1.div(r1);
+  const int i[3] = {(int)(pid - r1 * J.d0.d), (int)(DIM == 3 ? r1 - r2 * J.d1.d : r1), (int)(DIM == 3 ? r2 : 0)};
+  int v[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) v[d] = J.colour < 0 ? i[d] + 1 : 2 * i[d] + (((J.colour >> d) & 1) ? 1 : 2);
+  const int64_t N1 = J.n + 1, node = v[0] + N1 * (v[1] + (DIM == 3 ? N1 * v[2] : 0));
+  const int64_t N = DIM == 3 ? N1 * N1 * N1 : N1 * N1;
+  const int pc = (v[0] & 1) | ((v[1] & 1) << 1) | (DIM == 3 ? (v[2] & 1) << 2 : 0);
+  if (J.colour < 0) J.dst[pc * N + node] = J.c * J.r[node];
+  else J.dst[node] += J.c * J.r[node];
+}
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(256) patch_point_kernel(const __grid_constant__ DenseJob<T> J) {
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t < J.npatch) point_body<DIM, T>(J, t);
+}
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(256) patch_point_group_kernel(const __grid_constant__ GroupOf<DenseJob<T>> G) {
+  const int j = group_find(G, blockIdx.x);
+  const uint32_t t = (uint32_t)(blockIdx.x - G.start[j]) * 256u + threadIdx.x;
+  if (t < G.job[j].npatch) point_body<DIM, T>(G.job[j], t);
+}
+
+// ---------------------------------------------------------------- the matrix
+// Columns of B at unit scale (the FP64 part serves both precisions): the local
+// solver applied to the unit vectors of the orbits' first nodes, one node per
+// patch of the block; out[column][node].  A further local cycle (Algorithm 2,
+// N_iter > 1) continues from out.  For FP64 products V = dd: the matrix is
+// rounded once, where the local solver in plain FP64 would leave 2-5 times
+// the error of a solve in the products (K = 3: 1.1e-15 against 3.3e-16).
+template <int DIM, typename V>
+__global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__ out, int np, bool first,
+                                                            const double* __restrict__ dinv, PatchParams<double> H) {
+  using S = Sectors<DIM>;
+  using PS = PatchShape<DIM>;
+  constexpr int SZT = PS::SZT, RT = PS::off_r(PS::L - 1), DT = PS::off_d(PS::L - 1);
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int c0 = blockIdx.x * np, nc = min(np, S::ORBITS - c0);
+  const PBlock<V, 0> pb{reinterpret_cast<V*>(smraw), PS::ELEMS, nc};
+  PatchParams<V> P;
+  P.scale = H.scale;
+  P.omega_as = H.omega_as;
+  for (int i = 0; i < 4; ++i) P.omega[i] = H.omega[i];
+  P.inv_a0 = H.inv_a0;
+  P.inv_scale = H.inv_scale;
+  P.half = H.half;
+  P.colour = H.colour;
+  const CartGeo<DIM, V> geo{dinv, P.scale, P.inv_scale, P.inv_a0};
+  pfor<SZT>(pb, [&](int g, int i) {
+    pb.at(g)[RT + i] = V(i == Orbit<DIM>(c0 + g).node(0) ? 1.0 : 0.0);
+    if (!first) pb.at(g)[DT + i] = V(out[(int64_t)(c0 + g) * SZT + i]);
+  });
+  __syncthreads();
+  if constexpr (PS::L > 1) {
+    if (!first) geo.template resid<PS::L - 1>(pb, DT, RT, RT);  // r = e_j - A x
+  }
+  pvcycle<DIM, PS::L - 1>(pb, geo, P);
+  pfor<SZT>(pb, [&](int g, int i) {
+    double& o = out[(int64_t)(c0 + g) * SZT + i];
+    const V d = pb.at(g)[DT + i];
+    o = first ? value_of(d) : value_of(V(o) + d);
+  });
+}
+
+// Sector matrices from the columns, one warp per row: the entry for
+// coefficient j is the signed sum of column j over the mirror images of the
+// row's node, over 2^d -- the operand of an orbit with c central coordinates,
+// which has only 2^(d-c) images, counts 2^c times.  rowexp: the largest exponent x
+// with entry 2^x below 0.98 2^55 (7 signed digits reach 127/128 of 2^55) and
+// the row's sum of magnitudes times 2^x below 2^57 (results and their even /
+// odd sums stay within 64 bits).  The sectors' results for one orbit are
+// summed, so they need a common exponent: minexp, the least one of the rows
+// of a class -- the nodes with the same number of central coordinates, whose
+// coefficients have the same size (kNoExp if an entry is not finite).
+template <int DIM>
+__global__ void __launch_bounds__(128) patch_entries_kernel(const double* __restrict__ columns,
+                                                            double* __restrict__ entries, int* __restrict__ rowexp,
+                                                            int* __restrict__ minexp) {
+  using S = Sectors<DIM>;
+  const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= S::ROWS) return;
+  int s = 0;
+  while (s + 1 < S::NS && row >= S::row(s + 1)) ++s;
+  const int m = row - S::row(s), sz = S::size(s), e0 = S::ext(s, 0), e1 = S::ext(s, 1);
+  auto orbit_of = [&](int k) { return k % e0 + S::E * ((k / e0) % e1 + S::E * (k / (e0 * e1))); };
+  const Orbit<DIM> om(orbit_of(m));
+  double* out = entries + S::entry(s) + (int64_t)m * sz;
+  double top = 0.0, sum = 0.0;
+  for (int k = lane; k < sz; k += 32) {
+    const Orbit<DIM> oj(orbit_of(k));
+    const double* col = columns + (int64_t)orbit_of(k) * S::NODES;
+    double a = 0.0;
+#pragma unroll
+    for (int b = 0; b < S::IMAGES; ++b) {
+      if (S::IMAGES > 1 && !oj.has(b)) continue;
+      const double v = col[om.node(b)];
+      a += (__popc(s & b) & 1) ? -v : v;
+    }
+    a /= S::IMAGES;
+    out[k] = a;
+    top = fmax(top, fabs(a));
+    sum += fabs(a);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  }
+  if (lane) return;
+  int te = 0, se = 0;
+  if (frexp(top, &te) > 0.98) ++te;
+  frexp(sum, &se);
+  const int x = sum == 0.0 ? 1000 : min(55 - te, 57 - se);
+  rowexp[row] = x;
+  atomicMin(minexp + om.centres(), x);
+  if (!isfinite(sum)) atomicMin(minexp, kNoExp);
+}
+
+// Fragments of the first operand of mma.m16n8k16, per 16 x 16 tile and part:
+// lane l holds rows l / 4 and l / 4 + 8, columns 2 (l % 4) and + 8.  FP64:
+// 8-bit signed digits of entry 2^(the row's exponent, at most 15 above its
+// class's); FP32: three BF16 parts, rounded.
+template <int DIM, typename T>
+__global__ void patch_table_kernel(const double* __restrict__ entries, const int* __restrict__ rowexp,
+                                   const int* __restrict__ minexp, uint32_t* __restrict__ table) {
+  using S = Sectors<DIM>;
+  constexpr int SL = Dense<DIM, T>::SL;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)S::TILES * 32 * 4) return;
+  const int reg = (int)(t & 3), lane = (int)(t >> 2) & 31, tile = (int)(t >> 7);
+  int s = 0;
+  while (s + 1 < S::NS && tile >= S::tile(s + 1)) ++s;
+  const int nt = S::tiles(s), sz = S::size(s), mt = (tile - S::tile(s)) / nt, kt = (tile - S::tile(s)) % nt;
+  const int m = 16 * mt + (lane >> 2) + 8 * (reg & 1), k0 = 16 * kt + 2 * (lane & 3) + 8 * (reg >> 1);
+  int re = 0;
+  if (sizeof(T) == 8 && m < sz) {
+    const int e0 = S::ext(s, 0), e1 = S::ext(s, 1);
+    const Orbit<DIM> om(m % e0 + S::E * ((m / e0) % e1 + S::E * (m / (e0 * e1))));
+    const int exp = minexp[om.centres()];
+    re = min(rowexp[S::row(s) + m], exp + 15);
+    int* tail = reinterpret_cast<int*>(table + (int64_t)Dense<DIM, T>::FRAGS * 4);
+    if (kt == 0 && (lane & 3) == 0 && reg < 2) tail[S::row(s) + m] = re - exp;
+    if (tile == 0 && lane == 0 && reg == 0)
+      for (int i = 0; i < 4; ++i) tail[S::ROWS + i] = minexp[i];
+  }
+  uint32_t part[SL] = {};
+  for (int h = 0; h < 2; ++h) {
+    const int k = k0 + h;
+    const double a = m < sz && k < sz ? entries[S::entry(s) + (int64_t)m * sz + k] : 0.0;
+    if constexpr (sizeof(T) == 8) {
+      const long long v = __double2ll_rn(scalbn(a, re)) + 0x0080808080808080ll;
+      for (int i = 0; i < SL; ++i) {
+        const int digit = (int)((v >> (8 * (SL - 1 - i))) & 0xFF) - 128;
+        part[i] |= (uint32_t)__half_as_ushort(__int2half_rn(digit)) << (16 * h);
+      }
+    } else {
+      const int e0 = S::ext(s, 0), e1 = S::ext(s, 1), kk = k < sz ? k : 0;
+      const Orbit<DIM> oj(kk % e0 + S::E * ((kk / e0) % e1 + S::E * (kk / (e0 * e1))));
+      double rest = a * (1 << oj.centres());  // FP32 operands are plain sums over the images
+      for (int i = 0; i < SL; ++i) {
+        const __nv_bfloat16 p = __double2bfloat16(rest);
+        rest -= (double)__bfloat162float(p);
+        part[i] |= (uint32_t)__bfloat16_as_ushort(p) << (16 * h);
+      }
+    }
+  }
+  for (int i = 0; i < SL; ++i) table[(((int64_t)tile * SL + i) * 32 + lane) * 4 + reg] = part[i];
+}
+
+}  // namespace PMG_KNS
+}  // namespace pmg

@@ -94,8 +94,7 @@ extern "C" int pmg_apply_cartesian_noalloc(int dim, int n_cells, int degree, con
       s.ready = true;
     }
     if (!s.coef[degree][dim - 2]) {
-      std::vector<double> coef(pmg::kMaxCoef, 0.0);
-      pmg::host::fill_coefficients(degree, coef.data());
+      const std::vector<double>& coef = pmg::host::coefficients(degree);
       e = kt->prepare();
       if (e == cudaSuccess) e = kt->upload(coef.data());
       if (e != cudaSuccess) return fail(PMG_ERR_CUDA, std::string("coefficient upload: ") + cudaGetErrorString(e));

@@ -217,6 +217,13 @@ int make_plan(const pmg_config* cfg, Plan& P) {
   // operator results (FP64 for the CG)
   const int nf = cfg->n_cells;
   P.pbuf = bump(cur, (int64_t)(1 << P.dim) * ipow64((int64_t)P.K * nf + 1, P.dim) * P.mg_es);
+  if (!P.deformed) {
+    const int64_t tb = kernel_table(P.K, P.dim, cfg->mg_precision)->patch_table_bytes(P.dim, cfg->mg_precision);
+    if (tb > 0) {
+      P.table = bump(cur, tb);
+      P.tscratch = bump(cur, kernel_table(P.K, P.dim, PMG_FP64)->patch_scratch_bytes(P.dim));
+    }
+  }
   if (cfg->geometry == PMG_GEOM_DISTORTED) P.verts = bump(cur, ipow64(nf + 1, P.dim) * P.dim * 8);
   if (P.deformed) P.cellbuf = bump(cur, ipow64(nf, P.dim) * ipow64(P.K + 1, P.dim) * 8);
   P.total = cur;
@@ -240,6 +247,7 @@ PatchParamsHost patch_params(const pmg_ctx* c, int level) {
   P.inv_a0 = c->lv[level].inv_a0;
   P.half = c->cfg.local_half;
   P.colour = -1;
+  P.table = c->table;
   return P;
 }
 }  // namespace pmg
@@ -673,7 +681,7 @@ int choose_patch_layout(pmg_ctx* c) {
   if (try_il) c->il_threads = 256;  // rule for meshes too small to time
   LevelData& F = c->lv[c->L - 1];
   const int64_t patches = ipow64(std::max(F.n - 1, 0), c->dim);
-  if (c->K == 1 || patches < 4096) return PMG_OK;
+  if (c->K == 1 || c->table || patches < 4096) return PMG_OK;
   const bool mult = cf.smoother == PMG_SMOOTHER_MULTIPLICATIVE;
   const TuneKey key{c->dim, c->K, c->mgprec, c->deformed ? 1 : 0, cf.local_cycles, mult ? 1 : 0, F.n};
   auto valid = [&](const TuneVal& v) {
@@ -887,6 +895,25 @@ void pinned_scalars_put(double* p) {
   g_pin_free.push_back(p);
 }
 
+// Sector matrices of the Cartesian local solver (kernels_patch.cuh): entries
+// from the FP64 part at unit scale, then the table of the MG precision.
+int setup_patch_table(pmg_ctx* c) {
+  if (c->plan.table < 0) return PMG_OK;
+  c->table = at(c, c->plan.table);
+  double* scratch = (double*)at(c, c->plan.tscratch);
+  PatchParamsHost P{};
+  P.scale = 1.0;
+  P.omega_as = 1.0;
+  for (int i = 0; i < 4; ++i) P.omega[i] = c->omega_j[i];
+  P.inv_a0 = 1.0 / (c->dim * 2.0 * std::pow(2.0 / 3.0, c->dim - 1));
+  P.half = c->cfg.local_half;
+  P.colour = -1;
+  PMG_CUDA(c->kt[PMG_FP64]->patch_entries(c->dim, P, c->cfg.local_cycles, c->mgprec, c->dtab64, scratch,
+                                            c->stream));
+  PMG_CUDA(c->km()->patch_table(c->dim, c->mgprec, scratch, c->table, c->stream));
+  return PMG_OK;
+}
+
 int setup_context(pmg_ctx* c) {
   const Plan& P = c->plan;
   c->lv.resize(c->L);
@@ -938,8 +965,7 @@ int setup_context(pmg_ctx* c) {
 
   // coefficients and kernel attributes: once per device and kernel part
   // (module state that every context of the part shares)
-  std::vector<double> coef(kMaxCoef, 0.0);
-  host::fill_coefficients(c->K, coef.data());
+  const std::vector<double>& coef = host::coefficients(c->K);
   {
     static std::mutex mu;
     static std::set<std::pair<int, const KernelTable*>> ready;
@@ -1033,6 +1059,8 @@ int setup_context(pmg_ctx* c) {
     PMG_CUDA(cudaStreamSynchronize(c->stream));
     if (bad) return fail(PMG_ERR_ARG, "inverted cell: det J <= 0 at a quadrature point of the mesh");
   }
+
+  if (int rc = setup_patch_table(c)) return rc;
 
   // patch-kernel layout and block shape: the autotuned choice (or the caller's)
   if (int rc = choose_patch_layout(c)) return rc;

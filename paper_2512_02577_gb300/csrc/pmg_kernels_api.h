@@ -24,6 +24,7 @@ struct PatchParamsHost {
   int colour;        // -1: every patch, additive output (omega_AS d_j per colour
                      // vector); c >= 0: only the patches of parity colour c,
                      // u += d_j added straight into dst (multiplicative sweep)
+  const void* table;  // Cartesian: the sector matrices of the local solver (patch_table)
 };
 
 // Deformed-geometry arrays of one mesh level (device pointers).
@@ -129,6 +130,16 @@ struct KernelTable {
                                     cudaStream_t s);
   cudaError_t (*h_prolong_add_group)(int dim, int prec, int count, const TransferSolveJob* jobs, cudaStream_t s);
   cudaError_t (*h_restrict_group)(int dim, int prec, int count, const TransferSolveJob* jobs, cudaStream_t s);
+  // Cartesian patches as products with the local solver's sector matrices:
+  // device bytes of the part's table (0: the part sum-factorises, or K = 1) and
+  // of the FP64 scratch of its set-up; the set-up on the degree's FP64 part
+  // (the local solver of n_iter cycles at unit scale, for products in precision
+  // prec), then the table on the part itself
+  int64_t (*patch_table_bytes)(int dim, int prec);
+  int64_t (*patch_scratch_bytes)(int dim);
+  cudaError_t (*patch_entries)(int dim, const PatchParamsHost& H, int n_iter, int prec, const double* dinv,
+                               double* scratch, cudaStream_t s);
+  cudaError_t (*patch_table)(int dim, int prec, const double* scratch, void* table, cudaStream_t s);
 };
 
 // nullptr when k, dim or prec is out of range

@@ -285,6 +285,14 @@ double default_omega_jacobi(int d, int p) {
   return c;
 }
 
+// The mean of an r x c table and its mirror image (both indices reversed):
+// the 1D matrices are centrosymmetric, their quadrature only up to rounding.
+// The sector matrices (kernels_patch.cuh) take one half for both, which would
+// double the effect of its rounding.
+static void make_centrosymmetric(double* a, int r, int c) {
+  for (int i = 0, j = r * c - 1; i < j; ++i, --j) a[i] = a[j] = 0.5 * (a[i] + a[j]);
+}
+
 void fill_coefficients(int K, double* out) {
   const CoefLayout L = coef_layout(K);
   std::memset(out, 0, sizeof(double) * L.total);
@@ -294,6 +302,8 @@ void fill_coefficients(int K, double* out) {
     out[L.Me + i] = M[i];
     out[L.Ke + i] = Kst[i];
   }
+  make_centrosymmetric(out + L.Me, K + 1, K + 1);
+  make_centrosymmetric(out + L.Ke, K + 1, K + 1);
   auto nd = gll_points(K);
   for (int ch = 0; ch < 2; ++ch)
     for (int i = 0; i <= K; ++i)
@@ -310,12 +320,15 @@ void fill_coefficients(int K, double* out) {
       out[L.MP[l] + i] = MP[i];
       out[L.KP[l] + i] = KP[i];
     }
+    make_centrosymmetric(out + L.MP[l], m, m);
+    make_centrosymmetric(out + L.KP[l], m, m);
     for (int i = 0; i < m; ++i) {
-      out[L.dM[l] + i] = MP[i * m + i];
-      out[L.dK[l] + i] = KP[i * m + i];
+      out[L.dM[l] + i] = out[L.MP[l] + i * m + i];
+      out[L.dK[l] + i] = out[L.KP[l] + i * m + i];
     }
     auto T = p_transfer(q, p);
     for (int i = 0; i < m * mc; ++i) out[L.Tr[l] + i] = T[i];
+    make_centrosymmetric(out + L.Tr[l], m, mc);
   }
   for (int l = 0; l < nlev(K); ++l) {
     const int p = plev(K, l);
@@ -329,6 +342,20 @@ void fill_coefficients(int K, double* out) {
   }
   out[L.dM0] = 2.0 / 3.0;
   out[L.dK0] = 2.0;
+}
+
+// One block per degree, formed once per process (the quadrature and Lagrange
+// tables cost 0.1-8 ms of host time at k = 2..7, most of a context's set-up).
+const std::vector<double>& coefficients(int K) {
+  static std::mutex mu;
+  static std::vector<double> block[9];
+  std::lock_guard<std::mutex> g(mu);
+  std::vector<double>& b = block[K];
+  if (b.empty()) {
+    b.resize(kMaxCoef, 0.0);
+    fill_coefficients(K, b.data());
+  }
+  return b;
 }
 
 // Global-fine-level variants of S / Dq / W for degree K (used by the cell

@@ -14,6 +14,7 @@ void patch_1d(int p, std::vector<double>& MP, std::vector<double>& KP);
 std::vector<double> p_transfer(int q, int p);
 double default_omega_jacobi(int d, int p);
 void fill_coefficients(int K, double* out);
+const std::vector<double>& coefficients(int K);  // the block of degree K, kept for the process
 void cell_tables(int p, std::vector<double>& S, std::vector<double>& Dq, std::vector<double>& W);
 
 }  // namespace host

@@ -1,0 +1,85 @@
+"""Cartesian patch smoother as products with the local solver's sector
+matrices: partial batches of patches, the smallest meshes, the fixed-point
+scaling of the FP64 products and values that are not finite.
+
+Tolerances as in test_gpu_parity (FP64 sweep 1e-11, FP32 2e-5).  Scaling the
+right-hand side by a power of two is exact in every step, so those results
+are compared bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2512_02577_gb300 as p
+from paper_2512_02577_gb300.inputs import random_vector
+from tests.parity import rel
+from tests.test_gpu_defaults_high_degree import _tol, ctx_default
+from tests.test_gpu_parity import full, oracle_level, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+# patches: 1, 8, 27 in 3D; 1, 16, 17^2 = 18 * 16 + 1 in 2D
+@pytest.mark.parametrize("d,n,k", [(3, 2, 1), (3, 2, 2), (3, 3, 3), (3, 2, 5), (3, 4, 5), (3, 2, 4), (2, 2, 8),
+                                   (2, 5, 8), (2, 18, 2), (2, 18, 3), (2, 5, 4), (2, 5, 7), (2, 3, 1)])
+@pytest.mark.parametrize("prec", [p.FP64, p.FP32])
+@pytest.mark.parametrize("smoother", [p.ADDITIVE, p.MULTIPLICATIVE])
+def test_sweep_matches_oracle(d, n, k, prec, smoother):
+    dt = torch.float64 if prec == p.FP64 else torch.float32
+    ctx = ctx_default(d, n, k, L=1, prec=prec, smoother=smoother)
+    fine = oracle_level(d, n, k, "cartesian")
+    b, u0 = random_vector(d, n, k, seed=501 + k), random_vector(d, n, k, seed=502 + k)
+    u = to_dev(u0, dt)
+    ctx.smooth(to_dev(b, dt), u)
+    sweep = fine.smooth if smoother == p.ADDITIVE else fine.mult_sweep
+    assert rel(u, full(fine, sweep(b[fine.I], u0[fine.I]))) < _tol(prec)
+
+
+@pytest.mark.parametrize("d,n,k,prec,power", [(3, 4, 4, p.FP64, 900), (3, 4, 4, p.FP64, -900), (2, 6, 2, p.FP64, 600),
+                                              (3, 3, 4, p.FP32, 60), (3, 3, 3, p.FP32, -60)])
+def test_scaling_by_a_power_of_two_is_exact(d, n, k, prec, power):
+    dt = torch.float64 if prec == p.FP64 else torch.float32
+    ctx = ctx_default(d, n, k, L=1, prec=prec)
+    b = to_dev(random_vector(d, n, k, seed=511), dt)
+    s = torch.tensor(2.0 ** power, dtype=dt, device=b.device)
+    u, us = torch.zeros_like(b), torch.zeros_like(b)
+    ctx.smooth(b, u)
+    ctx.smooth(b * s, us)
+    assert torch.equal(us, u * s) and float(u.abs().max()) > 0
+
+
+@pytest.mark.parametrize("prec", [p.FP64, p.FP32])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+def test_values_that_are_not_finite_stay_in_their_patches(prec, value):
+    # one bad entry strictly inside cell (0, 0, 0): only the patch of vertex (1, 1, 1) holds it
+    d, n, k = 3, 4, 3
+    dt = torch.float64 if prec == p.FP64 else torch.float32
+    ctx = ctx_default(d, n, k, L=1, prec=prec)
+    N1 = k * n + 1
+    b = to_dev(random_vector(d, n, k, seed=521), dt).reshape(N1, N1, N1)
+    clean = torch.zeros_like(b)
+    ctx.smooth(b.reshape(-1), clean.reshape(-1))
+    b[1, 1, 1] = value
+    u = torch.zeros_like(b)
+    ctx.smooth(b.reshape(-1), u.reshape(-1))
+    inside = torch.zeros_like(b, dtype=torch.bool)
+    inside[1:2 * k, 1:2 * k, 1:2 * k] = True
+    assert not torch.isfinite(u[inside]).any()
+    assert torch.equal(u[~inside], clean[~inside])
+
+
+def test_zero_right_hand_side_and_extreme_range():
+    d, n, k = 3, 3, 4
+    ctx = ctx_default(d, n, k, L=1)
+    b = torch.zeros((k * n + 1) ** d, dtype=torch.float64, device="cuda:0")
+    u = torch.zeros_like(b)
+    ctx.smooth(b, u)
+    assert not u.any()
+    # subnormal residuals: results no further off than the subnormal spacing allows
+    r = random_vector(d, n, k, seed=531)
+    ctx.smooth(to_dev(r * 2.0 ** -1060), u)
+    ref = torch.zeros_like(b)
+    ctx.smooth(to_dev(r * 2.0 ** -1060 * 2.0 ** 900), ref)
+    assert np.abs(u.cpu().numpy() * 2.0 ** 900 - ref.cpu().numpy()).max() <= 8 * 2.0 ** (-1074 + 900)
