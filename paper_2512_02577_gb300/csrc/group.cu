@@ -87,9 +87,12 @@ int g_apply(const std::vector<GSel>& S, int prec, void* const* x, void* const* y
     for (int t = 0; t < 4; ++t) J[i].t[t] = (ff || prec == PMG_FP64) ? (void*)c->t64[t] : c->t_mg[t];
     J[i].n = L.n;
     J[i].scale = L.scale;
+    J[i].table = c->ctable;
   }
   const int cnt = (int)S.size();
   if (ff) return gcheck(c0->kt[PMG_FP64]->cart_apply_ff_group(c0->dim, cnt, J, st), "grouped apply");
+  if (prec == PMG_FP64 && c0->ctable)
+    return gcheck(c0->kt[PMG_FP64]->cell_apply_group(c0->dim, cnt, J, st), "grouped apply");
   return gcheck(c0->kt[prec]->cart_apply_group(c0->dim, prec, cnt, J, st), "grouped apply");
 }
 

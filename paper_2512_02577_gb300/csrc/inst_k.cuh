@@ -17,7 +17,13 @@ namespace PMG_KNS {
 constexpr int DP = PMG_DIM;
 // the Cartesian patches of this part are solved by the dense sector products
 // (K = 1: pointwise) instead of sum factorisation
-constexpr bool kDense = K == 1 || Dense<DP, TP>::ok();
+constexpr bool kDense = K == 1 || PatchDense<DP, TP>::ok();
+// FP64 operator applies by cells; line passes where they are as fast (2D K = 2:
+// 9 of a tile's 16 rows used, 0.218 against 0.195 ms at 1024^2 cells) and for
+// K = 1 (the 2^d results per cell need more scratch than the passes)
+constexpr bool kCellDense = PMG_PREC == 0 && CellDense<DP>::ok() && !(DP == 2 && K == 2);
+
+static int64_t ipow64(int64_t b, int e) { return e == 0 ? 1 : b * ipow64(b, e - 1); }
 
 static bool mine(int dim, int prec) { return dim == DP && prec == PMG_PREC; }
 
@@ -161,7 +167,7 @@ static DenseJob<T> dense_job(const T* r, T* dst, int n, const PatchParamsHost& H
   const bool finite = std::isfinite(c);
   J.cmul = finite ? (unsigned long long)std::ldexp(std::frexp(c, &e), 64) : 0;
   // the operands are scaled by 2^(1080 - SH - e_patch), the products by 2^-52 (dense_body)
-  constexpr int SH = Sectors<DIM>::SPLIT ? DIM + 3 : 3;
+  constexpr int SH = Sectors<DIM, kPatchM>::SPLIT ? DIM + 3 : 3;
   J.vexp = finite ? e - 64 + 52 - (1080 - SH) : 0;
   J.npatch = (uint32_t)patch_count(DIM, n, H.colour);
   J.d0 = FastDiv(std::max(1, patch_count_1d(n, H.colour, 0)));
@@ -171,7 +177,7 @@ static DenseJob<T> dense_job(const T* r, T* dst, int n, const PatchParamsHost& H
 
 // patches per block of the dense kernels
 template <int DIM, typename T>
-constexpr uint32_t dense_batch() { return K == 1 ? 256 : Dense<DIM, T>::P; }
+constexpr uint32_t dense_batch() { return K == 1 ? 256 : PatchDense<DIM, T>::P; }
 
 template <int DIM, typename T>
 static cudaError_t patch_dense_t(const T* r, T* dst, int n, const PatchParamsHost& H, cudaStream_t st) {
@@ -179,7 +185,7 @@ static cudaError_t patch_dense_t(const T* r, T* dst, int n, const PatchParamsHos
   const DenseJob<T> J = dense_job<DIM, T>(r, dst, n, H);
   const unsigned grid = (J.npatch + dense_batch<DIM, T>() - 1) / dense_batch<DIM, T>();
   if constexpr (K == 1) patch_point_kernel<DIM, T><<<grid, 256, 0, st>>>(J);
-  else patch_dense_kernel<DIM, T><<<grid, 32 * Dense<DIM, T>::NW, Dense<DIM, T>::SMEM, st>>>(J);
+  else patch_dense_kernel<DIM, T><<<grid, 32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::SMEM, st>>>(J);
   g_launches += 1;
   return cudaGetLastError();
 }
@@ -453,7 +459,7 @@ static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int 
     if (G.count == 0) return cudaSuccess;
     if (grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
     if constexpr (K == 1) patch_point_group_kernel<DIM, T><<<(unsigned)grid, 256, 0, st>>>(G);
-    else patch_dense_group_kernel<DIM, T><<<(unsigned)grid, 32 * Dense<DIM, T>::NW, Dense<DIM, T>::SMEM, st>>>(G);
+    else patch_dense_group_kernel<DIM, T><<<(unsigned)grid, 32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::SMEM, st>>>(G);
     g_launches += 1;
     return cudaGetLastError();
   } else {
@@ -501,11 +507,11 @@ static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int 
 // and of the FP64 scratch its set-up needs: columns, entries, statistics.
 static int64_t patch_table_bytes(int dim, int prec) {
   if (!mine(dim, prec) || !kDense || K == 1) return 0;
-  return Dense<DP, TP>::TABLE_BYTES;
+  return PatchDense<DP, TP>::TABLE_BYTES;
 }
 
 static int64_t patch_scratch_bytes(int dim) {
-  using S = Sectors<DP>;
+  using S = Sectors<DP, kPatchM>;  // the cell's matrices need less
   return dim == DP ? 8 * ((int64_t)S::ORBITS * S::NODES + S::ENTRIES) + 4 * (S::ROWS + 4) : 0;
 }
 
@@ -513,7 +519,10 @@ static int64_t patch_scratch_bytes(int dim) {
 // inverse diagonals) into the scratch: entries, columns, the classes' least
 // row exponents (4) and the row exponents
 template <int DIM>
-static int64_t scratch_ints() { return (int64_t)Sectors<DIM>::ORBITS * Sectors<DIM>::NODES + Sectors<DIM>::ENTRIES; }
+static int64_t scratch_ints() {
+  using S = Sectors<DIM, kPatchM>;
+  return (int64_t)S::ORBITS * S::NODES + S::ENTRIES;
+}
 
 template <int DIM, typename V>
 static cudaError_t patch_columns(const PatchParamsHost& H, int n_iter, const double* dinv, double* columns,
@@ -523,7 +532,7 @@ static cudaError_t patch_columns(const PatchParamsHost& H, int n_iter, const dou
   const int smem = np * PatchShape<DIM>::ELEMS * (int)sizeof(V);
   if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
   for (int it = 0; it < n_iter; ++it)
-    patch_columns_kernel<DIM, V><<<(Sectors<DIM>::ORBITS + np - 1) / np, threads, smem, st>>>(
+    patch_columns_kernel<DIM, V><<<(Sectors<DIM, kPatchM>::ORBITS + np - 1) / np, threads, smem, st>>>(
         columns, np, it == 0, dinv, to_params<double>(H));
   g_launches += n_iter;
   return cudaGetLastError();
@@ -537,7 +546,7 @@ template <int DIM, typename T>
 static cudaError_t patch_entries_t(const PatchParamsHost& H, int n_iter, bool fp64, const double* dinv,
                                    double* scratch, cudaStream_t st) {
   if constexpr (sizeof(T) == 8 && K > 1) {
-    using S = Sectors<DIM>;
+    using S = Sectors<DIM, kPatchM>;
     double* columns = scratch + S::ENTRIES;
     int* minexp = (int*)(scratch + scratch_ints<DIM>());
     cudaError_t e = cudaMemsetAsync(minexp, 0x7F, 16, st);
@@ -547,7 +556,7 @@ static cudaError_t patch_entries_t(const PatchParamsHost& H, int n_iter, bool fp
                : patch_columns<DIM, double>(H, n_iter, dinv, columns, st);
     else e = patch_columns<DIM, double>(H, n_iter, dinv, columns, st);
     if (e != cudaSuccess) return e;
-    patch_entries_kernel<DIM><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, scratch, minexp + 4, minexp);
+    sector_entries_kernel<DIM, false><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, scratch, minexp + 4, minexp);
     g_launches += 1;
     return cudaGetLastError();
   }
@@ -565,12 +574,105 @@ template <int DIM, typename T>
 static cudaError_t patch_table_t(const double* scratch, void* table, cudaStream_t st) {
   if constexpr (kDense && K > 1) {
     const int* minexp = (const int*)(scratch + scratch_ints<DIM>());
-    const int64_t work = (int64_t)Sectors<DIM>::TILES * 128;
-    patch_table_kernel<DIM, T><<<(unsigned)((work + 255) / 256), 256, 0, st>>>(scratch, minexp + 4, minexp, (uint32_t*)table);
+    const int64_t work = (int64_t)Sectors<DIM, kPatchM>::TILES * 128;
+    sector_table_kernel<DIM, T, false><<<(unsigned)((work + 255) / 256), 256, 0, st>>>(scratch, minexp + 4, minexp, (uint32_t*)table);
     g_launches += 1;
     return cudaGetLastError();
   }
   return cudaErrorInvalidValue;
+}
+
+// ---------------------------------------------------------------- FP64 apply by cells
+static int64_t cell_table_bytes(int dim) { return dim == DP && kCellDense ? CellDense<DP>::TABLE_BYTES : 0; }
+
+// the cell's table, by way of the scratch (used on the stream, free again afterwards)
+template <int DIM, typename T>
+static cudaError_t cell_table_t(double* scratch, void* table, cudaStream_t st) {
+  if constexpr (kCellDense) {
+    using S = Sectors<DIM, kCellM>;
+    int* minexp = (int*)(scratch + S::ENTRIES);
+    cudaError_t e = cudaMemsetAsync(minexp, 0x7F, 16, st);
+    if (e != cudaSuccess) return e;
+    sector_entries_kernel<DIM, true><<<(S::ROWS + 3) / 4, 128, 0, st>>>(nullptr, scratch, minexp + 4, minexp);
+    sector_table_kernel<DIM, double, true><<<(S::TILES * 128 + 255) / 256, 256, 0, st>>>(scratch, minexp + 4, minexp,
+                                                                                        (uint32_t*)table);
+    g_launches += 2;
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
+static cudaError_t cell_table(int dim, double* scratch, void* table, cudaStream_t st) {
+  if (dim != DP) return cudaErrorInvalidValue;
+  return cell_table_t<DP, TP>(scratch, table, st);
+}
+
+// the cells of a level; cells: n^d (K+1)^d doubles of scratch
+template <int DIM>
+static DenseJob<double> cell_job(const double* x, double* cells, const void* table, int n, double scale) {
+  DenseJob<double> J{};
+  J.r = x;
+  J.dst = cells;
+  J.table = (const uint4*)table;
+  J.n = n;
+  J.colour = -1;
+  int e = 0;
+  J.cmul = (unsigned long long)std::ldexp(std::frexp(scale, &e), 64);
+  constexpr int SH = Sectors<DIM, kCellM>::SPLIT ? DIM + 3 : 3;
+  J.vexp = e - 64 + 52 - (1080 - SH);  // as dense_job
+  J.npatch = (uint32_t)ipow64(n, DIM);
+  J.d0 = FastDiv(n);
+  J.d1 = FastDiv(DIM == 3 ? n : 1);
+  return J;
+}
+
+template <int DIM, typename T>
+static cudaError_t cell_apply_t(const double* x, double* y, const double* b, double* cells, const void* table, int n,
+                                double scale, cudaStream_t st) {
+  if constexpr (kCellDense) {
+    using D = CellDense<DIM>;
+    const DenseJob<double> J = cell_job<DIM>(x, cells, table, n, scale);
+    cell_dense_kernel<DIM><<<(J.npatch + D::P - 1) / D::P, 32 * D::NW, D::SMEM, st>>>(J);
+    const int64_t N = ipow64(K * n + 1, DIM);
+    cell_sum_kernel<DIM><<<(unsigned)((N + 255) / 256), 256, 0, st>>>(CellSumJob<DIM>{cells, b, y, n, FastDiv(K * n + 1)}, N);
+    g_launches += 2;
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
+static cudaError_t cell_apply(int dim, const double* x, double* y, const double* b, double* cells, const void* table,
+                              int n, double scale, cudaStream_t st) {
+  if (dim != DP) return cudaErrorInvalidValue;
+  return cell_apply_t<DP, TP>(x, y, b, cells, table, n, scale, st);
+}
+
+template <int DIM, typename T>
+static cudaError_t cell_apply_group_t(int count, const ApplyJob* jobs, cudaStream_t st) {
+  if constexpr (kCellDense) {
+    using D = CellDense<DIM>;
+    GroupOf<DenseJob<double>> G;
+    GroupOf<CellSumJob<DIM>> H;
+    G.count = H.count = count;
+    G.start[0] = H.start[0] = 0;
+    for (int j = 0; j < count; ++j) {
+      const ApplyJob& a = jobs[j];
+      G.job[j] = cell_job<DIM>((const double*)a.x, (double*)a.t[0], a.table, a.n, a.scale);
+      G.start[j + 1] = G.start[j] + (G.job[j].npatch + D::P - 1) / D::P;
+      H.job[j] = CellSumJob<DIM>{(const double*)a.t[0], (const double*)a.b, (double*)a.y, a.n, FastDiv(K * a.n + 1)};
+      H.start[j + 1] = H.start[j] + ipow64(K * a.n + 1, DIM);
+    }
+    cell_dense_group_kernel<DIM><<<(unsigned)G.start[count], 32 * D::NW, D::SMEM, st>>>(G);
+    cell_sum_group_kernel<DIM><<<(unsigned)((H.start[count] + 255) / 256), 256, 0, st>>>(H);
+    g_launches += 2;
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
+static cudaError_t cell_apply_group(int dim, int count, const ApplyJob* jobs, cudaStream_t st) {
+  if (dim != DP || !group_ok(count)) return cudaErrorInvalidValue;
+  return cell_apply_group_t<DP, TP>(count, jobs, st);
 }
 
 static cudaError_t patch_table(int dim, int prec, const double* scratch, void* table, cudaStream_t st) {
@@ -755,6 +857,10 @@ static void prepare_cart(int optin, const Acc& acc) {
     acc(allow_smem(patch_dense_kernel<DIM, T>, optin));
     acc(allow_smem(patch_dense_group_kernel<DIM, T>, optin));
   }
+  if constexpr (kCellDense) {
+    acc(allow_smem(cell_dense_kernel<DIM>, optin));
+    acc(allow_smem(cell_dense_group_kernel<DIM>, optin));
+  }
   if constexpr (sizeof(T) == 8 && K > 1) {
     acc(allow_smem(patch_columns_kernel<DIM, double>, optin));
     if constexpr (columns_dd<DIM>()) acc(allow_smem(patch_columns_kernel<DIM, dd>, optin));
@@ -814,6 +920,10 @@ const KernelTable* PMG_TABLE_FN() {
       PMG_KNS::patch_scratch_bytes,
       PMG_KNS::patch_entries,
       PMG_KNS::patch_table,
+      PMG_KNS::cell_table_bytes,
+      PMG_KNS::cell_table,
+      PMG_KNS::cell_apply,
+      PMG_KNS::cell_apply_group,
   };
   return &t;
 }

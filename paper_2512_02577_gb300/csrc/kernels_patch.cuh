@@ -28,9 +28,9 @@
 // (8 bits each, exact), the six products of weight 2^-16 and above.
 //
 // Patch launch of one sweep, before and now (GB300): FP64 K = 4 at 32^3 cells
-// 2.344 and 0.210 ms (tensor pipe 40% of its cycles, issue slots 45%: the
+// 2.344 and 0.195 ms (tensor pipe 35% of its cycles, issue slots 40%: the
 // digit conversions and the 64-bit gather and scatter); FP64 K = 5 at 24^3
-// 2.12 and 0.38 ms; FP32 K = 4 at 32^3 0.135 and 0.055 ms (shared-memory and
+// 2.12 and 0.36 ms; FP32 K = 4 at 32^3 0.135 and 0.055 ms (shared-memory and
 // L1 wavefronts: 80% of their rate), K = 5 at 40^3 0.473 and 0.319 ms, K = 3
 // at 67^3 0.328 and 0.203 ms, K = 2 at 100^3 0.283 and 0.162 ms.
 #pragma once
@@ -45,20 +45,23 @@ namespace PMG_KNS {
 
 using TP = std::conditional_t<PMG_PREC == 0, double, float>;  // this part's precision
 
-// Sectors of the patch operator: sector s is odd in direction d where bit d
-// of s is set.  Even coefficients 0..K-1 (K-1: the centre node), odd ones
-// 0..K-2.  Patches of at most 32 nodes are not split: their single matrix
-// fits the same number of 16 x 16 tiles.
-template <int DIM>
+// Sectors of an operator on a window of M nodes per direction (a patch's
+// interior, M = 2K - 1, or a cell, M = K + 1): sector s is odd in direction d
+// where bit d of s is set.  Even coefficients 0..E-1 (E - 1: the centre node
+// if M is odd), odd ones 0..O-1.  Windows of at most 32 nodes are not split:
+// their single matrix fits the same number of 16 x 16 tiles.
+template <int DIM, int M_>
 struct Sectors {
-  static constexpr int M = mp(K);
+  static constexpr int M = M_;
   static constexpr int NODES = ipow(M, DIM);
   static constexpr bool SPLIT = NODES > 32;
   static constexpr int NS = SPLIT ? 1 << DIM : 1;
-  static constexpr int E = SPLIT ? K : M;          // coefficients per direction of an even sector
+  static constexpr int E = SPLIT ? (M + 1) / 2 : M;  // coefficients per direction of an even sector
+  static constexpr int O = SPLIT ? M / 2 : 0;        // and of an odd one
+  static constexpr bool CENTRE = SPLIT && E > O;     // coordinate E - 1 is its own mirror image
   static constexpr int ORBITS = ipow(E, DIM);      // nodes up to reflection
   static constexpr int IMAGES = SPLIT ? 1 << DIM : 1;
-  __host__ __device__ static constexpr int ext(int s, int d) { return d >= DIM ? 1 : ((s >> d) & 1) ? E - 1 : E; }
+  __host__ __device__ static constexpr int ext(int s, int d) { return d >= DIM ? 1 : ((s >> d) & 1) ? O : E; }
   __host__ __device__ static constexpr int size(int s) { return ext(s, 0) * ext(s, 1) * ext(s, 2); }
   __host__ __device__ static constexpr int tiles(int s) { return (size(s) + 15) / 16; }  // 16-row tiles per side
   // offsets of sector s: padded rows, rows, 16 x 16 tiles, matrix entries
@@ -72,9 +75,9 @@ struct Sectors {
 
 // An orbit: a node of the first orthant (coordinates 0..E-1) and its mirror
 // images; image b is mirrored in the directions of b's bits.
-template <int DIM>
+template <int DIM, int M>
 struct Orbit {
-  using S = Sectors<DIM>;
+  using S = Sectors<DIM, M>;
   int c[3];
   __device__ __forceinline__ explicit Orbit(int o) {
     c[0] = o % S::E;
@@ -86,7 +89,7 @@ struct Orbit {
   __device__ __forceinline__ bool has(int b) const {
     bool h = true;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) h = h && !(((b >> d) & 1) && c[d] == S::E - 1);
+    for (int d = 0; d < DIM; ++d) h = h && !(S::CENTRE && ((b >> d) & 1) && c[d] == S::E - 1);
     return h;
   }
   __device__ __forceinline__ int at(int d, int b) const { return ((b >> d) & 1) ? S::M - 1 - c[d] : c[d]; }
@@ -97,18 +100,18 @@ struct Orbit {
   __device__ __forceinline__ int centres() const {
     int n = 0;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) n += S::SPLIT && c[d] == S::E - 1;
+    for (int d = 0; d < DIM; ++d) n += S::CENTRE && c[d] == S::E - 1;
     return n;
   }
 };
 
-// Lines of a patch along x up to reflection in the other directions: line L
+// Lines of a window along x up to reflection in the other directions: line L
 // holds the nodes (0..M-1, c_1, c_2), c_d < E; image b is mirrored in
 // direction d where bit d - 1 of b is set.  A thread takes all images of a
 // line, so the offsets of its nodes and coefficients along x are immediates.
-template <int DIM>
+template <int DIM, int M>
 struct Lines {
-  using S = Sectors<DIM>;
+  using S = Sectors<DIM, M>;
   static constexpr int N = ipow(S::E, DIM - 1);
   static constexpr int IMAGES = S::SPLIT ? 1 << (DIM - 1) : 1;
   int c[2];
@@ -119,12 +122,12 @@ struct Lines {
   __device__ __forceinline__ bool has(int b) const {
     bool h = true;
 #pragma unroll
-    for (int d = 0; d < DIM - 1; ++d) h = h && !(((b >> d) & 1) && c[d] == S::E - 1);
+    for (int d = 0; d < DIM - 1; ++d) h = h && !(S::CENTRE && ((b >> d) & 1) && c[d] == S::E - 1);
     return h;
   }
   // directions in which the line passes through the centre
   __device__ __forceinline__ int centres() const {
-    return S::SPLIT ? (c[0] == S::E - 1) + (DIM == 3 && c[1] == S::E - 1) : 0;
+    return S::CENTRE ? (c[0] == S::E - 1) + (DIM == 3 && c[1] == S::E - 1) : 0;
   }
   // offset of image b's first node on a grid of N1 nodes per direction
   __device__ __forceinline__ int node(int b, int N1) const {
@@ -137,27 +140,27 @@ struct Lines {
 
 // even / odd combinations of a line's images in every direction: entry i of
 // image b becomes the coefficient of parity b in the other directions and,
-// along x, even coefficient i for i < K, odd coefficient M - 1 - i beyond.
+// along x, even coefficient i for i < E, odd coefficient M - 1 - i beyond.
 // (Its own inverse up to the factor 2 per direction, which the matrix absorbs.)
-template <int DIM, typename V>
-__device__ __forceinline__ void reflect(V (&v)[Lines<DIM>::IMAGES][Sectors<DIM>::M]) {
-  using S = Sectors<DIM>;
+template <int DIM, int M, typename V>
+__device__ __forceinline__ void reflect(V (&v)[Lines<DIM, M>::IMAGES][M]) {
+  using S = Sectors<DIM, M>;
   if constexpr (S::SPLIT) {
 #pragma unroll
-    for (int b = 0; b < Lines<DIM>::IMAGES; ++b)
+    for (int b = 0; b < Lines<DIM, M>::IMAGES; ++b)
 #pragma unroll
-      for (int i = 0; i < K - 1; ++i) {
-        const V e = v[b][i] + v[b][S::M - 1 - i], o = v[b][i] - v[b][S::M - 1 - i];
+      for (int i = 0; i < S::O; ++i) {
+        const V e = v[b][i] + v[b][M - 1 - i], o = v[b][i] - v[b][M - 1 - i];
         v[b][i] = e;
-        v[b][S::M - 1 - i] = o;
+        v[b][M - 1 - i] = o;
       }
 #pragma unroll
     for (int d = 0; d < DIM - 1; ++d)
 #pragma unroll
-      for (int b = 0; b < Lines<DIM>::IMAGES; ++b)
+      for (int b = 0; b < Lines<DIM, M>::IMAGES; ++b)
         if (!((b >> d) & 1))
 #pragma unroll
-          for (int i = 0; i < S::M; ++i) {
+          for (int i = 0; i < M; ++i) {
             const V e = v[b][i] + v[b | (1 << d)][i], o = v[b][i] - v[b | (1 << d)][i];
             v[b][i] = e;
             v[b | (1 << d)][i] = o;
@@ -166,31 +169,31 @@ __device__ __forceinline__ void reflect(V (&v)[Lines<DIM>::IMAGES][Sectors<DIM>:
 }
 
 // f(entry, sector, coefficient along x) for the entries of image b after reflect
-template <int DIM, class F>
+template <int DIM, int M, class F>
 __device__ __forceinline__ void for_coefs(int b, F&& f) {
-  using S = Sectors<DIM>;
+  using S = Sectors<DIM, M>;
 #pragma unroll
-  for (int i = 0; i < S::M; ++i) {
-    if (!S::SPLIT || i < K) f(i, 2 * b, i);
-    else f(i, 2 * b + 1, S::M - 1 - i);
+  for (int i = 0; i < M; ++i) {
+    if (i < S::E) f(i, S::SPLIT ? 2 * b : 0, i);
+    else f(i, 2 * b + 1, M - 1 - i);
   }
 }
 
 // ---------------------------------------------------------------- block shape
-// P patches per block (the n extent of the products), NW warps.  3D patches of
+// P windows per block (the n extent of the products), NW warps.  3D patches of
 // K >= 6 keep the sum-factorised kernel: their operands fill an SM's shared
 // memory with 8-16 patches, and the matrix is streamed from L2 for so few
 // columns (K = 6 FP32 at 33^3 cells: 0.67 ms against 0.49 ms).
-template <int DIM, typename T>
+template <int DIM, int M, typename T>
 struct Dense {
-  using S = Sectors<DIM>;
+  using S = Sectors<DIM, M>;
   static constexpr bool F64 = sizeof(T) == 8;
   static constexpr int SL = F64 ? 7 : 3;                        // parts per value
   static constexpr int P = 16;
   static constexpr int NT = P / 8;                              // 8-column tiles
   static constexpr int NSUB = 32 / P;                           // lines a warp handles at once
   static constexpr int UNITS = S::PROWS / 16;                   // 16-row tiles of the result
-  static constexpr int NW = UNITS >= 8 ? 8 : (UNITS > 2 ? 4 : 2);
+  static constexpr int NW = UNITS >= 16 ? 8 : (UNITS > 2 ? 4 : 2);
   static constexpr int UPW = (UNITS + NW - 1) / NW;             // units per warp
   // Operands: FP64 fixed-point values [row][XP], FP32 the three parts as
   // planes of BF16 [part][row][XP]; the pitch spreads the rows over the banks.
@@ -213,7 +216,7 @@ struct Dense {
     const int bs = 227 * 1024 / (SMEM + 1536), br = 65536 / (32 * NW * (F64 ? 128 : 64)), b = bs < br ? bs : br;
     return b < 1 ? 1 : (b > 8 ? 8 : b);
   }
-  static constexpr bool ok() { return K >= 2 && (DIM == 2 || K <= 5) && SMEM <= kMaxDynSmem; }
+  static constexpr bool ok() { return K >= 2 && M <= (DIM == 2 ? 15 : 9) && SMEM <= kMaxDynSmem; }
   // table: 16-byte fragments, then (FP64) per row its exponent above its
   // class's, and the exponents of the four classes (Orbit::centres)
   static constexpr int FRAGS = S::TILES * SL * 32;
@@ -232,10 +235,10 @@ template <int N>
 struct DenseUnits {
   DenseUnit u[N];
 };
-template <int DIM, typename T>
-constexpr DenseUnits<Dense<DIM, T>::UNITS> dense_units() {
-  using S = Sectors<DIM>;
-  DenseUnits<Dense<DIM, T>::UNITS> r{};
+template <int DIM, int M, typename T>
+constexpr DenseUnits<Dense<DIM, M, T>::UNITS> dense_units() {
+  using S = Sectors<DIM, M>;
+  DenseUnits<Dense<DIM, M, T>::UNITS> r{};
   int n = 0;
   for (int s = 0; s < S::NS; ++s)
     for (int m = 0; m < S::tiles(s); ++m) {
@@ -244,7 +247,7 @@ constexpr DenseUnits<Dense<DIM, T>::UNITS> dense_units() {
       u.kt = (short)S::tiles(s);
       u.row = (short)(S::row(s) + 16 * m);
       u.valid = (short)(S::size(s) - 16 * m < 16 ? S::size(s) - 16 * m : 16);
-      u.frag = (S::tile(s) + m * S::tiles(s)) * Dense<DIM, T>::SL;
+      u.frag = (S::tile(s) + m * S::tiles(s)) * Dense<DIM, M, T>::SL;
     }
   return r;
 }
@@ -328,94 +331,88 @@ constexpr int kMagicBits = 0x4B400000;
 // operand rows, in units of 2^-52 of (table integer x operand integer) at the
 // exponent of the row's class.  Two k tiles add at most 14 products of 2^18 to an
 // accumulator (below its exact range of 2^22 around kMagic) before it is
-// emptied into y.
-template <int DIM>
+// emptied into Y.
+template <class D>
 __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table, const long long* X,
                                           long long* Y, int lane) {
-  using D = Dense<DIM, double>;
   constexpr int SL = D::SL, NT = D::NT, ND = SL + 1;  // ND: digit sums kept, i + j < ND
   const int g = lane >> 2, q = lane & 3;
   const int* shift = reinterpret_cast<const int*>(table + D::FRAGS) + u.row + g;  // row exponent - its class's
-  long long y[NT][4] = {};
-  float acc[ND][NT][4];
-  auto reset = [&]() {
+  const uint4* tp = table + (int64_t)u.frag * 32 + lane;
+  const long long* xp = X + (u.prow + 2 * q) * D::XP + g;
+  for (int k0 = 0; k0 < u.kt; k0 += 2) {
+    float acc[ND][NT][4];
 #pragma unroll
     for (int d = 0; d < ND; ++d)
 #pragma unroll
       for (int t = 0; t < NT; ++t)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[d][t][i] = kMagic;
-  };
-  auto empty = [&]() {
-#pragma unroll
-    for (int t = 0; t < NT; ++t)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        auto pair = [&](int d) {
-          return (__float_as_int(acc[d][t][i]) - kMagicBits) * 256 + (__float_as_int(acc[d + 1][t][i]) - kMagicBits);
-        };
-        y[t][i] += ((long long)pair(0) << 36) + ((long long)pair(2) << 20) + ((long long)pair(4) << 4) +
-                   ((pair(6) + 2048) >> 12);  // rounded: a bias would add up over the mirror images
-      }
-  };
-  reset();
-  const uint4* tp = table + (int64_t)u.frag * 32 + lane;
-  for (int k = 0; k < u.kt; ++k) {
-    // digits of the operand values of rows 2q, 2q+1, 2q+8, 2q+9 of the tile
-    uint32_t b[SL][NT][2];
-#pragma unroll
-    for (int t = 0; t < NT; ++t)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const long long* x = X + (u.prow + 16 * k + 2 * q + 8 * h) * D::XP + 8 * t + g;
-        // biased so that byte SL - 1 - j holds digit j + 128
-        const long long w0 = x[0] + 0x0080808080808080ll, w1 = x[D::XP] + 0x0080808080808080ll;
-#pragma unroll
-        for (int j = 0; j < SL; ++j) {
-          const int byte = SL - 1 - j, bb = byte & 3;
-          const uint32_t v0 = (uint32_t)(byte < 4 ? w0 : w0 >> 32), v1 = (uint32_t)(byte < 4 ? w1 : w1 >> 32);
-          const uint32_t pr = __byte_perm(v0, v1, bb | (bb << 4) | ((4 + bb) << 8) | ((4 + bb) << 12));
-          const uint32_t hb = (pr & 0x00FF00FFu) | 0x64006400u;  // 1024 + digit + 128 as halves
-          const __half2 dg = __hsub2(*reinterpret_cast<const __half2*>(&hb), __half2half2(__ushort_as_half(0x6480)));
-          b[j][t][h] = *reinterpret_cast<const uint32_t*>(&dg);
-        }
-      }
-#pragma unroll
-    for (int i = 0; i < SL; ++i) {
-      const uint4 a = __ldg(tp + (k * SL + i) * 32);
-#pragma unroll
-      for (int j = 0; j < SL; ++j)
-        if (i + j < ND) {
-#pragma unroll
-          for (int t = 0; t < NT; ++t) mma_f16(acc[i + j][t], a, b[j][t][0], b[j][t][1]);
-        }
-    }
-    if ((k & 1) && k + 1 < u.kt) {
-      empty();
-      reset();
-    }
-  }
-  empty();
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-    if (g + 8 * h < u.valid) {
-      const int sh = __ldg(shift + 8 * h);
-      const long long half = (1ll << sh) >> 1;
+    for (int k = k0; k < min(k0 + 2, (int)u.kt); ++k) {
+      uint4 a = __ldg(tp + k * SL * 32);
+      // digits of the operand values of rows 2q, 2q+1, 2q+8, 2q+9 of the tile
+      uint32_t b[SL][NT][2];
 #pragma unroll
       for (int t = 0; t < NT; ++t)
 #pragma unroll
-        for (int i = 0; i < 2; ++i) Y[(u.row + g + 8 * h) * D::YP + 8 * t + 2 * q + i] = (y[t][2 * h + i] + half) >> sh;
+        for (int h = 0; h < 2; ++h) {
+          const long long* x = xp + (16 * k + 8 * h) * D::XP + 8 * t;
+          // biased so that byte SL - 1 - j holds digit j + 128
+          const long long w0 = x[0] + 0x0080808080808080ll, w1 = x[D::XP] + 0x0080808080808080ll;
+#pragma unroll
+          for (int j = 0; j < SL; ++j) {
+            const int byte = SL - 1 - j, bb = byte & 3;
+            const uint32_t v0 = (uint32_t)(byte < 4 ? w0 : w0 >> 32), v1 = (uint32_t)(byte < 4 ? w1 : w1 >> 32);
+            const uint32_t pr = __byte_perm(v0, v1, bb | (bb << 4) | ((4 + bb) << 8) | ((4 + bb) << 12));
+            const uint32_t hb = (pr & 0x00FF00FFu) | 0x64006400u;  // 1024 + digit + 128 as halves
+            const __half2 dg = __hsub2(*reinterpret_cast<const __half2*>(&hb), __half2half2(__ushort_as_half(0x6480)));
+            b[j][t][h] = *reinterpret_cast<const uint32_t*>(&dg);
+          }
+        }
+#pragma unroll
+      for (int i = 0; i < SL; ++i) {
+        const uint4 next = i + 1 < SL ? __ldg(tp + (k * SL + i + 1) * 32) : a;
+#pragma unroll
+        for (int j = 0; j < SL; ++j)
+          if (i + j < ND) {
+#pragma unroll
+            for (int t = 0; t < NT; ++t) mma_f16(acc[i + j][t], a, b[j][t][0], b[j][t][1]);
+          }
+        a = next;
+      }
     }
+    // into Y: partial sums at the row's exponent, at the end rounded to the class's
+    const bool last = k0 + 2 >= u.kt;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (g + 8 * h < u.valid) {
+        const int sh = last ? __ldg(shift + 8 * h) : 0;
+        const long long half = (1ll << sh) >> 1;
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            auto pair = [&](int d) {
+              return (__float_as_int(acc[d][t][2 * h + i]) - kMagicBits) * 256 +
+                     (__float_as_int(acc[d + 1][t][2 * h + i]) - kMagicBits);
+            };
+            long long* y = Y + (u.row + g + 8 * h) * D::YP + 8 * t + 2 * q + i;
+            // rounded, not cut off: a bias would add up over the mirror images
+            const long long v = ((long long)pair(0) << 36) + ((long long)pair(2) << 20) + ((long long)pair(4) << 4) +
+                                ((pair(6) + 2048) >> 12) + (k0 ? *y : 0);
+            *y = (v + half) >> sh;
+          }
+      }
+  }
 }
 
 // FP32 products of one unit into y.  The leading products are taken out of
 // the accumulator after every k tile and summed with rounding (the tensor
 // cores truncate their sums); the five small products share an accumulator.
-template <int DIM>
+template <class D>
 __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table, const uint16_t* X,
-                                          float (&y)[Dense<DIM, float>::NT][4], int lane) {
-  using D = Dense<DIM, float>;
-  using S = Sectors<DIM>;
+                                          float (&y)[D::NT][4], int lane) {
+  using S = typename D::S;
   constexpr int SL = D::SL, NT = D::NT;
   float lo[NT][4] = {};
 #pragma unroll
@@ -455,17 +452,28 @@ __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __res
     for (int i = 0; i < 4; ++i) y[t][i] += lo[t][i];
 }
 
-static __constant__ const DenseUnits<Dense<PMG_DIM, TP>::UNITS> c_units = dense_units<PMG_DIM, TP>();
+// the patch's window and the cell's (FP64 operator apply)
+constexpr int kPatchM = mp(K), kCellM = K + 1;
+static __constant__ const DenseUnits<Dense<PMG_DIM, kPatchM, TP>::UNITS> c_units = dense_units<PMG_DIM, kPatchM, TP>();
+#if PMG_PREC == 0
+static __constant__ const DenseUnits<Dense<PMG_DIM, kCellM, double>::UNITS> c_cell_units =
+    dense_units<PMG_DIM, kCellM, double>();
+#endif
 
 // The patches of batch `batch` of a level: gather r_j, even / odd
 // combinations, products, and back; omega_AS d_j to the colour's vector
 // (additive) or d_j added to u (multiplicative).  A lane holds one patch (P
 // lanes) and the warps share the nodes, so index arithmetic is uniform and
 // shared-memory accesses fall on consecutive patches.
-template <int DIM, typename T>
+//
+// CELL: the windows are cells, the matrix the element stiffness matrix of
+// Eq. (3) at unit scale; boundary nodes are read as zero and the results go
+// to the cell's block of dst (summed per node by cell_sum).
+template <int DIM, typename T, bool CELL>
 __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch) {
-  using S = Sectors<DIM>;
-  using D = Dense<DIM, T>;
+  constexpr int M = CELL ? kCellM : kPatchM;
+  using S = Sectors<DIM, M>;
+  using D = Dense<DIM, M, T>;
   constexpr int P = D::P, NSUB = D::NSUB, NW = D::NW;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int64_t s_base[P];
@@ -479,15 +487,23 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
   const uint32_t pid = batch * P + pn;
   const bool active = pid < J.npatch;
   int64_t base;
+  unsigned edge = 0;  // CELL: bits of the grid's boundary faces that the cell touches
   {
     const uint32_t t = active ? pid : 0, r1 = J.d0.div(t), r2 = J.d1.div(r1);
     const int i[3] = {(int)(t - r1 * J.d0.d), (int)(DIM == 3 ? r1 - r2 * J.d1.d : r1), (int)(DIM == 3 ? r2 : 0)};
     int v[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d)
-      v[d] = J.colour < 0 ? i[d] + 1 : 2 * i[d] + (((J.colour >> d) & 1) ? 1 : 2);
-    base = (int64_t)(K * (v[0] - 1) + 1) + (int64_t)N1 * (K * (v[1] - 1) + 1);
-    if (DIM == 3) base += (int64_t)N1 * N1 * (K * (v[2] - 1) + 1);
+    for (int d = 0; d < 3; ++d) {
+      if constexpr (CELL) {
+        v[d] = i[d];
+        edge |= (v[d] == 0 ? 1u << (2 * d) : 0u) | (v[d] == J.n - 1 ? 2u << (2 * d) : 0u);
+      } else {
+        v[d] = J.colour < 0 ? i[d] + 1 : 2 * i[d] + (((J.colour >> d) & 1) ? 1 : 2);
+      }
+    }
+    const int o = CELL ? 0 : 1;  // a window starts at node K (v - o) + o
+    base = (int64_t)(K * (v[0] - o) + o) + (int64_t)N1 * (K * (v[1] - o) + o);
+    if (DIM == 3) base += (int64_t)N1 * N1 * (K * (v[2] - o) + o);
     if (threadIdx.x < P) {
       s_base[pn] = active ? base : -1;
       s_colour[pn] = J.colour < 0 ? (v[0] & 1) | ((v[1] & 1) << 1) | (DIM == 3 ? (v[2] & 1) << 2 : 0) : 0;
@@ -495,7 +511,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     }
   }
   const T* rp = J.r + base;
-  using L = Lines<DIM>;
+  using L = Lines<DIM, M>;
   using XT = std::conditional_t<D::F64, long long, uint16_t>;
   using YT = std::conditional_t<D::F64, long long, float>;
   XT* X = reinterpret_cast<XT*>(smraw);
@@ -516,21 +532,26 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
   }
   int e = 0;         // FP64: biased exponent bound of the patch's values
   bool bad = false;  // FP64: an infinity or NaN among them
-  bool tiny = false;
+  bool tiny = false, any_tiny = false;
   const int* classexp = reinterpret_cast<const int*>(J.table + D::FRAGS) + S::ROWS;
   if constexpr (D::F64) {
     __syncthreads();  // s_max
     double* R = reinterpret_cast<double*>(Y);
     unsigned mx = 0;
     for (int l = item0; l < S::NODES / S::M; l += STEP) {
-      const double* q = rp + N1 * (DIM == 3 ? l % S::M + N1 * (l / S::M) : l);
-      double v[S::M];
+      const int ly = DIM == 3 ? l % M : l, lz = DIM == 3 ? l / M : 0;
+      const double* q = rp + N1 * (ly + N1 * lz);
+      const bool in = active && !(CELL && (((edge & 4) && ly == 0) || ((edge & 8) && ly == M - 1) ||
+                                           (DIM == 3 && (((edge & 16) && lz == 0) || ((edge & 32) && lz == M - 1)))));
+      double v[M];
 #pragma unroll
-      for (int i = 0; i < S::M; ++i) v[i] = active ? q[i] : 0.0;
+      for (int i = 0; i < M; ++i)
+        v[i] = in && !(CELL && ((i == 0 && (edge & 1)) || (i == M - 1 && (edge & 2)))) ? q[i] : 0.0;
 #pragma unroll
       for (int i = 0; i < S::M; ++i) {
         R[(l * S::M + i) * P + pn] = v[i];
-        mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu);
+        // the low bit: a value below the high word's range is not zero
+        mx = max(mx, ((unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu) | (__double2loint(v[i]) != 0));
       }
     }
 #pragma unroll
@@ -542,7 +563,9 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     // the bound leaves 0.8% to the top digit's range; subnormal patches are
     // scaled by 2^100 and bounded by the high word's leading bit
     tiny = mx < 0x00100000u;
-    e = tiny ? 113 - __clz((int)mx) : (int)((mx + 0x4000u) >> 20);
+    any_tiny = __any_sync(0xffffffffu, tiny && mx != 0);  // the products with 2^100 only where needed
+    tiny = tiny && any_tiny;
+    e = tiny ? 113 - __clz((int)mx) : max((int)((mx + 0x4000u) >> 20), 1);
   }
   // even / odd combinations, stored as operands
   for (int l = item0; l < L::N; l += STEP) {
@@ -553,17 +576,23 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
 #pragma unroll
       for (int b = 0; b < L::IMAGES; ++b) {
         const double* q = R + ln.node(b, S::M) * P + pn;
+        double r[M];
 #pragma unroll
-        for (int i = 0; i < S::M; ++i)
-          v[b][i] = ln.has(b) || !S::SPLIT ? fixed_of(tiny ? q[i * P] * 0x1p100 : q[i * P], e) : 0;
+        for (int i = 0; i < M; ++i) r[i] = ln.has(b) || !S::SPLIT ? q[i * P] : 0.0;
+        if (any_tiny) {
+#pragma unroll
+          for (int i = 0; i < M; ++i) r[i] = tiny ? r[i] * 0x1p100 : r[i];
+        }
+#pragma unroll
+        for (int i = 0; i < M; ++i) v[b][i] = fixed_of(r[i], e);
       }
-      reflect<DIM>(v);
+      reflect<DIM, M>(v);
       const int sh0 = (S::SPLIT ? DIM + 3 : 3) - ln.centres();  // to 55 bits and sign: 2^(d-c) images were summed
 #pragma unroll
       for (int b = 0; b < L::IMAGES; ++b)
         if (ln.has(b) || !S::SPLIT)
-          for_coefs<DIM>(b, [&](int i, int s, int ox) {
-            const int sh = S::SPLIT && i == K - 1 ? sh0 - 1 : sh0;
+          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
+            const int sh = S::CENTRE && i == S::E - 1 ? sh0 - 1 : sh0;
             X[(S::prow(s) + ox + ln.coef(s)) * D::XP + pn] = (v[b][i] + (1ll << (sh - 1))) >> sh;
           });
     } else {
@@ -575,11 +604,11 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
 #pragma unroll
         for (int i = 0; i < S::M; ++i) v[b][i] = in ? q[i] : 0.f;
       }
-      reflect<DIM>(v);
+      reflect<DIM, M>(v);
 #pragma unroll
       for (int b = 0; b < L::IMAGES; ++b)
         if (ln.has(b) || !S::SPLIT)
-          for_coefs<DIM>(b, [&](int i, int s, int ox) {
+          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
             XT* x = X + (S::prow(s) + ox + ln.coef(s)) * D::XP + pn;
             const uint32_t b1 = __float_as_uint(v[b][i]);
             const float f2 = v[b][i] - __uint_as_float(b1 & 0xFFFF0000u);
@@ -593,12 +622,16 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
   }
   __syncthreads();
   if constexpr (D::F64) {
-    for (int u = warp; u < D::UNITS; u += NW) dense_mma<DIM>(c_units.u[u], J.table, X, Y, lane);
+    for (int u = warp; u < D::UNITS; u += NW) {
+#if PMG_PREC == 0
+      dense_mma<D>(CELL ? c_cell_units.u[CELL ? u : 0] : c_units.u[CELL ? 0 : u], J.table, X, Y, lane);
+#endif
+    }
   } else {
     float y[D::UPW][D::NT][4];
 #pragma unroll
     for (int i = 0; i < D::UPW; ++i)
-      if (warp + i * NW < D::UNITS) dense_mma<DIM>(c_units.u[warp + i * NW], J.table, X, y[i], lane);
+      if (warp + i * NW < D::UNITS) dense_mma<D>(c_units.u[warp + i * NW], J.table, X, y[i], lane);
     __syncthreads();  // the results take the operands' place
 #pragma unroll
     for (int i = 0; i < D::UPW; ++i)
@@ -623,11 +656,11 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
 #pragma unroll
     for (int b = 0; b < L::IMAGES; ++b) {
       const bool in = ln.has(b) || !S::SPLIT;
-      for_coefs<DIM>(b, [&](int i, int s, int ox) {
+      for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
         v[b][i] = in ? Y[(S::row(s) + ox + ln.coef(s)) * D::YP + pn] : YT(0);
       });
     }
-    reflect<DIM>(v);
+    reflect<DIM, M>(v);
 #pragma unroll
     for (int b = 0; b < L::IMAGES; ++b)
       if (ln.has(b) || !S::SPLIT) {
@@ -637,13 +670,22 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
 #pragma unroll
         for (int i = 0; i < S::M; ++i) {
           if constexpr (D::F64)
-            z[i] = bad ? __longlong_as_double(0x7FF8000000000000ll) : double_of(v[b][i], J.cmul, S::SPLIT && i == K - 1 ? ve1 : ve0);
+            z[i] = bad ? __longlong_as_double(0x7FF8000000000000ll) : double_of(v[b][i], J.cmul, S::CENTRE && i == S::E - 1 ? ve1 : ve0);
           else
             z[i] = J.c * v[b][i];
         }
       }
   }
   __syncthreads();
+  if constexpr (CELL) {  // the block's cells are consecutive, like their results
+    T* o = J.dst + (int64_t)batch * P * S::NODES;
+    const int cells = min(P, (int)(J.npatch - batch * P));
+    for (int i = threadIdx.x; i < cells * S::NODES; i += 32 * NW) {
+      const int gp = i / S::NODES;
+      o[i] = Z[gp * D::ZP + i - gp * S::NODES];
+    }
+    return;
+  }
   // a warp writes a patch; each lane keeps the offsets of its nodes
   constexpr int NO = (S::NODES + 31) / 32;
   int off[NO];
@@ -670,16 +712,119 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
 }
 
 template <int DIM, typename T>
-__global__ void __launch_bounds__(32 * Dense<DIM, T>::NW, Dense<DIM, T>::MINB()) patch_dense_kernel(const __grid_constant__ DenseJob<T> J) {
-  dense_body<DIM, T>(J, blockIdx.x);
+using PatchDense = Dense<DIM, kPatchM, T>;
+template <int DIM>
+using CellDense = Dense<DIM, kCellM, double>;
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::MINB())
+    patch_dense_kernel(const __grid_constant__ DenseJob<T> J) {
+  dense_body<DIM, T, false>(J, blockIdx.x);
 }
 
 // Grouped launch: the batches of all jobs, job after job
 template <int DIM, typename T>
-__global__ void __launch_bounds__(32 * Dense<DIM, T>::NW, Dense<DIM, T>::MINB())
+__global__ void __launch_bounds__(32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::MINB())
     patch_dense_group_kernel(const __grid_constant__ GroupOf<DenseJob<T>> G) {
   const int j = group_find(G, blockIdx.x);
-  dense_body<DIM, T>(G.job[j], blockIdx.x - (uint32_t)G.start[j]);
+  dense_body<DIM, T, false>(G.job[j], blockIdx.x - (uint32_t)G.start[j]);
+}
+
+// FP64 operator apply on Cartesian meshes: cell results, one block of dst per
+// cell, then cell_sum per node.  The line passes (cart_pass) are bound by the
+// FP64 pipe; here it only sums the one to 2^d cells of a node.  One apply,
+// before and now: 3D K = 4 at 32^3 cells 0.231 and 0.112 ms, K = 2 at 100^3
+// 0.62 and 0.52, K = 3 at 67^3 0.72 and 0.43, K = 6 at 33^3 1.01 and 0.35,
+// K = 8 at 25^3 1.23 and 0.57; 2D K = 8 at 300^2 0.51 and 0.18.
+template <int DIM>
+__global__ void __launch_bounds__(32 * CellDense<DIM>::NW, CellDense<DIM>::MINB())
+    cell_dense_kernel(const __grid_constant__ DenseJob<double> J) {
+  dense_body<DIM, double, true>(J, blockIdx.x);
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(32 * CellDense<DIM>::NW, CellDense<DIM>::MINB())
+    cell_dense_group_kernel(const __grid_constant__ GroupOf<DenseJob<double>> G) {
+  const int j = group_find(G, blockIdx.x);
+  dense_body<DIM, double, true>(G.job[j], blockIdx.x - (uint32_t)G.start[j]);
+}
+
+// y = sum of the cells' results at each node, or b - that sum; boundary nodes
+// of y are 0.  Cells in a fixed order: the node's own, then its lower
+// neighbours in x, y and z.
+template <int DIM>
+struct CellSumJob {
+  const double* cells;
+  const double* b;
+  double* y;
+  int n;
+  FastDiv dN1;
+};
+
+template <int DIM>
+__device__ __forceinline__ void cell_sum(const CellSumJob<DIM>& J, int64_t t) {
+  constexpr int n1 = K + 1, NP = ipow(n1, DIM);
+  const int N1 = K * J.n + 1, n = J.n;
+  int g[3];
+  const int64_t N = (int64_t)N1 * N1 * (DIM == 3 ? N1 : 1);
+  if (N < kFastDivItems) {
+    const uint32_t v = (uint32_t)t, r = J.dN1.div(v), z = DIM == 3 ? J.dN1.div(r) : 0;
+    g[0] = (int)(v - r * J.dN1.d);
+    g[1] = (int)(r - z * J.dN1.d);
+    g[2] = (int)z;
+  } else {
+    g[0] = (int)(t % N1);
+    g[1] = (int)((t / N1) % N1);
+    g[2] = DIM == 3 ? (int)(t / ((int64_t)N1 * N1)) : 0;
+  }
+  bool bnd = false;
+  int c[3] = {0, 0, 0}, a[3] = {0, 0, 0};
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) {
+    bnd = bnd || g[d] == 0 || g[d] == N1 - 1;
+    c[d] = g[d] / K;
+    a[d] = g[d] - K * c[d];
+  }
+  if (bnd) {
+    J.y[t] = 0.0;
+    return;
+  }
+  // an interior node with a_d = 0 also lies on cell c_d - 1, at its end
+  const double* p = J.cells + (c[0] + (int64_t)n * (c[1] + (DIM == 3 ? (int64_t)n * c[2] : 0))) * NP + a[0] +
+                    n1 * (a[1] + (DIM == 3 ? n1 * a[2] : 0));
+  double v[1 << DIM];
+  bool has[1 << DIM];
+#pragma unroll
+  for (int s = 0; s < 1 << DIM; ++s) {
+    int64_t o = 0;
+    has[s] = true;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d)
+      if ((s >> d) & 1) {
+        has[s] = has[s] && a[d] == 0;
+        o -= (d == 0 ? 1 : (d == 1 ? (int64_t)n : (int64_t)n * n)) * NP - K * (d == 0 ? 1 : (d == 1 ? n1 : n1 * n1));
+      }
+    v[s] = has[s] ? p[o] : 0.0;
+  }
+  double r = v[0];
+#pragma unroll
+  for (int s = 1; s < 1 << DIM; ++s)
+    if (__any_sync(__activemask(), has[s])) r = has[s] ? r + v[s] : r;  // FP64 adds only where a lane needs one
+  J.y[t] = J.b ? J.b[t] - r : r;
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(256) cell_sum_kernel(const __grid_constant__ CellSumJob<DIM> J, int64_t N) {
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (t < N) cell_sum<DIM>(J, t);
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(256) cell_sum_group_kernel(const __grid_constant__ GroupOf<CellSumJob<DIM>> G) {
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (t >= G.start[G.count]) return;
+  const int j = group_find(G, t);
+  cell_sum<DIM>(G.job[j], t - G.start[j]);
 }
 
 // K = 1: the patch is its vertex, the local solve one multiplication by
@@ -721,7 +866,7 @@ __global__ void __launch_bounds__(256) patch_point_group_kernel(const __grid_con
 template <int DIM, typename V>
 __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__ out, int np, bool first,
                                                             const double* __restrict__ dinv, PatchParams<double> H) {
-  using S = Sectors<DIM>;
+  using S = Sectors<DIM, kPatchM>;
   using PS = PatchShape<DIM>;
   constexpr int SZT = PS::SZT, RT = PS::off_r(PS::L - 1), DT = PS::off_d(PS::L - 1);
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -737,7 +882,7 @@ __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__
   P.colour = H.colour;
   const CartGeo<DIM, V> geo{dinv, P.scale, P.inv_scale, P.inv_a0};
   pfor<SZT>(pb, [&](int g, int i) {
-    pb.at(g)[RT + i] = V(i == Orbit<DIM>(c0 + g).node(0) ? 1.0 : 0.0);
+    pb.at(g)[RT + i] = V(i == Orbit<DIM, kPatchM>(c0 + g).node(0) ? 1.0 : 0.0);
     if (!first) pb.at(g)[DT + i] = V(out[(int64_t)(c0 + g) * SZT + i]);
   });
   __syncthreads();
@@ -752,41 +897,76 @@ __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__
   });
 }
 
-// Sector matrices from the columns, one warp per row: the entry for
-// coefficient j is the signed sum of column j over the mirror images of the
-// row's node, over 2^d -- the operand of an orbit with c central coordinates,
-// which has only 2^(d-c) images, counts 2^c times.  rowexp: the largest exponent x
-// with entry 2^x below 0.98 2^55 (7 signed digits reach 127/128 of 2^55) and
-// the row's sum of magnitudes times 2^x below 2^57 (results and their even /
-// odd sums stay within 64 bits).  The sectors' results for one orbit are
-// summed, so they need a common exponent: minexp, the least one of the rows
-// of a class -- the nodes with the same number of central coordinates, whose
-// coefficients have the same size (kNoExp if an entry is not finite).
-template <int DIM>
-__global__ void __launch_bounds__(128) patch_entries_kernel(const double* __restrict__ columns,
-                                                            double* __restrict__ entries, int* __restrict__ rowexp,
-                                                            int* __restrict__ minexp) {
-  using S = Sectors<DIM>;
+// coefficient k of sector s: its orbit
+template <int DIM, int M>
+__device__ __forceinline__ Orbit<DIM, M> orbit_of(int s, int k) {
+  using S = Sectors<DIM, M>;
+  const int e0 = S::ext(s, 0), e1 = S::ext(s, 1);
+  return Orbit<DIM, M>(k % e0 + S::E * ((k / e0) % e1 + S::E * (k / (e0 * e1))));
+}
+
+// Sector matrices, one warp per row: the entry of row m and coefficient j is
+// the signed sum over the mirror images of m's node of the operator's entry
+// for j's node, over 2^d -- the operand of an orbit with c central
+// coordinates, which has only 2^(d-c) images, counts 2^c times.  Patch: from
+// the columns; cell: from the 1D element matrices (coef: the coefficient
+// block), in pairs of doubles.
+// rowexp: the largest exponent x with entry 2^x below 0.98 2^55 (7 signed
+// digits reach 127/128 of 2^55) and the row's sum of magnitudes times 2^x
+// below 2^57 (results and their even / odd sums stay within 64 bits).  The
+// sectors' results for one orbit are summed, so they need a common exponent:
+// minexp, the least one of the rows of a class -- the nodes with the same
+// number of central coordinates, whose coefficients have the same size
+// (kNoExp if an entry is not finite).
+template <int DIM, bool CELL>
+__global__ void __launch_bounds__(128) sector_entries_kernel(const double* __restrict__ columns,
+                                                             double* __restrict__ entries, int* __restrict__ rowexp,
+                                                             int* __restrict__ minexp) {
+  constexpr int M = CELL ? kCellM : kPatchM;
+  using S = Sectors<DIM, M>;
   const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= S::ROWS) return;
   int s = 0;
   while (s + 1 < S::NS && row >= S::row(s + 1)) ++s;
-  const int m = row - S::row(s), sz = S::size(s), e0 = S::ext(s, 0), e1 = S::ext(s, 1);
-  auto orbit_of = [&](int k) { return k % e0 + S::E * ((k / e0) % e1 + S::E * (k / (e0 * e1))); };
-  const Orbit<DIM> om(orbit_of(m));
+  const int m = row - S::row(s), sz = S::size(s);
+  const Orbit<DIM, M> om = orbit_of<DIM, M>(s, m);
   double* out = entries + S::entry(s) + (int64_t)m * sz;
   double top = 0.0, sum = 0.0;
   for (int k = lane; k < sz; k += 32) {
-    const Orbit<DIM> oj(orbit_of(k));
-    const double* col = columns + (int64_t)orbit_of(k) * S::NODES;
-    double a = 0.0;
+    const Orbit<DIM, M> oj = orbit_of<DIM, M>(s, k);
+    double a;
+    if constexpr (CELL) {
+      const double* C = coef<double>();
+      dd f[2][3];  // 1D mass and stiffness between the two coefficients, per direction
 #pragma unroll
-    for (int b = 0; b < S::IMAGES; ++b) {
-      if (S::IMAGES > 1 && !oj.has(b)) continue;
-      const double v = col[om.node(b)];
-      a += (__popc(s & b) & 1) ? -v : v;
+      for (int d = 0; d < DIM; ++d)
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+          const double* T1 = C + (w ? LAY.Ke : LAY.Me) + oj.c[d];
+          const double r = T1[om.c[d] * M], q = T1[(M - 1 - om.c[d]) * M];
+          const bool centre = S::CENTRE && oj.c[d] == S::E - 1;  // one image in this direction
+          f[w][d] = !S::SPLIT ? dd(r) : centre ? dd(0.5 * r) : 0.5 * (dd(r) + dd(((s >> d) & 1) ? -q : q));
+        }
+      dd acc(0.0);
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) {
+        dd p = f[d == 0][0];
+#pragma unroll
+        for (int e = 1; e < DIM; ++e) p = p * f[d == e][e];
+        acc += p;
+      }
+      a = value_of(acc);
+    } else {
+      const double* col = columns + (int64_t)(oj.c[0] + S::E * (oj.c[1] + S::E * oj.c[2])) * S::NODES;
+      a = 0.0;
+#pragma unroll
+      for (int b = 0; b < S::IMAGES; ++b) {
+        if (S::IMAGES > 1 && !oj.has(b)) continue;
+        const double v = col[om.node(b)];
+        a += (__popc(s & b) & 1) ? -v : v;
+      }
+      a /= S::IMAGES;
     }
-    a /= S::IMAGES;
     out[k] = a;
     top = fmax(top, fabs(a));
     sum += fabs(a);
@@ -810,11 +990,15 @@ __global__ void __launch_bounds__(128) patch_entries_kernel(const double* __rest
 // lane l holds rows l / 4 and l / 4 + 8, columns 2 (l % 4) and + 8.  FP64:
 // 8-bit signed digits of entry 2^(the row's exponent, at most 15 above its
 // class's); FP32: three BF16 parts, rounded.
-template <int DIM, typename T>
-__global__ void patch_table_kernel(const double* __restrict__ entries, const int* __restrict__ rowexp,
-                                   const int* __restrict__ minexp, uint32_t* __restrict__ table) {
-  using S = Sectors<DIM>;
-  constexpr int SL = Dense<DIM, T>::SL;
+template <int DIM, typename T, bool CELL>
+__global__ void __launch_bounds__(256) sector_table_kernel(const double* __restrict__ entries,
+                                                           const int* __restrict__ rowexp,
+                                                           const int* __restrict__ minexp,
+                                                           uint32_t* __restrict__ table) {
+  constexpr int M = CELL ? kCellM : kPatchM;
+  using S = Sectors<DIM, M>;
+  using D = Dense<DIM, M, T>;
+  constexpr int SL = D::SL;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)S::TILES * 32 * 4) return;
   const int reg = (int)(t & 3), lane = (int)(t >> 2) & 31, tile = (int)(t >> 7);
@@ -824,11 +1008,9 @@ __global__ void patch_table_kernel(const double* __restrict__ entries, const int
   const int m = 16 * mt + (lane >> 2) + 8 * (reg & 1), k0 = 16 * kt + 2 * (lane & 3) + 8 * (reg >> 1);
   int re = 0;
   if (sizeof(T) == 8 && m < sz) {
-    const int e0 = S::ext(s, 0), e1 = S::ext(s, 1);
-    const Orbit<DIM> om(m % e0 + S::E * ((m / e0) % e1 + S::E * (m / (e0 * e1))));
-    const int exp = minexp[om.centres()];
+    const int exp = minexp[orbit_of<DIM, M>(s, m).centres()];
     re = min(rowexp[S::row(s) + m], exp + 15);
-    int* tail = reinterpret_cast<int*>(table + (int64_t)Dense<DIM, T>::FRAGS * 4);
+    int* tail = reinterpret_cast<int*>(table + (int64_t)D::FRAGS * 4);
     if (kt == 0 && (lane & 3) == 0 && reg < 2) tail[S::row(s) + m] = re - exp;
     if (tile == 0 && lane == 0 && reg == 0)
       for (int i = 0; i < 4; ++i) tail[S::ROWS + i] = minexp[i];
@@ -844,9 +1026,8 @@ __global__ void patch_table_kernel(const double* __restrict__ entries, const int
         part[i] |= (uint32_t)__half_as_ushort(__int2half_rn(digit)) << (16 * h);
       }
     } else {
-      const int e0 = S::ext(s, 0), e1 = S::ext(s, 1), kk = k < sz ? k : 0;
-      const Orbit<DIM> oj(kk % e0 + S::E * ((kk / e0) % e1 + S::E * (kk / (e0 * e1))));
-      double rest = a * (1 << oj.centres());  // FP32 operands are plain sums over the images
+      // FP32 operands are plain sums over the images
+      double rest = a * (1 << orbit_of<DIM, M>(s, k < sz ? k : 0).centres());
       for (int i = 0; i < SL; ++i) {
         const __nv_bfloat16 p = __double2bfloat16(rest);
         rest -= (double)__bfloat162float(p);

@@ -219,10 +219,11 @@ int make_plan(const pmg_config* cfg, Plan& P) {
   P.pbuf = bump(cur, (int64_t)(1 << P.dim) * ipow64((int64_t)P.K * nf + 1, P.dim) * P.mg_es);
   if (!P.deformed) {
     const int64_t tb = kernel_table(P.K, P.dim, cfg->mg_precision)->patch_table_bytes(P.dim, cfg->mg_precision);
-    if (tb > 0) {
-      P.table = bump(cur, tb);
-      P.tscratch = bump(cur, kernel_table(P.K, P.dim, PMG_FP64)->patch_scratch_bytes(P.dim));
-    }
+    const KernelTable* k64 = kernel_table(P.K, P.dim, PMG_FP64);
+    const int64_t cb = k64->cell_table_bytes(P.dim);
+    if (tb > 0) P.table = bump(cur, tb);
+    if (cb > 0) P.ctable = bump(cur, cb);
+    if (tb > 0 || cb > 0) P.tscratch = bump(cur, k64->patch_scratch_bytes(P.dim));
   }
   if (cfg->geometry == PMG_GEOM_DISTORTED) P.verts = bump(cur, ipow64(nf + 1, P.dim) * P.dim * 8);
   if (P.deformed) P.cellbuf = bump(cur, ipow64(nf, P.dim) * ipow64(P.K + 1, P.dim) * 8);
@@ -297,6 +298,10 @@ int level_apply(pmg_ctx* c, int level, int prec, const void* u, void* r, const v
   } else if (c->deformed) {
     e = c->kt[prec]->def_apply(c->dim, prec, u, r, b, L.G[c->nplev - 1], c->cfg.geom_precision, c->cellbuf, L.n,
                                prec == c->mgprec ? c->def_cpb : 0, c->stream);
+  } else if (prec == PMG_FP64 && c->ctable) {
+    // the four scratch vectors hold the cells' results: (K+1)^d n^d <= 4 (K n + 1)^d for K >= 2
+    e = c->kt[PMG_FP64]->cell_apply(c->dim, (const double*)u, (double*)r, (const double*)b, c->t64[0], c->ctable, L.n,
+                                    L.scale, c->stream);
   } else {
     void** t = prec == PMG_FP64 ? (void**)c->t64 : c->t_mg;
     e = c->kt[prec]->cart_apply(c->dim, prec, u, r, b, t[0], t[1], t[2], t[3], L.n, L.scale, c->stream);
@@ -898,9 +903,13 @@ void pinned_scalars_put(double* p) {
 // Sector matrices of the Cartesian local solver (kernels_patch.cuh): entries
 // from the FP64 part at unit scale, then the table of the MG precision.
 int setup_patch_table(pmg_ctx* c) {
+  double* scratch = (double*)at(c, c->plan.tscratch);
+  if (c->plan.ctable >= 0) {
+    c->ctable = at(c, c->plan.ctable);
+    PMG_CUDA(c->kt[PMG_FP64]->cell_table(c->dim, scratch, c->ctable, c->stream));
+  }
   if (c->plan.table < 0) return PMG_OK;
   c->table = at(c, c->plan.table);
-  double* scratch = (double*)at(c, c->plan.tscratch);
   PatchParamsHost P{};
   P.scale = 1.0;
   P.omega_as = 1.0;

@@ -45,6 +45,7 @@ struct ApplyJob {       // y = A x or y = b - A x (b != nullptr); t: scratch of 
   void* t[4];
   int n;
   double scale;
+  const void* table;  // the cell's table (cell_apply_group)
 };
 struct PatchSolveJob {  // patch smoother of one level (output as patch_cart)
   const void* r;
@@ -140,6 +141,14 @@ struct KernelTable {
   cudaError_t (*patch_entries)(int dim, const PatchParamsHost& H, int n_iter, int prec, const double* dinv,
                                double* scratch, cudaStream_t s);
   cudaError_t (*patch_table)(int dim, int prec, const double* scratch, void* table, cudaStream_t s);
+  // FP64 Cartesian apply as products with the cell's sector matrices (FP64
+  // part): bytes of their table (0: line passes only), its set-up (scratch as
+  // above), y = A x or b - A x; cells: n^d (K+1)^d doubles of scratch
+  int64_t (*cell_table_bytes)(int dim);
+  cudaError_t (*cell_table)(int dim, double* scratch, void* table, cudaStream_t s);
+  cudaError_t (*cell_apply)(int dim, const double* x, double* y, const double* b, double* cells, const void* table,
+                            int n, double scale, cudaStream_t s);
+  cudaError_t (*cell_apply_group)(int dim, int count, const ApplyJob* jobs, cudaStream_t s);
 };
 
 // nullptr when k, dim or prec is out of range

@@ -1,8 +1,8 @@
-"""Cartesian patch smoother as products with the local solver's sector
-matrices: partial batches of patches, the smallest meshes, the fixed-point
+"""Cartesian patch smoother and FP64 apply as products with sector matrices:
+partial batches of patches and cells, the smallest meshes, the fixed-point
 scaling of the FP64 products and values that are not finite.
 
-Tolerances as in test_gpu_parity (FP64 sweep 1e-11, FP32 2e-5).  Scaling the
+Tolerances as in test_gpu_parity (FP64 apply 1e-12, sweep 1e-11, FP32 2e-5).  Scaling the
 right-hand side by a power of two is exact in every step, so those results
 are compared bit for bit."""
 import numpy as np
@@ -16,6 +16,7 @@ import paper_2512_02577_gb300 as p
 from paper_2512_02577_gb300.inputs import random_vector
 from tests.parity import rel
 from tests.test_gpu_defaults_high_degree import _tol, ctx_default
+from oracle import fem
 from tests.test_gpu_parity import full, oracle_level, to_dev
 
 pytestmark = pytest.mark.gpu
@@ -83,3 +84,23 @@ def test_zero_right_hand_side_and_extreme_range():
     ref = torch.zeros_like(b)
     ctx.smooth(to_dev(r * 2.0 ** -1060 * 2.0 ** 900), ref)
     assert np.abs(u.cpu().numpy() * 2.0 ** 900 - ref.cpu().numpy()).max() <= 8 * 2.0 ** (-1074 + 900)
+
+
+# cells: 1, 8, 27 (27 = 16 + 11) in 3D; 1, 16, 25 in 2D; even and odd numbers of nodes per cell
+@pytest.mark.parametrize("d,n,k", [(3, 1, 2), (3, 2, 3), (3, 3, 4), (3, 3, 5), (3, 2, 7), (3, 2, 8), (2, 1, 3), (2, 4, 4),
+                                   (2, 5, 5), (2, 5, 8), (2, 5, 2)])
+def test_fp64_apply_and_residual_match_oracle(d, n, k):
+    ctx = ctx_default(d, n, k, L=1)
+    m = fem.Mesh(d, n, k)
+    A = fem.assemble(m)
+    x, b = random_vector(d, n, k, seed=541), random_vector(d, n, k, seed=542)
+    ref = fem.apply_full(m, A, x)
+    dirty = x + (1.0 - (random_vector(d, n, k, seed=1) != 0)) * 7.0  # boundary entries are ignored
+    y, r = to_dev(np.full_like(x, np.nan)), to_dev(np.full_like(x, np.nan))
+    ctx.apply(to_dev(dirty), y)
+    ctx.residual(to_dev(b), to_dev(dirty), r)
+    assert rel(y, ref) < 1e-12 and rel(r, b - ref) < 1e-12
+    for power in (800, -800):
+        ys = torch.empty_like(y)
+        ctx.apply(to_dev(x * 2.0 ** power), ys)
+        assert torch.equal(ys, y * 2.0 ** power)
