@@ -60,6 +60,7 @@ struct Plan {
   std::vector<LOff> lo;
   int64_t t_mg[4], t64[4], cg[6], scal, partial, dtab64, dtab32, cidx, ainv, a64, gjrow, gjcol, gjbad, cx0, cy0;
   int64_t pbuf = -1, cellbuf = -1, counter = -1;
+  int64_t stage = -1, stage_batches = 0;  // staged patch products: buffers
   int64_t ctable = -1;                // Cartesian: the FP64 operator's cell table
   int64_t table = -1, tscratch = -1;  // Cartesian: sector matrices of the local solver, their set-up's scratch
   int64_t verts = -1;  // distorted: positions of the finest mesh's vertices
@@ -120,6 +121,7 @@ struct pmg_ctx {
   int* cidx = nullptr;
   void* ainv = nullptr;
   bool coarse_ready = false;
+  void* stage = nullptr;    // staged patch products: buffers of plan.stage_batches batches
   void* ctable = nullptr;   // Cartesian: table of the FP64 apply by cells (nullptr: line passes)
   void* table = nullptr;    // Cartesian: sector matrices of the local solver (nullptr: sum-factorised)
   void* pbuf = nullptr;

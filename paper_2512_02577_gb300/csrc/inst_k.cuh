@@ -17,7 +17,7 @@ namespace PMG_KNS {
 constexpr int DP = PMG_DIM;
 // the Cartesian patches of this part are solved by the dense sector products
 // (K = 1: pointwise) instead of sum factorisation
-constexpr bool kDense = K == 1 || PatchDense<DP, TP>::ok();
+constexpr bool kDense = K == 1 || PatchDense<DP, TP>::ok() || kStaged;
 // FP64 operator applies by cells; line passes where they are as fast (2D K = 2:
 // 9 of a tile's 16 rows used, 0.218 against 0.195 ms at 1024^2 cells) and for
 // K = 1 (the 2^d results per cell need more scratch than the passes)
@@ -166,9 +166,10 @@ static DenseJob<T> dense_job(const T* r, T* dst, int n, const PatchParamsHost& H
   int e = 0;
   const bool finite = std::isfinite(c);
   J.cmul = finite ? (unsigned long long)std::ldexp(std::frexp(c, &e), 64) : 0;
-  // the operands are scaled by 2^(1080 - SH - e_patch), the products by 2^-52 (dense_body)
+  // the operands are scaled by 2^(1080 - SH - e_patch), the products by 2^-52 (dense_body); SL digits: 2^8 and
+  // 2^-16 for the eighth
   constexpr int SH = Sectors<DIM, kPatchM>::SPLIT ? DIM + 3 : 3;
-  J.vexp = finite ? e - 64 + 52 - (1080 - SH) : 0;
+  J.vexp = finite ? e - 64 + 52 + 8 * (PatchDense<DIM, double>::SL - 7) - (1080 - SH) : 0;
   J.npatch = (uint32_t)patch_count(DIM, n, H.colour);
   J.d0 = FastDiv(std::max(1, patch_count_1d(n, H.colour, 0)));
   J.d1 = FastDiv(DIM == 3 ? std::max(1, patch_count_1d(n, H.colour, 1)) : 1);
@@ -183,11 +184,28 @@ template <int DIM, typename T>
 static cudaError_t patch_dense_t(const T* r, T* dst, int n, const PatchParamsHost& H, cudaStream_t st) {
   if (patch_count(DIM, n, H.colour) > 0xFFFFFFFFll - 256) return cudaErrorInvalidConfiguration;
   const DenseJob<T> J = dense_job<DIM, T>(r, dst, n, H);
+  if constexpr (kStaged) {
+    using St = Stage<DIM>;
+    const int64_t batches = (J.npatch + St::P - 1) / St::P;
+    if (H.stage_batches < 1) return cudaErrorInvalidValue;
+    long long* X = (long long*)H.stage;
+    long long* Y = X + H.stage_batches * St::XWORDS;
+    int* words = (int*)(Y + H.stage_batches * St::YWORDS);
+    for (int64_t first = 0; first < batches; first += H.stage_batches) {
+      const unsigned nb = (unsigned)std::min<int64_t>(H.stage_batches, batches - first);
+      patch_split_kernel<DIM><<<nb, 256, 0, st>>>(J, (uint32_t)first, X, words);
+      patch_product_kernel<DIM><<<dim3(nb, St::S::NS), 256, St::XSM + St::YSM, st>>>(J.table, X, Y);
+      patch_merge_kernel<DIM><<<dim3(nb, St::S::E), 128, St::ZSM, st>>>(J, (uint32_t)first, Y, words);
+      g_launches += 3;
+    }
+    return cudaGetLastError();
+  } else {
   const unsigned grid = (J.npatch + dense_batch<DIM, T>() - 1) / dense_batch<DIM, T>();
   if constexpr (K == 1) patch_point_kernel<DIM, T><<<grid, 256, 0, st>>>(J);
   else patch_dense_kernel<DIM, T><<<grid, 32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::SMEM, st>>>(J);
   g_launches += 1;
   return cudaGetLastError();
+  }
 }
 
 template <int DIM, typename T>
@@ -443,7 +461,14 @@ static cudaError_t cart_apply_ff_group(int dim, int count, const ApplyJob* jobs,
 template <int DIM, typename T>
 static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int ppc, int n_iter, const T* dinv,
                                       int* counter, cudaStream_t st) {
-  if constexpr (kDense) {
+  if constexpr (kStaged) {  // each job in its own stage buffers
+    for (int j = 0; j < count; ++j) {
+      if (patch_count(DIM, jobs[j].n, jobs[j].P.colour) == 0) continue;
+      cudaError_t e = patch_dense_t<DIM, T>((const T*)jobs[j].r, (T*)jobs[j].dst, jobs[j].n, jobs[j].P, st);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  } else if constexpr (kDense) {
     GroupOf<DenseJob<T>> G;
     G.count = 0;
     G.start[0] = 0;
@@ -581,6 +606,22 @@ static cudaError_t patch_table_t(const double* scratch, void* table, cudaStream_
   }
   return cudaErrorInvalidValue;
 }
+
+// bytes of the stage buffers for `batches` batches of patches, and the batches
+// they are to hold for a level of n cells (0: not a staged part)
+template <int DIM>
+static int64_t stage_bytes_t(int64_t batches) {
+  if constexpr (kStaged) return batches * Stage<DIM>::BYTES;
+  return 0;
+}
+template <int DIM>
+static int64_t stage_batches_t(int n) {
+  if constexpr (kStaged)
+    return std::min<int64_t>(kStageBatches, (patch_count(DIM, n, -1) + Stage<DIM>::P - 1) / Stage<DIM>::P);
+  return 0;
+}
+static int64_t patch_stage_bytes(int64_t batches) { return stage_bytes_t<DP>(batches); }
+static int64_t patch_stage_batches(int n) { return stage_batches_t<DP>(n); }
 
 // ---------------------------------------------------------------- FP64 apply by cells
 static int64_t cell_table_bytes(int dim) { return dim == DP && kCellDense ? CellDense<DP>::TABLE_BYTES : 0; }
@@ -853,6 +894,9 @@ static void prepare_cart(int optin, const Acc& acc) {
     acc(allow_smem(patch_cart_kernel<DIM, T>, optin));
     acc(allow_smem(patch_cart_group_kernel<DIM, T>, optin));
     if (patch_il<DIM, T>() > 0) acc(allow_smem(patch_cart_il_kernel<DIM, T>, optin));
+  } else if constexpr (kStaged) {
+    acc(allow_smem(patch_product_kernel<DIM>, optin));
+    acc(allow_smem(patch_merge_kernel<DIM>, optin));
   } else if constexpr (K > 1) {
     acc(allow_smem(patch_dense_kernel<DIM, T>, optin));
     acc(allow_smem(patch_dense_group_kernel<DIM, T>, optin));
@@ -920,6 +964,8 @@ const KernelTable* PMG_TABLE_FN() {
       PMG_KNS::patch_scratch_bytes,
       PMG_KNS::patch_entries,
       PMG_KNS::patch_table,
+      PMG_KNS::patch_stage_bytes,
+      PMG_KNS::patch_stage_batches,
       PMG_KNS::cell_table_bytes,
       PMG_KNS::cell_table,
       PMG_KNS::cell_apply,

@@ -17,14 +17,15 @@
 // shared-memory traffic and the barriers between the line passes.
 //
 // FP64 arithmetic: operands in fixed point (one exponent per matrix row and per
-// patch), split into 7 signed digits of 8 bits that are exact in FP16;
+// patch), split into 7 or 8 signed digits of 8 bits that are exact in FP16;
 // products of digits are summed exactly by the tensor cores (integers in the
-// FP32 accumulator) and across digit pairs in 64-bit integers, keeping the 34
-// digit pairs i + j <= 7 (0-based; without i + j = 7 the error is 100 times
+// FP32 accumulator) and across digit pairs in 64-bit integers, keeping the 34 or
+// 36 digit pairs i + j <= 7 (0-based; without i + j = 7 the error is 100 times
 // larger).  No FP64 instruction is executed.  Error of one local solve
 // against extended precision, N(0,1) residuals, before (sum factorisation)
 // and now: K = 3 3.3e-16, 3.3e-16; K = 4 3.9e-16, 3.7e-16; K = 5 3.6e-16,
-// 3.7e-16; 2D K = 7 4.1e-16, 3.1e-16.  FP32: three BF16 parts of each value
+// 3.7e-16; 2D K = 7 4.1e-16, 2.5e-16;
+// K = 6 5.4e-16, 5.4e-16; K = 7 6.3e-16, 6.1e-16.  FP32: three BF16 parts of each value
 // (8 bits each, exact), the six products of weight 2^-16 and above.
 //
 // Patch launch of one sweep, before and now (GB300): FP64 K = 4 at 32^3 cells
@@ -188,7 +189,11 @@ template <int DIM, int M, typename T>
 struct Dense {
   using S = Sectors<DIM, M>;
   static constexpr bool F64 = sizeof(T) == 8;
-  static constexpr int SL = F64 ? 7 : 3;                        // parts per value
+  // parts per value.  FP64: an eighth digit for the large matrices (M = 13,
+  // 15), whose rows hold many entries far below their largest: K = 7 in 3D
+  // has an error of 8.1e-16 with seven digits, above sum factorisation's 6.3e-16
+  static constexpr int SL = F64 ? (M > 11 ? 8 : 7) : 3;
+  static constexpr unsigned long long BIAS = 0x8080808080808080ull >> (F64 ? 64 - 8 * SL : 0);  // digits + 128
   static constexpr int P = 16;
   static constexpr int NT = P / 8;                              // 8-column tiles
   static constexpr int NSUB = 32 / P;                           // lines a warp handles at once
@@ -281,6 +286,40 @@ __device__ __forceinline__ long long fixed_of(double v, int e) {
   return (x ^ sg) - sg;
 }
 
+// Scale of a patch's (or cell's) values for the fixed point: mx the largest
+// high word, with its low bit set where only a low word is not zero.  The
+// bound e leaves 0.8% to the top digit's range; subnormal windows are scaled
+// by 2^100 and bounded by the high word's leading bit.
+struct PatchScale {
+  int e;
+  bool bad;  // an infinity or NaN, or a matrix that is not finite
+  bool tiny, any_tiny;
+  __device__ __forceinline__ PatchScale() {}
+  __device__ __forceinline__ PatchScale(unsigned mx, bool broken) {
+    bad = mx >= 0x7FF00000u || broken;
+    tiny = mx < 0x00100000u;
+    any_tiny = __any_sync(0xffffffffu, tiny && mx != 0);  // the FP64 products with 2^100 only where needed
+    tiny = tiny && any_tiny;
+    e = tiny ? 113 - __clz((int)mx) : max((int)((mx + 0x4000u) >> 20), 1);
+  }
+  template <int M>
+  __device__ __forceinline__ void fixed(double (&r)[M], long long (&v)[M]) const {
+    if (any_tiny) {
+#pragma unroll
+      for (int i = 0; i < M; ++i) r[i] = tiny ? r[i] * 0x1p100 : r[i];
+    }
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = fixed_of(r[i], e);
+  }
+};
+
+// an even / odd combination (of 55 + sh bits) as operand of SL digits
+template <int SL>
+__device__ __forceinline__ long long operand_of(long long v, int sh) {
+  if constexpr (SL == 8) return (long long)((unsigned long long)v << (8 - sh));
+  else return (v + (1ll << (sh - 1))) >> sh;
+}
+
 // y cmul 2^(ve + 64) rounded to nearest (ties away), in integer arithmetic
 __device__ __forceinline__ double double_of(long long y, unsigned long long cmul, int ve) {
   const unsigned long long sg = (unsigned long long)(y >> 63);
@@ -329,15 +368,16 @@ constexpr int kMagicBits = 0x4B400000;
 
 // FP64 products of one unit: result rows of sector coefficients times the
 // operand rows, in units of 2^-52 of (table integer x operand integer) at the
-// exponent of the row's class.  Two k tiles add at most 14 products of 2^18 to an
-// accumulator (below its exact range of 2^22 around kMagic) before it is
+// exponent of the row's class.  Two k tiles add at most 16 products of 2^18 to an
+// accumulator (within its exact range of 2^22 around kMagic) before it is
 // emptied into Y.
 template <class D>
-__device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table, const long long* X,
-                                          long long* Y, int lane) {
-  constexpr int SL = D::SL, NT = D::NT, ND = SL + 1;  // ND: digit sums kept, i + j < ND
+__device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table,
+                                          const int* __restrict__ shifts, const long long* X, long long* Y,
+                                          int lane) {
+  constexpr int SL = D::SL, NT = D::NT, ND = 8;  // ND: digit sums kept, i + j < ND
   const int g = lane >> 2, q = lane & 3;
-  const int* shift = reinterpret_cast<const int*>(table + D::FRAGS) + u.row + g;  // row exponent - its class's
+  const int* shift = shifts + u.row + g;  // row exponent - its class's
   const uint4* tp = table + (int64_t)u.frag * 32 + lane;
   const long long* xp = X + (u.prow + 2 * q) * D::XP + g;
   for (int k0 = 0; k0 < u.kt; k0 += 2) {
@@ -358,7 +398,7 @@ __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __res
         for (int h = 0; h < 2; ++h) {
           const long long* x = xp + (16 * k + 8 * h) * D::XP + 8 * t;
           // biased so that byte SL - 1 - j holds digit j + 128
-          const long long w0 = x[0] + 0x0080808080808080ll, w1 = x[D::XP] + 0x0080808080808080ll;
+          const unsigned long long w0 = (unsigned long long)x[0] + D::BIAS, w1 = (unsigned long long)x[D::XP] + D::BIAS;
 #pragma unroll
           for (int j = 0; j < SL; ++j) {
             const int byte = SL - 1 - j, bb = byte & 3;
@@ -530,9 +570,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
         }
     }
   }
-  int e = 0;         // FP64: biased exponent bound of the patch's values
-  bool bad = false;  // FP64: an infinity or NaN among them
-  bool tiny = false, any_tiny = false;
+  PatchScale sc;  // FP64
   const int* classexp = reinterpret_cast<const int*>(J.table + D::FRAGS) + S::ROWS;
   if constexpr (D::F64) {
     __syncthreads();  // s_max
@@ -558,14 +596,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     for (int o = P; o < 32; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane < P) atomicMax(&s_max[pn], mx);
     __syncthreads();
-    mx = s_max[pn];
-    bad = mx >= 0x7FF00000u || J.cmul == 0 || classexp[0] == kNoExp;
-    // the bound leaves 0.8% to the top digit's range; subnormal patches are
-    // scaled by 2^100 and bounded by the high word's leading bit
-    tiny = mx < 0x00100000u;
-    any_tiny = __any_sync(0xffffffffu, tiny && mx != 0);  // the products with 2^100 only where needed
-    tiny = tiny && any_tiny;
-    e = tiny ? 113 - __clz((int)mx) : max((int)((mx + 0x4000u) >> 20), 1);
+    sc = PatchScale(s_max[pn], J.cmul == 0 || classexp[0] == kNoExp);
   }
   // even / odd combinations, stored as operands
   for (int l = item0; l < L::N; l += STEP) {
@@ -579,12 +610,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
         double r[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) r[i] = ln.has(b) || !S::SPLIT ? q[i * P] : 0.0;
-        if (any_tiny) {
-#pragma unroll
-          for (int i = 0; i < M; ++i) r[i] = tiny ? r[i] * 0x1p100 : r[i];
-        }
-#pragma unroll
-        for (int i = 0; i < M; ++i) v[b][i] = fixed_of(r[i], e);
+        sc.template fixed<M>(r, v[b]);
       }
       reflect<DIM, M>(v);
       const int sh0 = (S::SPLIT ? DIM + 3 : 3) - ln.centres();  // to 55 bits and sign: 2^(d-c) images were summed
@@ -592,8 +618,8 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
       for (int b = 0; b < L::IMAGES; ++b)
         if (ln.has(b) || !S::SPLIT)
           for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
-            const int sh = S::CENTRE && i == S::E - 1 ? sh0 - 1 : sh0;
-            X[(S::prow(s) + ox + ln.coef(s)) * D::XP + pn] = (v[b][i] + (1ll << (sh - 1))) >> sh;
+            X[(S::prow(s) + ox + ln.coef(s)) * D::XP + pn] =
+                operand_of<D::SL>(v[b][i], S::CENTRE && i == S::E - 1 ? sh0 - 1 : sh0);
           });
     } else {
       float v[L::IMAGES][S::M];
@@ -624,7 +650,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
   if constexpr (D::F64) {
     for (int u = warp; u < D::UNITS; u += NW) {
 #if PMG_PREC == 0
-      dense_mma<D>(CELL ? c_cell_units.u[CELL ? u : 0] : c_units.u[CELL ? 0 : u], J.table, X, Y, lane);
+      dense_mma<D>(CELL ? c_cell_units.u[CELL ? u : 0] : c_units.u[CELL ? 0 : u], J.table, classexp - S::ROWS, X, Y, lane);
 #endif
     }
   } else {
@@ -665,12 +691,12 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     for (int b = 0; b < L::IMAGES; ++b)
       if (ln.has(b) || !S::SPLIT) {
         T* z = Z + pn * D::ZP + ln.node(b, S::M);
-        const int ve = J.vexp + e - (tiny ? 100 : 0), nc = ln.centres();
+        const int ve = D::F64 ? J.vexp + sc.e - (sc.tiny ? 100 : 0) : 0, nc = ln.centres();
         const int ve0 = D::F64 ? ve - __ldg(classexp + nc) : 0, ve1 = D::F64 ? ve - __ldg(classexp + nc + 1) : 0;
 #pragma unroll
         for (int i = 0; i < S::M; ++i) {
           if constexpr (D::F64)
-            z[i] = bad ? __longlong_as_double(0x7FF8000000000000ll) : double_of(v[b][i], J.cmul, S::CENTRE && i == S::E - 1 ? ve1 : ve0);
+            z[i] = sc.bad ? __longlong_as_double(0x7FF8000000000000ll) : double_of(v[b][i], J.cmul, S::CENTRE && i == S::E - 1 ? ve1 : ve0);
           else
             z[i] = J.c * v[b][i];
         }
@@ -827,6 +853,198 @@ __global__ void __launch_bounds__(256) cell_sum_group_kernel(const __grid_consta
   cell_sum<DIM>(G.job[j], t - G.start[j]);
 }
 
+// ---------------------------------------------------------------- staged products
+// FP64 patches of K = 6, 7 in 3D: the operands of 16 patches (180-290 KB) do
+// not fit an SM, so the steps of dense_body run as three launches over a chunk
+// of batches, whose operands and results (kStageBatches x 0.35-0.57 MB) stay
+// in L2: patch_split (gather to fixed point, even / odd combinations), one
+// block per batch and sector for the products, patch_merge (back to the
+// nodes), one block per batch and pair of mirrored z planes.  Patch
+// launch, sum factorisation before and now: K = 7 at 28^3 cells 11.8 and 3.65
+// ms, at 12^3 1.02 and 0.35, at 4^3 0.123 and 0.106; K = 6 at 32^3 9.80 and
+// 2.76 ms (the matrix, 4-10 MB, is streamed from L2 for every 16 patches).
+constexpr bool kStaged = PMG_PREC == 0 && PMG_DIM == 3 && (K == 6 || K == 7);
+constexpr int kStageBatches = 76;  // 8 sectors each: two waves of two blocks per SM
+
+template <int DIM>
+struct Stage {
+  using D = Dense<DIM, kPatchM, double>;
+  using S = Sectors<DIM, kPatchM>;
+  static constexpr int P = D::P;
+  static constexpr int64_t XWORDS = (int64_t)S::ROWS * P, YWORDS = XWORDS;  // per batch
+  static constexpr int64_t BYTES = 8 * (XWORDS + YWORDS) + 4 * P;          // and the patches' exponents
+  static constexpr int MAXT = S::tiles(0);
+  static constexpr int XSM = 16 * MAXT * D::XP * 8, YSM = S::size(0) * P * 8;  // products: one sector
+  static constexpr int MP2 = kPatchM * kPatchM, ZP = (2 * MP2) | 1, ZSM = P * ZP * 8;  // merge: two planes
+};
+
+// exponent word of a patch: bits 0-11 the exponent bound, 12 tiny, 13 bad
+struct PatchOrigin {
+  int64_t base;
+  int colour;
+  bool active;
+};
+template <int DIM>
+__device__ __forceinline__ PatchOrigin patch_origin(const DenseJob<double>& J, uint32_t pid) {
+  const int N1 = K * J.n + 1;
+  PatchOrigin o;
+  o.active = pid < J.npatch;
+  const uint32_t t = o.active ? pid : 0, r1 = J.d0.div(t), r2 = J.d1.div(r1);
+  const int i[3] = {(int)(t - r1 * J.d0.d), (int)(r1 - r2 * J.d1.d), (int)r2};
+  int v[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) v[d] = J.colour < 0 ? i[d] + 1 : 2 * i[d] + (((J.colour >> d) & 1) ? 1 : 2);
+  o.base = (int64_t)(K * (v[0] - 1) + 1) + (int64_t)N1 * ((K * (v[1] - 1) + 1) + (int64_t)N1 * (K * (v[2] - 1) + 1));
+  o.colour = J.colour < 0 ? (v[0] & 1) | ((v[1] & 1) << 1) | ((v[2] & 1) << 2) : 0;
+  return o;
+}
+
+// X [row][P] and the exponent words of batch first + blockIdx.x
+template <int DIM>
+__global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant__ DenseJob<double> J, uint32_t first,
+                                                          long long* __restrict__ X, int* __restrict__ words) {
+  constexpr int M = kPatchM;
+  using S = Sectors<DIM, M>;
+  using L = Lines<DIM, M>;
+  constexpr int P = Stage<DIM>::P;
+  __shared__ unsigned s_max[P];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pn = lane % P, item0 = warp * (32 / P) + lane / P;
+  constexpr int STEP = 8 * (32 / P);
+  const int N1 = K * J.n + 1;
+  const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + pn);
+  const double* rp = J.r + o.base;
+  const int* classexp = reinterpret_cast<const int*>(J.table + Stage<DIM>::D::FRAGS) + S::ROWS;
+  X += blockIdx.x * Stage<DIM>::XWORDS;
+  if (threadIdx.x < P) s_max[threadIdx.x] = 0;
+  __syncthreads();
+  unsigned mx = 0;
+  for (int l = item0; l < M * M; l += STEP) {
+    const double* q = rp + N1 * (l % M + N1 * (l / M));
+    double v[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = o.active ? q[i] : 0.0;
+#pragma unroll
+    for (int i = 0; i < M; ++i)
+      mx = max(mx, ((unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu) | (__double2loint(v[i]) != 0));
+  }
+#pragma unroll
+  for (int w = P; w < 32; w <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+  if (lane < P) atomicMax(&s_max[pn], mx);
+  __syncthreads();
+  mx = s_max[pn];
+  const PatchScale sc(mx, J.cmul == 0 || classexp[0] == kNoExp);
+  if (threadIdx.x < P) words[blockIdx.x * P + pn] = sc.e | (sc.tiny ? 1 << 12 : 0) | (sc.bad ? 1 << 13 : 0);
+  for (int l = item0; l < L::N; l += STEP) {
+    const L ln(l);
+    long long v[L::IMAGES][M];
+#pragma unroll
+    for (int b = 0; b < L::IMAGES; ++b) {
+      const double* q = rp + ln.node(b, N1);
+      const bool in = o.active && ln.has(b);
+      double r[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) r[i] = in ? q[i] : 0.0;
+      sc.template fixed<M>(r, v[b]);
+    }
+    reflect<DIM, M>(v);
+    const int sh0 = DIM + 3 - ln.centres();
+#pragma unroll
+    for (int b = 0; b < L::IMAGES; ++b)
+      if (ln.has(b))
+        for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
+          X[(S::row(s) + ox + ln.coef(s)) * P + pn] =
+              operand_of<Stage<DIM>::D::SL>(v[b][i], S::CENTRE && i == S::E - 1 ? sh0 - 1 : sh0);
+        });
+  }
+}
+
+// products of sector blockIdx.y for batch blockIdx.x
+template <int DIM>
+__global__ void __launch_bounds__(256, 2) patch_product_kernel(const uint4* __restrict__ table,
+                                                               const long long* __restrict__ X,
+                                                               long long* __restrict__ Y) {
+  using St = Stage<DIM>;
+  using D = typename St::D;
+  using S = typename St::S;
+  constexpr int P = St::P;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  long long* xs = reinterpret_cast<long long*>(smraw);
+  long long* ys = reinterpret_cast<long long*>(smraw + St::XSM);
+  const int s = blockIdx.y, size = S::size(s), tiles = S::tiles(s), row = S::row(s);
+  const long long* x = X + blockIdx.x * St::XWORDS + (int64_t)row * P;
+  for (int i = threadIdx.x; i < 16 * tiles * P; i += 256)
+    xs[i / P * D::XP + i % P] = i < size * P ? x[i] : 0;
+  __syncthreads();
+  const int* shifts = reinterpret_cast<const int*>(table + D::FRAGS) + row;
+  for (int m = threadIdx.x >> 5; m < tiles; m += 8) {
+    DenseUnit u;
+    u.prow = 0;
+    u.kt = (short)tiles;
+    u.row = (short)(16 * m);
+    u.valid = (short)min(16, size - 16 * m);
+    u.frag = (S::tile(s) + m * tiles) * D::SL;
+    dense_mma<D>(u, table, shifts, xs, ys, threadIdx.x & 31);
+  }
+  __syncthreads();
+  long long* y = Y + blockIdx.x * St::YWORDS + (int64_t)row * P;
+  for (int i = threadIdx.x; i < size * P; i += 256) y[i] = ys[i];
+}
+
+// nodes of the planes z = blockIdx.y and its mirror image, batch first + blockIdx.x
+template <int DIM>
+__global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant__ DenseJob<double> J, uint32_t first,
+                                                          const long long* __restrict__ Y,
+                                                          const int* __restrict__ words) {
+  constexpr int M = kPatchM;
+  using St = Stage<DIM>;
+  using S = typename St::S;
+  using L = Lines<DIM, M>;
+  constexpr int P = St::P, MP2 = St::MP2, ZP = St::ZP;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  double* Z = reinterpret_cast<double*>(smraw);
+  const int pn = threadIdx.x % P, cz = blockIdx.y;
+  const int N1 = K * J.n + 1;
+  const int* classexp = reinterpret_cast<const int*>(J.table + St::D::FRAGS) + S::ROWS;
+  const int word = words[blockIdx.x * P + pn];
+  const int ve = J.vexp + (word & 0xFFF) - (word & (1 << 12) ? 100 : 0);
+  Y += blockIdx.x * St::YWORDS;
+  for (int cy = threadIdx.x / P; cy < S::E; cy += 128 / P) {
+    const L ln(cy + S::E * cz);
+    long long v[L::IMAGES][M];
+#pragma unroll
+    for (int b = 0; b < L::IMAGES; ++b) {
+      const bool in = ln.has(b);
+      for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
+        v[b][i] = in ? __ldg(Y + (S::row(s) + ox + ln.coef(s)) * P + pn) : 0ll;
+      });
+    }
+    reflect<DIM, M>(v);
+    const int nc = ln.centres(), ve0 = ve - __ldg(classexp + nc), ve1 = ve - __ldg(classexp + nc + 1);
+#pragma unroll
+    for (int b = 0; b < L::IMAGES; ++b)
+      if (ln.has(b)) {
+        double* z = Z + pn * ZP + (b >> 1) * MP2 + M * ((b & 1) ? M - 1 - cy : cy);
+#pragma unroll
+        for (int i = 0; i < M; ++i)
+          z[i] = word & (1 << 13) ? __longlong_as_double(0x7FF8000000000000ll)
+                                  : double_of(v[b][i], J.cmul, S::CENTRE && i == S::E - 1 ? ve1 : ve0);
+      }
+  }
+  __syncthreads();
+  const int64_t N = (int64_t)N1 * N1 * N1;
+  const int planes = cz == S::E - 1 ? 1 : 2;
+  for (int gp = threadIdx.x >> 5; gp < P; gp += 4) {
+    const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + gp);
+    if (!o.active) break;
+    for (int i = threadIdx.x & 31; i < planes * MP2; i += 32) {
+      const int pl = i >= MP2, r = (i - pl * MP2) / M, ix = i - pl * MP2 - r * M, iz = pl ? M - 1 - cz : cz;
+      double* d = J.dst + (J.colour < 0 ? o.colour * N : 0) + o.base + ix + N1 * (r + N1 * iz);
+      if (J.colour < 0) *d = Z[gp * ZP + i];
+      else *d += Z[gp * ZP + i];  // one patch of the colour per node
+    }
+  }
+}
+
 // K = 1: the patch is its vertex, the local solve one multiplication by
 // c = omega_AS / A_{j,1} (additive) or 1 / A_{j,1}.
 template <int DIM, typename T>
@@ -913,7 +1131,7 @@ __device__ __forceinline__ Orbit<DIM, M> orbit_of(int s, int k) {
 // block), in pairs of doubles.
 // rowexp: the largest exponent x with entry 2^x below 0.98 2^55 (7 signed
 // digits reach 127/128 of 2^55) and the row's sum of magnitudes times 2^x
-// below 2^57 (results and their even / odd sums stay within 64 bits).  The
+// below 2^57 (8 digits: 2^63, 2^65; results and their even / odd sums stay within 64 bits).  The
 // sectors' results for one orbit are summed, so they need a common exponent:
 // minexp, the least one of the rows of a class -- the nodes with the same
 // number of central coordinates, whose coefficients have the same size
@@ -977,10 +1195,11 @@ __global__ void __launch_bounds__(128) sector_entries_kernel(const double* __res
     sum += __shfl_xor_sync(0xffffffffu, sum, o);
   }
   if (lane) return;
+  constexpr int SL = Dense<DIM, M, double>::SL;
   int te = 0, se = 0;
   if (frexp(top, &te) > 0.98) ++te;
   frexp(sum, &se);
-  const int x = sum == 0.0 ? 1000 : min(55 - te, 57 - se);
+  const int x = sum == 0.0 ? 1000 : min(8 * SL - 1 - te, 8 * SL + 1 - se);
   rowexp[row] = x;
   atomicMin(minexp + om.centres(), x);
   if (!isfinite(sum)) atomicMin(minexp, kNoExp);
@@ -1020,7 +1239,7 @@ __global__ void __launch_bounds__(256) sector_table_kernel(const double* __restr
     const int k = k0 + h;
     const double a = m < sz && k < sz ? entries[S::entry(s) + (int64_t)m * sz + k] : 0.0;
     if constexpr (sizeof(T) == 8) {
-      const long long v = __double2ll_rn(scalbn(a, re)) + 0x0080808080808080ll;
+      const unsigned long long v = (unsigned long long)__double2ll_rn(scalbn(a, re)) + D::BIAS;
       for (int i = 0; i < SL; ++i) {
         const int digit = (int)((v >> (8 * (SL - 1 - i))) & 0xFF) - 128;
         part[i] |= (uint32_t)__half_as_ushort(__int2half_rn(digit)) << (16 * h);

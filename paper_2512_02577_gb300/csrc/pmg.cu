@@ -221,7 +221,12 @@ int make_plan(const pmg_config* cfg, Plan& P) {
     const int64_t tb = kernel_table(P.K, P.dim, cfg->mg_precision)->patch_table_bytes(P.dim, cfg->mg_precision);
     const KernelTable* k64 = kernel_table(P.K, P.dim, PMG_FP64);
     const int64_t cb = k64->cell_table_bytes(P.dim);
-    if (tb > 0) P.table = bump(cur, tb);
+    if (tb > 0) {
+      P.table = bump(cur, tb);
+      const KernelTable* km = kernel_table(P.K, P.dim, cfg->mg_precision);
+      P.stage_batches = km->patch_stage_batches(cfg->n_cells);
+      if (P.stage_batches > 0) P.stage = bump(cur, km->patch_stage_bytes(P.stage_batches));
+    }
     if (cb > 0) P.ctable = bump(cur, cb);
     if (tb > 0 || cb > 0) P.tscratch = bump(cur, k64->patch_scratch_bytes(P.dim));
   }
@@ -249,6 +254,8 @@ PatchParamsHost patch_params(const pmg_ctx* c, int level) {
   P.half = c->cfg.local_half;
   P.colour = -1;
   P.table = c->table;
+  P.stage = c->stage;
+  P.stage_batches = c->plan.stage_batches;
   return P;
 }
 }  // namespace pmg
@@ -910,6 +917,7 @@ int setup_patch_table(pmg_ctx* c) {
   }
   if (c->plan.table < 0) return PMG_OK;
   c->table = at(c, c->plan.table);
+  c->stage = at(c, c->plan.stage);
   PatchParamsHost P{};
   P.scale = 1.0;
   P.omega_as = 1.0;

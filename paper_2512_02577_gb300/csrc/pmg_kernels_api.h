@@ -25,6 +25,8 @@ struct PatchParamsHost {
                      // vector); c >= 0: only the patches of parity colour c,
                      // u += d_j added straight into dst (multiplicative sweep)
   const void* table;  // Cartesian: the sector matrices of the local solver (patch_table)
+  void* stage;        // staged parts: buffers for stage_batches batches of patches
+  int64_t stage_batches;
 };
 
 // Deformed-geometry arrays of one mesh level (device pointers).
@@ -141,6 +143,10 @@ struct KernelTable {
   cudaError_t (*patch_entries)(int dim, const PatchParamsHost& H, int n_iter, int prec, const double* dinv,
                                double* scratch, cudaStream_t s);
   cudaError_t (*patch_table)(int dim, int prec, const double* scratch, void* table, cudaStream_t s);
+  // staged parts (FP64 K = 6, 7 in 3D): bytes of the buffers for a number of
+  // batches, the batches to provide for a finest level of n cells (else 0)
+  int64_t (*patch_stage_bytes)(int64_t batches);
+  int64_t (*patch_stage_batches)(int n);
   // FP64 Cartesian apply as products with the cell's sector matrices (FP64
   // part): bytes of their table (0: line passes only), its set-up (scratch as
   // above), y = A x or b - A x; cells: n^d (K+1)^d doubles of scratch

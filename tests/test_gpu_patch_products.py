@@ -23,7 +23,8 @@ pytestmark = pytest.mark.gpu
 
 
 # patches: 1, 8, 27 in 3D; 1, 16, 17^2 = 18 * 16 + 1 in 2D
-@pytest.mark.parametrize("d,n,k", [(3, 2, 1), (3, 2, 2), (3, 3, 3), (3, 2, 5), (3, 4, 5), (3, 2, 4), (2, 2, 8),
+@pytest.mark.parametrize("d,n,k", [(3, 2, 1), (3, 2, 2), (3, 3, 3), (3, 2, 5), (3, 4, 5), (3, 2, 4), (3, 2, 6),
+                                   (3, 3, 7), (3, 4, 6), (2, 2, 8),
                                    (2, 5, 8), (2, 18, 2), (2, 18, 3), (2, 5, 4), (2, 5, 7), (2, 3, 1)])
 @pytest.mark.parametrize("prec", [p.FP64, p.FP32])
 @pytest.mark.parametrize("smoother", [p.ADDITIVE, p.MULTIPLICATIVE])
@@ -104,3 +105,25 @@ def test_fp64_apply_and_residual_match_oracle(d, n, k):
         ys = torch.empty_like(y)
         ctx.apply(to_dev(x * 2.0 ** power), ys)
         assert torch.equal(ys, y * 2.0 ** power)
+
+
+@pytest.mark.parametrize("k,prec", [(6, p.FP64), (7, p.FP64), (5, p.FP64), (6, p.FP32)])
+def test_corrections_do_not_depend_on_the_batch(k, prec):
+    # 11^3 = 1331 patches: more than one chunk of batches of the staged
+    # products; the same values 8 cells further along z (the same parity
+    # colours, so the same order of the sum per node) give the same correction
+    d, n = 3, 12
+    dt = torch.float64 if prec == p.FP64 else torch.float32
+    ctx = ctx_default(d, n, k, L=1, prec=prec)
+    N1 = k * n + 1
+    gen = torch.Generator().manual_seed(551)
+    patch = torch.randn((2 * k, 3 * k, 4 * k), generator=gen, dtype=torch.float64).to("cuda:0", dt)
+    us = []
+    for z in (1, 9):
+        b = torch.zeros((N1, N1, N1), dtype=dt, device="cuda:0")
+        b[k * z:k * (z + 2), 3 * k:6 * k, 4 * k:8 * k] = patch
+        u = torch.zeros_like(b)
+        ctx.smooth(b.reshape(-1), u.reshape(-1))
+        us.append(u[k * (z - 1):k * (z + 3)].clone())
+        assert torch.isfinite(u).all()
+    assert us[0].any() and torch.equal(us[0], us[1])
