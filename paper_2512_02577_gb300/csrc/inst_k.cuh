@@ -308,37 +308,45 @@ static cudaError_t patch_gather(int dim, int prec, const void* dst, void* u, int
   return patch_gather_t<DP, TP>((const TP*)dst, (TP*)u, n, add, s);
 }
 
+// one pass of a transfer; ex, ey, ez: extents of its output
+template <int AX, bool ADD, typename T>
+static void prolong_pass(const T* in, T* out, int nc, int ex, int ey, int ez, cudaStream_t st) {
+  hprolong_pass<AX, ADD, T><<<grid_for(transfer_items<AX>(nc, ex, ey, ez), 256), 256, 0, st>>>(
+      in, out, nc, ex, ey, ez, FastDiv(ex), FastDiv(ey), FastDiv(nc + 1));
+}
+template <int AX, typename T>
+static void restrict_pass(const T* in, T* out, int nc, int ex, int ey, int ez, cudaStream_t st) {
+  hrestrict_pass<AX, T><<<grid_for(transfer_items<AX>(nc, ex, ey, ez), 256), 256, 0, st>>>(
+      in, out, nc, ex, ey, ez, FastDiv(ex), FastDiv(ey), FastDiv(nc + 1));
+}
+
 template <int DIM, typename T>
 static cudaError_t h_prolong_t(const T* uc, T* uf, T* t0, T* t1, int nc, cudaStream_t st) {
   const int c1 = K * nc + 1, f1 = 2 * K * nc + 1;
-  const int bs = 256;
   if (DIM == 3) {
-    hprolong_pass<0, false, T><<<grid_for((int64_t)f1 * c1 * c1, bs), bs, 0, st>>>(uc, t0, nc, f1, c1, c1, FastDiv(f1), FastDiv(c1));
-    hprolong_pass<1, false, T><<<grid_for((int64_t)f1 * f1 * c1, bs), bs, 0, st>>>(t0, t1, nc, f1, f1, c1, FastDiv(f1), FastDiv(f1));
-    hprolong_pass<2, true, T><<<grid_for((int64_t)f1 * f1 * f1, bs), bs, 0, st>>>(t1, uf, nc, f1, f1, f1, FastDiv(f1), FastDiv(f1));
-    g_launches += 3;
+    prolong_pass<0, false, T>(uc, t0, nc, f1, c1, c1, st);
+    prolong_pass<1, false, T>(t0, t1, nc, f1, f1, c1, st);
+    prolong_pass<2, true, T>(t1, uf, nc, f1, f1, f1, st);
   } else {
-    hprolong_pass<0, false, T><<<grid_for((int64_t)f1 * c1, bs), bs, 0, st>>>(uc, t0, nc, f1, c1, 1, FastDiv(f1), FastDiv(c1));
-    hprolong_pass<1, true, T><<<grid_for((int64_t)f1 * f1, bs), bs, 0, st>>>(t0, uf, nc, f1, f1, 1, FastDiv(f1), FastDiv(f1));
-    g_launches += 2;
+    prolong_pass<0, false, T>(uc, t0, nc, f1, c1, 1, st);
+    prolong_pass<1, true, T>(t0, uf, nc, f1, f1, 1, st);
   }
+  g_launches += DIM;
   return cudaGetLastError();
 }
 
 template <int DIM, typename T>
 static cudaError_t h_restrict_t(const T* rf, T* rc, T* t0, T* t1, int nc, cudaStream_t st) {
   const int c1 = K * nc + 1, f1 = 2 * K * nc + 1;
-  const int bs = 256;
   if (DIM == 3) {
-    hrestrict_pass<2, T><<<grid_for((int64_t)f1 * f1 * c1, bs), bs, 0, st>>>(rf, t0, nc, f1, f1, c1, FastDiv(f1), FastDiv(f1));
-    hrestrict_pass<1, T><<<grid_for((int64_t)f1 * c1 * c1, bs), bs, 0, st>>>(t0, t1, nc, f1, c1, c1, FastDiv(f1), FastDiv(c1));
-    hrestrict_pass<0, T><<<grid_for((int64_t)c1 * c1 * c1, bs), bs, 0, st>>>(t1, rc, nc, c1, c1, c1, FastDiv(c1), FastDiv(c1));
-    g_launches += 3;
+    restrict_pass<2, T>(rf, t0, nc, f1, f1, c1, st);
+    restrict_pass<1, T>(t0, t1, nc, f1, c1, c1, st);
+    restrict_pass<0, T>(t1, rc, nc, c1, c1, c1, st);
   } else {
-    hrestrict_pass<1, T><<<grid_for((int64_t)f1 * c1, bs), bs, 0, st>>>(rf, t0, nc, f1, c1, 1, FastDiv(f1), FastDiv(c1));
-    hrestrict_pass<0, T><<<grid_for((int64_t)c1 * c1, bs), bs, 0, st>>>(t0, rc, nc, c1, c1, 1, FastDiv(c1), FastDiv(c1));
-    g_launches += 2;
+    restrict_pass<1, T>(rf, t0, nc, f1, c1, 1, st);
+    restrict_pass<0, T>(t0, rc, nc, c1, c1, 1, st);
   }
+  g_launches += DIM;
   return cudaGetLastError();
 }
 
@@ -751,6 +759,11 @@ static cudaError_t patch_gather_group(int dim, int prec, int count, const Gather
 }
 
 // The passes of h_prolong_t / h_restrict_t with each job's extents.
+template <typename T>
+static TransferJob<T> transfer_job(const T* in, T* out, int nc, int ex, int ey, int ez) {
+  return TransferJob<T>{in, out, nc, ex, ey, ez, FastDiv(ex), FastDiv(ey), FastDiv(nc + 1)};
+}
+
 template <int DIM, typename T>
 static cudaError_t h_prolong_group_t(int count, const TransferSolveJob* jobs, cudaStream_t st) {
   GroupOf<TransferJob<T>> g[3];
@@ -765,17 +778,17 @@ static cudaError_t h_prolong_group_t(int count, const TransferSolveJob* jobs, cu
     const T* uc = (const T*)a.in;
     T *uf = (T*)a.out, *t0 = (T*)a.t0, *t1 = (T*)a.t1;
     if (DIM == 3) {
-      g[0].job[j] = TransferJob<T>{uc, t0, nc, f1, c1, c1, FastDiv(f1), FastDiv(c1)};
-      g[1].job[j] = TransferJob<T>{t0, t1, nc, f1, f1, c1, FastDiv(f1), FastDiv(f1)};
-      g[2].job[j] = TransferJob<T>{t1, uf, nc, f1, f1, f1, FastDiv(f1), FastDiv(f1)};
-      work[0] += (int64_t)f1 * c1 * c1;
-      work[1] += (int64_t)f1 * f1 * c1;
-      work[2] += (int64_t)f1 * f1 * f1;
+      g[0].job[j] = transfer_job<T>(uc, t0, nc, f1, c1, c1);
+      g[1].job[j] = transfer_job<T>(t0, t1, nc, f1, f1, c1);
+      g[2].job[j] = transfer_job<T>(t1, uf, nc, f1, f1, f1);
+      work[0] += transfer_items<0>(nc, f1, c1, c1);
+      work[1] += transfer_items<1>(nc, f1, f1, c1);
+      work[2] += transfer_items<2>(nc, f1, f1, f1);
     } else {
-      g[0].job[j] = TransferJob<T>{uc, t0, nc, f1, c1, 1, FastDiv(f1), FastDiv(c1)};
-      g[1].job[j] = TransferJob<T>{t0, uf, nc, f1, f1, 1, FastDiv(f1), FastDiv(f1)};
-      work[0] += (int64_t)f1 * c1;
-      work[1] += (int64_t)f1 * f1;
+      g[0].job[j] = transfer_job<T>(uc, t0, nc, f1, c1, 1);
+      g[1].job[j] = transfer_job<T>(t0, uf, nc, f1, f1, 1);
+      work[0] += transfer_items<0>(nc, f1, c1, 1);
+      work[1] += transfer_items<1>(nc, f1, f1, 1);
     }
     for (int i = 0; i < 3; ++i) g[i].start[j + 1] = work[i];
   }
@@ -807,17 +820,17 @@ static cudaError_t h_restrict_group_t(int count, const TransferSolveJob* jobs, c
     const T* rf = (const T*)a.in;
     T *rc = (T*)a.out, *t0 = (T*)a.t0, *t1 = (T*)a.t1;
     if (DIM == 3) {
-      g[0].job[j] = TransferJob<T>{rf, t0, nc, f1, f1, c1, FastDiv(f1), FastDiv(f1)};
-      g[1].job[j] = TransferJob<T>{t0, t1, nc, f1, c1, c1, FastDiv(f1), FastDiv(c1)};
-      g[2].job[j] = TransferJob<T>{t1, rc, nc, c1, c1, c1, FastDiv(c1), FastDiv(c1)};
-      work[0] += (int64_t)f1 * f1 * c1;
-      work[1] += (int64_t)f1 * c1 * c1;
-      work[2] += (int64_t)c1 * c1 * c1;
+      g[0].job[j] = transfer_job<T>(rf, t0, nc, f1, f1, c1);
+      g[1].job[j] = transfer_job<T>(t0, t1, nc, f1, c1, c1);
+      g[2].job[j] = transfer_job<T>(t1, rc, nc, c1, c1, c1);
+      work[0] += transfer_items<2>(nc, f1, f1, c1);
+      work[1] += transfer_items<1>(nc, f1, c1, c1);
+      work[2] += transfer_items<0>(nc, c1, c1, c1);
     } else {
-      g[0].job[j] = TransferJob<T>{rf, t0, nc, f1, c1, 1, FastDiv(f1), FastDiv(c1)};
-      g[1].job[j] = TransferJob<T>{t0, rc, nc, c1, c1, 1, FastDiv(c1), FastDiv(c1)};
-      work[0] += (int64_t)f1 * c1;
-      work[1] += (int64_t)c1 * c1;
+      g[0].job[j] = transfer_job<T>(rf, t0, nc, f1, c1, 1);
+      g[1].job[j] = transfer_job<T>(t0, rc, nc, c1, c1, 1);
+      work[0] += transfer_items<1>(nc, f1, c1, 1);
+      work[1] += transfer_items<0>(nc, c1, c1, 1);
     }
     for (int i = 0; i < 3; ++i) g[i].start[j + 1] = work[i];
   }
