@@ -37,12 +37,10 @@ D, NCELL, K = 3, 32, 4
 # latency each, about 0.2 ms in FP64 -- and no work worth the launch.
 COARSE_DOFS = 4096
 ORACLE_N = 4          # bounded CPU sample: same degree and dimension, 4^3 cells (4,913 DoFs)
-FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 (measured 1.255 with a project FMA probe)
 FP32_PEAK_TFLOPS = 78.5  # measured FP32 FMA (128 lanes x 152 SMs x 2 x ~2.0 GHz)
 # DRAM bytes (read + write) of one FP64 patch launch at 32^3 Q4, from one ncu
-# capture of that launch (57.12 MB + 54.64 MB); to be re-taken whenever
-# patch_cart_kernel changes.
-PATCH64_TRAFFIC_BYTES = 111762432
+# capture of that launch; to be re-taken whenever patch_dense_kernel changes.
+PATCH64_TRAFFIC_BYTES = 117700000
 
 
 # ----------------------------------------------------------------- flop model
@@ -60,10 +58,23 @@ def p_hierarchy(k):
     return lv + [k]
 
 
+def product_flops(d, k):
+    """Tensor-core operations of one FP64 Cartesian patch solve as the patch
+    kernel executes it (K <= 5): 34 digit products of the 16 x 16 tiles of the
+    sector matrices (k or k - 1 rows per direction).  Counts an FMA as 2."""
+    tiles = 0
+    for s in range(2 ** d):
+        rows = 1
+        for a in range(d):
+            rows *= k - ((s >> a) & 1)
+        tiles += ((rows + 15) // 16) ** 2
+    return 34 * tiles * 16 * 16 * 2
+
+
 def patch_flops(d, k, n_iter=1):
-    """Floating-point operations of one Cartesian patch solve as executed by
-    the patch kernel: gather, full p-multigrid V-cycle (two patch vmults per
-    level), scatter.  Counts an FMA as 2."""
+    """Floating-point operations of one Cartesian patch solve by sum
+    factorisation, the method's own work: gather, full p-multigrid V-cycle (two
+    patch vmults per level), scatter.  Counts an FMA as 2."""
     levels = p_hierarchy(k)
 
     def vmult(p):
@@ -198,6 +209,15 @@ def cpu_baseline_entry(res):
 
 
 # ----------------------------------------------------------------- extra sections
+def _measured_bf16_tflops():
+    """The pool's measured cuBLAS bf16 burst rate, else the fallback 1,900."""
+    try:
+        with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"])
+    except (OSError, ValueError, KeyError):
+        return 1900.0
+
+
 def _measured_hbm_gbs():
     """The machine's measured copy bandwidth (generated MEASURED_PEAKS.json
     beside this file), else the profiling recipe's fallback of 6.8 TB/s."""
@@ -209,6 +229,7 @@ def _measured_hbm_gbs():
 
 
 HBM_GBS, HBM_PEAK_KIND = _measured_hbm_gbs()
+BF16_TFLOPS = _measured_bf16_tflops()
 
 
 def _timed_ms(torch, stream, flush, fn, reps=5):
@@ -765,7 +786,7 @@ def main():
         patch_launch_ms = phases[1]
         n_patches = (NCELL - 1) ** D
         flops_launch = patch_flops(D, K) * n_patches
-        achieved = flops_launch / (patch_launch_ms * 1e-3) / 1e12
+        achieved = product_flops(D, K) * n_patches / (patch_launch_ms * 1e-3) / 1e12
         phases32 = ctx32.smoother_phase_times(reps=10)
 
         # ---- end-to-end through the host-buffer C-ABI path
@@ -821,11 +842,13 @@ def main():
             "rel_residual": infoff[-1].rel_residual, "true_rel_residual_fp64_operator": true_res_ff,
             "l2_error": l2err_ff, "apply_ms": statistics.median(t_apply_ff),
             "speedup_vs_fp64": pct(solve64, 50) / pct(solveff, 50)},
-        "roofline": {"kernel": "patch_cart_kernel<3,double> (all 29,791 patches of the finest level)",
-                     "bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                     "frac": achieved / FP64_PEAK_TFLOPS, "traffic": PATCH64_TRAFFIC_BYTES,
-                     "flops_per_launch": flops_launch, "launch_ms": patch_launch_ms,
-                     "peak_note": "nominal FP64 (measured FMA probe 1.255 TFLOP/s)"},
+        "roofline": {"kernel": "patch_dense_kernel<3,double> (all 29,791 patches of the finest level)",
+                     "bound": "tensor", "achieved": achieved, "peak": BF16_TFLOPS, "unit": "TFLOP/s",
+                     "frac": achieved / BF16_TFLOPS, "traffic": PATCH64_TRAFFIC_BYTES,
+                     "flops_per_launch": product_flops(D, K) * n_patches, "launch_ms": patch_launch_ms,
+                     "local_solver_tflops": flops_launch / (patch_launch_ms * 1e-3) / 1e12,
+                     "peak_note": "measured cuBLAS bf16 burst; the kernel's FP16 digit products use mma.sync "
+                                  "(604 TFLOP/s measured)"},
         "smoother_phases_ms": {"fp64": {"residual": phases[0], "patch": phases[1], "gather": phases[2]},
                                "fp32": {"residual": phases32[0], "patch": phases32[1], "gather": phases32[2],
                                         "patch_tflops": flops_launch / (phases32[1] * 1e-3) / 1e12,

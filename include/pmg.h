@@ -77,7 +77,12 @@ enum pmg_outer {
 };
 
 /* Layout of the patches of one thread block in shared memory (the smoother's
- * local solves, §3.2).  Both give bitwise the same results. */
+ * local solves, §3.2).  Both give bitwise the same results.  The layout,
+ * patches_per_block, patch_threads and patch_persistent shape the
+ * sum-factorised patch kernels: deformed and distorted meshes, and Cartesian
+ * 3D FP32 of degree >= 6 and FP64 of degree 8.  The other Cartesian patches are
+ * solved by products with the local solver's matrix, which have one block
+ * shape: there the values are checked and reported, without effect. */
 enum pmg_patch_layout {
   PMG_PATCH_AUTO = 0,         /* autotuned (or patch-major when patches_per_block > 0) */
   PMG_PATCH_MAJOR = 1,        /* each patch's vectors contiguous, patches_per_block patches per block */
@@ -94,7 +99,9 @@ enum pmg_outer_apply {
   PMG_OUTER_APPLY_FLOAT_FLOAT = 1   /* FP64 vectors in and out, every product and sum carried as an unevaluated
                                        pair of floats (about 48 significant bits, relative error of A x within
                                        a few 1e-14 of |A| |x|) on the FP32 pipes -- on GB300 several times
-                                       faster than the FP64 pipes; the coarse-matrix assembly stays in FP64.
+                                       faster than the FP64 pipes (Cartesian FP64 applies of degree >= 2 take
+                                       the tensor cores: 32^3 Q4 0.112 ms, float-float 0.093 ms); the
+                                       coarse-matrix assembly stays in FP64.
                                        Cartesian meshes; deformed and distorted ones in 3D with degree <= 3
                                        and geom_precision PMG_FP32 (else PMG_ERR_UNSUPPORTED) */
 };
@@ -280,7 +287,8 @@ int pmg_synchronize(pmg_ctx* ctx);
 int64_t pmg_launch_count(void);
 
 /* Patches per thread block the smoother kernels of this context use on the
- * finest level: the config's value, or the autotuned one (layout and block
+ * finest level: the config's value, or the autotuned one -- for the
+ * sum-factorised kernels (enum pmg_patch_layout), else a rule (layout and block
  * shape timed per dimension, degree, precision, geometry, local cycles,
  * smoother and finest n on the finest level's patch launches of one sweep;
  * cached for the process and, if the environment variable PMG_TUNE_FILE

@@ -200,11 +200,11 @@ static cudaError_t patch_dense_t(const T* r, T* dst, int n, const PatchParamsHos
     }
     return cudaGetLastError();
   } else {
-  const unsigned grid = (J.npatch + dense_batch<DIM, T>() - 1) / dense_batch<DIM, T>();
-  if constexpr (K == 1) patch_point_kernel<DIM, T><<<grid, 256, 0, st>>>(J);
-  else patch_dense_kernel<DIM, T><<<grid, 32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::SMEM, st>>>(J);
-  g_launches += 1;
-  return cudaGetLastError();
+    const unsigned grid = (J.npatch + dense_batch<DIM, T>() - 1) / dense_batch<DIM, T>();
+    if constexpr (K == 1) patch_point_kernel<DIM, T><<<grid, 256, 0, st>>>(J);
+    else patch_dense_kernel<DIM, T><<<grid, 32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T>::SMEM, st>>>(J);
+    g_launches += 1;
+    return cudaGetLastError();
   }
 }
 
@@ -216,28 +216,28 @@ static cudaError_t patch_cart_t(const T* r, T* dst, int n, int ppc, int n_iter, 
   if (np == 0) return cudaSuccess;  // no interior vertex (of this colour), no patch
   if constexpr (kDense) return patch_dense_t<DIM, T>(r, dst, n, H, st);
   else {
-  if (ppc < 1 || ppc > kMaxPatchesPerBlock) return cudaErrorInvalidValue;
-  const int64_t nbatch = (np + ppc - 1) / ppc;
-  // more patch lines than threads is fine: every step loops over its lines
-  const int threads = std::min(kPatchMaxThreads, (ppc * S::TPP + 31) / 32 * 32);
-  const int prec = sizeof(T) == 8 ? 0 : 1;
-  const int smem = ppc * patch_smem(DIM, prec, n_iter) + patch_cart_extra_smem(DIM, prec);
-  if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
-  unsigned grid = (unsigned)nbatch;
-  if (counter) {
-    grid = persistent_grid((const void*)patch_cart_kernel<DIM, T>, threads, smem, nbatch);
-    if (grid < nbatch) {  // more than one wave: persistent blocks
-      cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-      if (e != cudaSuccess) return e;
-    } else {
-      grid = (unsigned)nbatch;
-      counter = nullptr;
+    if (ppc < 1 || ppc > kMaxPatchesPerBlock) return cudaErrorInvalidValue;
+    const int64_t nbatch = (np + ppc - 1) / ppc;
+    // more patch lines than threads is fine: every step loops over its lines
+    const int threads = std::min(kPatchMaxThreads, (ppc * S::TPP + 31) / 32 * 32);
+    const int prec = sizeof(T) == 8 ? 0 : 1;
+    const int smem = ppc * patch_smem(DIM, prec, n_iter) + patch_cart_extra_smem(DIM, prec);
+    if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
+    unsigned grid = (unsigned)nbatch;
+    if (counter) {
+      grid = persistent_grid((const void*)patch_cart_kernel<DIM, T>, threads, smem, nbatch);
+      if (grid < nbatch) {  // more than one wave: persistent blocks
+        cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
+      } else {
+        grid = (unsigned)nbatch;
+        counter = nullptr;
+      }
     }
-  }
-  patch_cart_kernel<DIM, T><<<grid, threads, smem, st>>>(r, dst, n, ppc, n_iter, dinv, dinv_len(DIM), to_params<T>(H),
-                                                         counter, nbatch);
-  g_launches += 1;
-  return cudaGetLastError();
+    patch_cart_kernel<DIM, T><<<grid, threads, smem, st>>>(r, dst, n, ppc, n_iter, dinv, dinv_len(DIM), to_params<T>(H),
+                                                           counter, nbatch);
+    g_launches += 1;
+    return cudaGetLastError();
   }
 }
 
@@ -264,26 +264,26 @@ static cudaError_t patch_cart_il_t(const T* r, T* dst, int n, int threads, int n
   if (np == 0) return cudaSuccess;
   if constexpr (kDense) return patch_dense_t<DIM, T>(r, dst, n, H, st);
   else {
-  const int prec = sizeof(T) == 8 ? 0 : 1;
-  const int il = patch_il_of(DIM, prec, n_iter);
-  if (il == 0 || threads < 32 || threads > 1024 || threads % 32) return cudaErrorInvalidValue;
-  const int smem = il * patch_il_smem(DIM, prec, n_iter) + patch_cart_extra_smem(DIM, prec);
-  const int64_t nbatch = (np + il - 1) / il;
-  unsigned grid = (unsigned)nbatch;
-  if (counter) {
-    grid = persistent_grid((const void*)patch_cart_il_kernel<DIM, T>, threads, smem, nbatch);
-    if (grid < nbatch) {
-      cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-      if (e != cudaSuccess) return e;
-    } else {
-      grid = (unsigned)nbatch;
-      counter = nullptr;
+    const int prec = sizeof(T) == 8 ? 0 : 1;
+    const int il = patch_il_of(DIM, prec, n_iter);
+    if (il == 0 || threads < 32 || threads > 1024 || threads % 32) return cudaErrorInvalidValue;
+    const int smem = il * patch_il_smem(DIM, prec, n_iter) + patch_cart_extra_smem(DIM, prec);
+    const int64_t nbatch = (np + il - 1) / il;
+    unsigned grid = (unsigned)nbatch;
+    if (counter) {
+      grid = persistent_grid((const void*)patch_cart_il_kernel<DIM, T>, threads, smem, nbatch);
+      if (grid < nbatch) {
+        cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
+      } else {
+        grid = (unsigned)nbatch;
+        counter = nullptr;
+      }
     }
-  }
-  patch_cart_il_kernel<DIM, T><<<grid, threads, smem, st>>>(r, dst, n, n_iter, dinv, dinv_len(DIM), to_params<T>(H),
-                                                            counter, nbatch);
-  g_launches += 1;
-  return cudaGetLastError();
+    patch_cart_il_kernel<DIM, T><<<grid, threads, smem, st>>>(r, dst, n, n_iter, dinv, dinv_len(DIM), to_params<T>(H),
+                                                              counter, nbatch);
+    g_launches += 1;
+    return cudaGetLastError();
   }
 }
 
@@ -496,42 +496,42 @@ static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int 
     g_launches += 1;
     return cudaGetLastError();
   } else {
-  using S = PatchShape<DIM>;
-  if (ppc < 1 || ppc > kMaxPatchesPerBlock) return cudaErrorInvalidValue;
-  GroupOf<PatchJob<T>> G;
-  G.count = 0;
-  G.start[0] = 0;
-  int64_t nbatch = 0;
-  for (int j = 0; j < count; ++j) {
-    const int64_t np = patch_count(DIM, jobs[j].n, jobs[j].P.colour);
-    if (np == 0) continue;  // no patch (of this colour) on this job's level
-    PatchJob<T>& J = G.job[G.count++];
-    J.r = (const T*)jobs[j].r;
-    J.dst = (T*)jobs[j].dst;
-    J.n = jobs[j].n;
-    J.P = to_params<T>(jobs[j].P);
-    nbatch += (np + ppc - 1) / ppc;
-    G.start[G.count] = nbatch;
-  }
-  if (G.count == 0) return cudaSuccess;
-  const int threads = std::min(kPatchMaxThreads, (ppc * S::TPP + 31) / 32 * 32);
-  const int prec = sizeof(T) == 8 ? 0 : 1;
-  const int smem = ppc * patch_smem(DIM, prec, n_iter) + patch_cart_extra_smem(DIM, prec);
-  if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
-  unsigned grid = (unsigned)nbatch;
-  if (counter) {
-    grid = persistent_grid((const void*)patch_cart_group_kernel<DIM, T>, threads, smem, nbatch);
-    if (grid < nbatch) {
-      cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-      if (e != cudaSuccess) return e;
-    } else {
-      grid = (unsigned)nbatch;
-      counter = nullptr;
+    using S = PatchShape<DIM>;
+    if (ppc < 1 || ppc > kMaxPatchesPerBlock) return cudaErrorInvalidValue;
+    GroupOf<PatchJob<T>> G;
+    G.count = 0;
+    G.start[0] = 0;
+    int64_t nbatch = 0;
+    for (int j = 0; j < count; ++j) {
+      const int64_t np = patch_count(DIM, jobs[j].n, jobs[j].P.colour);
+      if (np == 0) continue;  // no patch (of this colour) on this job's level
+      PatchJob<T>& J = G.job[G.count++];
+      J.r = (const T*)jobs[j].r;
+      J.dst = (T*)jobs[j].dst;
+      J.n = jobs[j].n;
+      J.P = to_params<T>(jobs[j].P);
+      nbatch += (np + ppc - 1) / ppc;
+      G.start[G.count] = nbatch;
     }
-  }
-  patch_cart_group_kernel<DIM, T><<<grid, threads, smem, st>>>(ppc, n_iter, dinv, dinv_len(DIM), counter, nbatch, G);
-  g_launches += 1;
-  return cudaGetLastError();
+    if (G.count == 0) return cudaSuccess;
+    const int threads = std::min(kPatchMaxThreads, (ppc * S::TPP + 31) / 32 * 32);
+    const int prec = sizeof(T) == 8 ? 0 : 1;
+    const int smem = ppc * patch_smem(DIM, prec, n_iter) + patch_cart_extra_smem(DIM, prec);
+    if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
+    unsigned grid = (unsigned)nbatch;
+    if (counter) {
+      grid = persistent_grid((const void*)patch_cart_group_kernel<DIM, T>, threads, smem, nbatch);
+      if (grid < nbatch) {
+        cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
+      } else {
+        grid = (unsigned)nbatch;
+        counter = nullptr;
+      }
+    }
+    patch_cart_group_kernel<DIM, T><<<grid, threads, smem, st>>>(ppc, n_iter, dinv, dinv_len(DIM), counter, nbatch, G);
+    g_launches += 1;
+    return cudaGetLastError();
   }
 }
 

@@ -628,7 +628,10 @@ __global__ void __launch_bounds__(256) cart_pass_ff_group(const __grid_constant_
 }
 
 // ===========================================================================
-// Vertex-patch smoother with the local p-multigrid solver (§2.1, §2.2, §3).
+// Vertex-patch smoother with the local p-multigrid solver (§2.1, §2.2, §3) by
+// sum factorisation: 3D FP32 of K >= 6 and FP64 of K = 8, the deformed
+// patches (kernels_def.cuh), and the set-up of the matrices that the other
+// Cartesian parts multiply by (kernels_patch.cuh).
 // A thread block owns `np` patches, processed in lockstep.  Every step of
 // the local V-cycle is a set of independent 1D line contractions (or
 // element-wise updates); the (patch, line) pairs of all patches of the block
