@@ -95,7 +95,11 @@ enum pmg_patch_layout {
 
 /* Arithmetic of the FP64 operator apply. */
 enum pmg_outer_apply {
-  PMG_OUTER_APPLY_FP64 = 0,         /* IEEE double (default) */
+  PMG_OUTER_APPLY_FP64 = 0,         /* IEEE double vectors (default).  Cartesian, degree >= 2 (2D: >= 3): exact
+                                       products of the cells' values in 60-bit fixed point with the element
+                                       matrix; the error at every node is within about 30 (k + 1) roundings of
+                                       (|K|x|M|x|M| + ...) |x| (1D matrices, rounded themselves), whatever the
+                                       range of x.  An infinity or NaN makes every result of its cells NaN */
   PMG_OUTER_APPLY_FLOAT_FLOAT = 1   /* FP64 vectors in and out, every product and sum carried as an unevaluated
                                        pair of floats (about 48 significant bits, relative error of A x within
                                        a few 1e-14 of |A| |x|) on the FP32 pipes -- on GB300 several times
@@ -216,7 +220,11 @@ int pmg_residual(pmg_ctx* ctx, int level, int prec, const void* b, const void* u
  * multiplicative, Algorithm 1 itself (per parity colour: r = b - A u, then
  * u += Pi_j^T LocalSolve_j(Pi_j r) for every patch of the colour), colours in
  * increasing order.  LocalSolve = Algorithm 2 around the p-multigrid V-cycle
- * of Algorithm 3 (full, or half with local_half). */
+ * of Algorithm 3 (full, or half with local_half).  On Cartesian meshes it is
+ * one matrix B per method; solved as a product its error at every node is
+ * within 1e-12 (FP32: 5e-4) of |B||r|, and within about 20 roundings of the
+ * patch's largest correction.  An infinity or NaN in a patch makes every
+ * correction of the patch NaN (FP64). */
 int pmg_smooth(pmg_ctx* ctx, int level, int prec, const void* b, void* u, int sweeps);
 
 /* One geometric V-cycle on the finest level from a zero guess: z = B r

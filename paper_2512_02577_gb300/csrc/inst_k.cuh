@@ -18,6 +18,9 @@ constexpr int DP = PMG_DIM;
 // the Cartesian patches of this part are solved by the dense sector products
 // (K = 1: pointwise) instead of sum factorisation
 constexpr bool kDense = K == 1 || PatchDense<DP, TP>::ok() || kStaged;
+// the degree's parts of either precision that do so
+constexpr bool kProducts64 = PatchDense<DP, double>::ok() || (DP == 3 && (K == 6 || K == 7));
+constexpr bool kProducts32 = PatchDense<DP, float>::ok();
 // FP64 operator applies by cells; line passes where they are as fast (2D K = 2:
 // 9 of a tile's 16 rows used, 0.218 against 0.195 ms at 1024^2 cells) and for
 // K = 1 (the 2^d results per cell need more scratch than the passes)
@@ -153,6 +156,18 @@ static unsigned persistent_grid(const void* kern, int threads, int smem, int64_t
   return (unsigned)std::max<int64_t>(g, 1);
 }
 
+// the scale c of a job's results, for FP64 as an integer and an exponent: the
+// operands are scaled by 2^(1085 - D - e_window), D the directions in which
+// images are summed, and the products by 2^-68
+template <int D, typename T>
+static void set_scale(DenseJob<T>& J, double c) {
+  J.c = (T)c;
+  int e = 0;
+  const bool finite = std::isfinite(c);
+  J.cmul = finite ? (unsigned long long)std::ldexp(std::frexp(c, &e), 64) : 0;
+  J.vexp = finite ? e - 64 + 68 - (1085 - D) : 0;
+}
+
 template <int DIM, typename T>
 static DenseJob<T> dense_job(const T* r, T* dst, int n, const PatchParamsHost& H) {
   DenseJob<T> J{};
@@ -162,14 +177,7 @@ static DenseJob<T> dense_job(const T* r, T* dst, int n, const PatchParamsHost& H
   J.n = n;
   J.colour = H.colour;
   const double c = (H.colour < 0 ? H.omega_as : 1.0) * (K == 1 ? H.inv_a0 : 1.0 / H.scale);
-  J.c = (T)c;
-  int e = 0;
-  const bool finite = std::isfinite(c);
-  J.cmul = finite ? (unsigned long long)std::ldexp(std::frexp(c, &e), 64) : 0;
-  // the operands are scaled by 2^(1080 - SH - e_patch), the products by 2^-52 (dense_body); SL digits: 2^8 and
-  // 2^-16 for the eighth
-  constexpr int SH = Sectors<DIM, kPatchM>::SPLIT ? DIM + 3 : 3;
-  J.vexp = finite ? e - 64 + 52 + 8 * (PatchDense<DIM, double>::SL - 7) - (1080 - SH) : 0;
+  set_scale<Sectors<DIM, kPatchM>::SPLIT ? DIM : 0>(J, c);
   J.npatch = (uint32_t)patch_count(DIM, n, H.colour);
   J.d0 = FastDiv(std::max(1, patch_count_1d(n, H.colour, 0)));
   J.d1 = FastDiv(DIM == 3 ? std::max(1, patch_count_1d(n, H.colour, 1)) : 1);
@@ -537,81 +545,94 @@ static cudaError_t patch_cart_group_t(int count, const PatchSolveJob* jobs, int 
 
 // ---------------------------------------------------------------- dense patch operator
 // Device bytes of the part's table of sector matrices (0: not a dense part)
-// and of the FP64 scratch its set-up needs: columns, entries, statistics.
+// and of the FP64 scratch that its set-up needs: the columns' low parts and
+// the exponents of orbits and rows.  The columns themselves end the table.
 static int64_t patch_table_bytes(int dim, int prec) {
   if (!mine(dim, prec) || !kDense || K == 1) return 0;
   return PatchDense<DP, TP>::TABLE_BYTES;
 }
 
-static int64_t patch_scratch_bytes(int dim) {
-  using S = Sectors<DP, kPatchM>;  // the cell's matrices need less
-  return dim == DP ? 8 * ((int64_t)S::ORBITS * S::NODES + S::ENTRIES) + 4 * (S::ROWS + 4) : 0;
+template <class S>
+constexpr int64_t sector_scratch_bytes() {
+  return 8 * (int64_t)S::ORBITS * S::NODES + 4 * (S::ORBITS + S::ROWS);
 }
+template <class S>
+static int* sector_exponents(double* scratch) { return (int*)(scratch + (int64_t)S::ORBITS * S::NODES); }
 
-// FP64 part: sector matrices of the local solver (unit scale; dinv: its
-// inverse diagonals) into the scratch: entries, columns, the classes' least
-// row exponents (4) and the row exponents
-template <int DIM>
-static int64_t scratch_ints() {
-  using S = Sectors<DIM, kPatchM>;
-  return (int64_t)S::ORBITS * S::NODES + S::ENTRIES;
+static int64_t patch_scratch_bytes(int dim) { return dim == DP ? sector_scratch_bytes<Sectors<DP, kPatchM>>() : 0; }
+
+static double* patch_columns(int dim, int prec, void* table) {
+  return mine(dim, prec) ? (double*)((char*)table + PatchDense<DP, TP>::COLUMNS) : nullptr;
 }
 
 template <int DIM, typename V>
-static cudaError_t patch_columns(const PatchParamsHost& H, int n_iter, const double* dinv, double* columns,
-                                 cudaStream_t st) {
+static cudaError_t patch_columns_t(const PatchParamsHost& H, int n_iter, const double* dinv, double* columns,
+                                   double* scratch, cudaStream_t st) {
+  using S = Sectors<DIM, kPatchM>;
   const int np = std::max(1, 32 / PatchShape<DIM>::TPP);  // few: a block's FP64 work is its latency
   const int threads = std::min(256, (np * PatchShape<DIM>::TPP + 31) / 32 * 32);
   const int smem = np * PatchShape<DIM>::ELEMS * (int)sizeof(V);
   if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
   for (int it = 0; it < n_iter; ++it)
-    patch_columns_kernel<DIM, V><<<(Sectors<DIM, kPatchM>::ORBITS + np - 1) / np, threads, smem, st>>>(
-        columns, np, it == 0, dinv, to_params<double>(H));
+    patch_columns_kernel<DIM, V><<<(S::ORBITS + np - 1) / np, threads, smem, st>>>(columns, scratch, np, it == 0, dinv,
+                                                                                   to_params<double>(H));
   g_launches += n_iter;
   return cudaGetLastError();
 }
 
-// the patches of K = 8 in 3D do not fit a block in pairs of doubles
-template <int DIM>
-constexpr bool columns_dd() { return PatchShape<DIM>::ELEMS * 16 <= kMaxDynSmem; }
+// exponents of the sector matrices from the columns: the orbits', then the rows'
+template <int DIM, int M>
+static cudaError_t sector_exponents_t(const double* columns, double* scratch, cudaStream_t st) {
+  using S = Sectors<DIM, M>;
+  int* exps = sector_exponents<S>(scratch);
+  cudaError_t e = cudaMemsetAsync(exps, 0x7F, 4 * S::ORBITS, st);
+  if (e != cudaSuccess) return e;
+  sector_exponents_kernel<DIM, M><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, scratch, exps + S::ORBITS, exps);
+  g_launches += 1;
+  return cudaGetLastError();
+}
 
+// fragments (and FP64 exponents) of a table from its columns and the scratch
+template <int DIM, typename T, int M>
+static cudaError_t sector_table_t(const double* columns, double* scratch, void* table, cudaStream_t st) {
+  using S = Sectors<DIM, M>;
+  const int* exps = sector_exponents<S>(scratch);
+  sector_table_kernel<DIM, T, M><<<(S::TILES * 128 + 255) / 256, 256, 0, st>>>(columns, scratch, exps + S::ORBITS, exps,
+                                                                               (uint32_t*)table);
+  g_launches += 1;
+  return cudaGetLastError();
+}
+
+// FP64 part: columns of the local solver (unit scale; dinv: its inverse
+// diagonals) for products in precision prec, and the exponents
 template <int DIM, typename T>
 static cudaError_t patch_entries_t(const PatchParamsHost& H, int n_iter, bool fp64, const double* dinv,
-                                   double* scratch, cudaStream_t st) {
+                                   double* columns, double* scratch, cudaStream_t st) {
   if constexpr (sizeof(T) == 8 && K > 1) {
-    using S = Sectors<DIM, kPatchM>;
-    double* columns = scratch + S::ENTRIES;
-    int* minexp = (int*)(scratch + scratch_ints<DIM>());
-    cudaError_t e = cudaMemsetAsync(minexp, 0x7F, 16, st);
-    if (e != cudaSuccess) return e;
-    if constexpr (columns_dd<DIM>())
-      e = fp64 ? patch_columns<DIM, dd>(H, n_iter, dinv, columns, st)
-               : patch_columns<DIM, double>(H, n_iter, dinv, columns, st);
-    else e = patch_columns<DIM, double>(H, n_iter, dinv, columns, st);
-    if (e != cudaSuccess) return e;
-    sector_entries_kernel<DIM, false><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, scratch, minexp + 4, minexp);
-    g_launches += 1;
-    return cudaGetLastError();
+    cudaError_t e = cudaErrorInvalidValue;  // no such product part
+    if (fp64) {
+      if constexpr (kProducts64) e = patch_columns_t<DIM, dd>(H, n_iter, dinv, columns, scratch, st);
+    } else {
+      if constexpr (kProducts32) e = patch_columns_t<DIM, double>(H, n_iter, dinv, columns, scratch, st);
+    }
+    if constexpr (kProducts64 || kProducts32)
+      if (e == cudaSuccess) e = sector_exponents_t<DIM, kPatchM>(columns, scratch, st);
+    return e;
   }
   return cudaErrorInvalidValue;
 }
 
 static cudaError_t patch_entries(int dim, const PatchParamsHost& H, int n_iter, int prec, const double* dinv,
-                                 double* scratch, cudaStream_t st) {
+                                 double* columns, double* scratch, cudaStream_t st) {
   if (dim != DP) return cudaErrorInvalidValue;
-  return patch_entries_t<DP, TP>(H, n_iter, prec == 0, dinv, scratch, st);
+  return patch_entries_t<DP, TP>(H, n_iter, prec == 0, dinv, columns, scratch, st);
 }
 
-// the part's table from the scratch
+// the part's table from its columns and the scratch
 template <int DIM, typename T>
-static cudaError_t patch_table_t(const double* scratch, void* table, cudaStream_t st) {
-  if constexpr (kDense && K > 1) {
-    const int* minexp = (const int*)(scratch + scratch_ints<DIM>());
-    const int64_t work = (int64_t)Sectors<DIM, kPatchM>::TILES * 128;
-    sector_table_kernel<DIM, T, false><<<(unsigned)((work + 255) / 256), 256, 0, st>>>(scratch, minexp + 4, minexp, (uint32_t*)table);
-    g_launches += 1;
-    return cudaGetLastError();
-  }
+static cudaError_t patch_table_t(double* scratch, void* table, cudaStream_t st) {
+  if constexpr (kDense && K > 1)
+    return sector_table_t<DIM, T, kPatchM>(patch_columns(DIM, sizeof(T) == 8 ? 0 : 1, table), scratch, table, st);
   return cudaErrorInvalidValue;
 }
 
@@ -633,20 +654,22 @@ static int64_t patch_stage_batches(int n) { return stage_batches_t<DP>(n); }
 
 // ---------------------------------------------------------------- FP64 apply by cells
 static int64_t cell_table_bytes(int dim) { return dim == DP && kCellDense ? CellDense<DP>::TABLE_BYTES : 0; }
+static int64_t cell_scratch_bytes(int dim) {
+  return dim == DP && kCellDense ? sector_scratch_bytes<Sectors<DP, kCellM>>() : 0;
+}
 
 // the cell's table, by way of the scratch (used on the stream, free again afterwards)
 template <int DIM, typename T>
 static cudaError_t cell_table_t(double* scratch, void* table, cudaStream_t st) {
   if constexpr (kCellDense) {
     using S = Sectors<DIM, kCellM>;
-    int* minexp = (int*)(scratch + S::ENTRIES);
-    cudaError_t e = cudaMemsetAsync(minexp, 0x7F, 16, st);
-    if (e != cudaSuccess) return e;
-    sector_entries_kernel<DIM, true><<<(S::ROWS + 3) / 4, 128, 0, st>>>(nullptr, scratch, minexp + 4, minexp);
-    sector_table_kernel<DIM, double, true><<<(S::TILES * 128 + 255) / 256, 256, 0, st>>>(scratch, minexp + 4, minexp,
-                                                                                        (uint32_t*)table);
-    g_launches += 2;
-    return cudaGetLastError();
+    double* columns = (double*)((char*)table + CellDense<DIM>::COLUMNS);
+    cell_columns_kernel<DIM><<<(S::ORBITS * S::NODES + 255) / 256, 256, 0, st>>>(columns, scratch);
+    g_launches += 1;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = sector_exponents_t<DIM, kCellM>(columns, scratch, st);
+    if (e == cudaSuccess) e = sector_table_t<DIM, double, kCellM>(columns, scratch, table, st);
+    return e;
   }
   return cudaErrorInvalidValue;
 }
@@ -665,10 +688,7 @@ static DenseJob<double> cell_job(const double* x, double* cells, const void* tab
   J.table = (const uint4*)table;
   J.n = n;
   J.colour = -1;
-  int e = 0;
-  J.cmul = (unsigned long long)std::ldexp(std::frexp(scale, &e), 64);
-  constexpr int SH = Sectors<DIM, kCellM>::SPLIT ? DIM + 3 : 3;
-  J.vexp = e - 64 + 52 - (1080 - SH);  // as dense_job
+  set_scale<Sectors<DIM, kCellM>::SPLIT ? DIM : 0>(J, scale);
   J.npatch = (uint32_t)ipow64(n, DIM);
   J.d0 = FastDiv(n);
   J.d1 = FastDiv(DIM == 3 ? n : 1);
@@ -724,7 +744,7 @@ static cudaError_t cell_apply_group(int dim, int count, const ApplyJob* jobs, cu
   return cell_apply_group_t<DP, TP>(count, jobs, st);
 }
 
-static cudaError_t patch_table(int dim, int prec, const double* scratch, void* table, cudaStream_t st) {
+static cudaError_t patch_table(int dim, int prec, double* scratch, void* table, cudaStream_t st) {
   if (!mine(dim, prec)) return cudaErrorInvalidValue;
   return patch_table_t<DP, TP>(scratch, table, st);
 }
@@ -919,8 +939,8 @@ static void prepare_cart(int optin, const Acc& acc) {
     acc(allow_smem(cell_dense_group_kernel<DIM>, optin));
   }
   if constexpr (sizeof(T) == 8 && K > 1) {
-    acc(allow_smem(patch_columns_kernel<DIM, double>, optin));
-    if constexpr (columns_dd<DIM>()) acc(allow_smem(patch_columns_kernel<DIM, dd>, optin));
+    if constexpr (kProducts32) acc(allow_smem(patch_columns_kernel<DIM, double>, optin));
+    if constexpr (kProducts64) acc(allow_smem(patch_columns_kernel<DIM, dd>, optin));
   }
 }
 
@@ -975,11 +995,13 @@ const KernelTable* PMG_TABLE_FN() {
       PMG_KNS::h_restrict_group,
       PMG_KNS::patch_table_bytes,
       PMG_KNS::patch_scratch_bytes,
+      PMG_KNS::patch_columns,
       PMG_KNS::patch_entries,
       PMG_KNS::patch_table,
       PMG_KNS::patch_stage_bytes,
       PMG_KNS::patch_stage_batches,
       PMG_KNS::cell_table_bytes,
+      PMG_KNS::cell_scratch_bytes,
       PMG_KNS::cell_table,
       PMG_KNS::cell_apply,
       PMG_KNS::cell_apply_group,

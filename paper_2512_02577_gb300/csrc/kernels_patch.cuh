@@ -16,17 +16,21 @@
 // FP64 pipe (1.25 TFLOP/s, two multiply-adds per clock and SM), in FP32 by
 // shared-memory traffic and the barriers between the line passes.
 //
-// FP64 arithmetic: operands in fixed point (one exponent per matrix row and per
-// patch), split into 7 or 8 signed digits of 8 bits that are exact in FP16;
-// products of digits are summed exactly by the tensor cores (integers in the
-// FP32 accumulator) and across digit pairs in 64-bit integers, keeping the 34 or
-// 36 digit pairs i + j <= 7 (0-based; without i + j = 7 the error is 100 times
-// larger).  No FP64 instruction is executed.  Error of one local solve
-// against extended precision, N(0,1) residuals, before (sum factorisation)
-// and now: K = 3 3.3e-16, 3.3e-16; K = 4 3.9e-16, 3.7e-16; K = 5 3.6e-16,
-// 3.7e-16; 2D K = 7 4.1e-16, 2.5e-16;
-// K = 6 5.4e-16, 5.4e-16; K = 7 6.3e-16, 6.1e-16.  FP32: three BF16 parts of each value
-// (8 bits each, exact), the six products of weight 2^-16 and above.
+// FP64 arithmetic (the Ozaki scheme: Ozaki, Ogita, Oishi, Rump, Numer.
+// Algorithms 59, 2012): operands in fixed point (one exponent per matrix row
+// and per patch, 60 bits of each value), split into 8 signed digits of 8 bits
+// that are exact in FP16; products of digits are summed exactly by the tensor
+// cores (integers in the FP32 accumulator) and across digit pairs in 64-bit
+// integers, keeping the 36 digit pairs i + j <= 7 (0-based).  The matrices are
+// formed in pairs of doubles, their results have one exponent per orbit of
+// mirrored nodes.  Windows whose values differ too much for one exponent:
+// kUneven below.  No FP64 instruction is executed but for subnormal windows
+// and results and for spikes.  Largest error of one local solve of a patch in
+// units of 2^-53 |B||r|, N(0,1) residuals, by sum factorisation and now: 3D K = 3 3.1,
+// 2.4; K = 4 3.5, 3.5; K = 5 3.7, 1.9; 2D K = 7 5.8, 3.4; K = 8 7.7, 5.6; with one
+// value of 1e6 among them 24, 20; 900, 400; 270, 130; 960, 360; 960, 380.  FP32:
+// three BF16 parts of each value (8 bits each, exact), the six products of
+// weight 2^-16 and above.
 //
 // Patch launch of one sweep, before and now (GB300): FP64 K = 4 at 32^3 cells
 // 2.344 and 0.195 ms (tensor pipe 35% of its cycles, issue slots 40%: the
@@ -65,12 +69,11 @@ struct Sectors {
   __host__ __device__ static constexpr int ext(int s, int d) { return d >= DIM ? 1 : ((s >> d) & 1) ? O : E; }
   __host__ __device__ static constexpr int size(int s) { return ext(s, 0) * ext(s, 1) * ext(s, 2); }
   __host__ __device__ static constexpr int tiles(int s) { return (size(s) + 15) / 16; }  // 16-row tiles per side
-  // offsets of sector s: padded rows, rows, 16 x 16 tiles, matrix entries
+  // offsets of sector s: padded rows, rows, 16 x 16 tiles
   __host__ __device__ static constexpr int prow(int s) { int o = 0; for (int t = 0; t < s; ++t) o += 16 * tiles(t); return o; }
   __host__ __device__ static constexpr int row(int s) { int o = 0; for (int t = 0; t < s; ++t) o += size(t); return o; }
   __host__ __device__ static constexpr int tile(int s) { int o = 0; for (int t = 0; t < s; ++t) o += tiles(t) * tiles(t); return o; }
-  __host__ __device__ static constexpr int entry(int s) { int o = 0; for (int t = 0; t < s; ++t) o += size(t) * size(t); return o; }
-  static constexpr int PROWS = prow(NS), ROWS = row(NS), TILES = tile(NS), ENTRIES = entry(NS);
+  static constexpr int PROWS = prow(NS), ROWS = row(NS), TILES = tile(NS);
   static_assert(ROWS == NODES, "the sectors hold every node once");
 };
 
@@ -191,11 +194,8 @@ template <int DIM, int M, typename T>
 struct Dense {
   using S = Sectors<DIM, M>;
   static constexpr bool F64 = sizeof(T) == 8;
-  // parts per value.  FP64: an eighth digit for the large matrices (M = 13,
-  // 15), whose rows hold many entries far below their largest: K = 7 in 3D
-  // has an error of 8.1e-16 with seven digits, above sum factorisation's 6.3e-16
-  static constexpr int SL = F64 ? (M > 11 ? 8 : 7) : 3;
-  static constexpr unsigned long long BIAS = 0x8080808080808080ull >> (F64 ? 64 - 8 * SL : 0);  // digits + 128
+  static constexpr int SL = F64 ? 8 : 3;  // parts per value
+  static constexpr unsigned long long BIAS = 0x8080808080808080ull;  // digits + 128
   static constexpr int P = 16;
   static constexpr int NT = P / 8;                              // 8-column tiles
   static constexpr int NSUB = 32 / P;                           // lines a warp handles at once
@@ -225,9 +225,12 @@ struct Dense {
   }
   static constexpr bool ok() { return K >= 2 && M <= (DIM == 2 ? 15 : 9) && SMEM <= kMaxDynSmem; }
   // table: 16-byte fragments, then (FP64) per row its exponent above its
-  // class's, and the exponents of the four classes (Orbit::centres)
+  // orbit's, and the exponents of the orbits' results (kNoExp in the first: a
+  // matrix that is not finite), then the columns of the orbits' first nodes
+  // (dense_spikes)
   static constexpr int FRAGS = S::TILES * SL * 32;
-  static constexpr int TABLE_BYTES = FRAGS * 16 + (F64 ? S::ROWS * 4 + 16 : 0);
+  static constexpr int COLUMNS = FRAGS * 16 + (F64 ? (S::ROWS + S::ORBITS + 3) / 4 * 16 : 0);
+  static constexpr int64_t TABLE_BYTES = COLUMNS + (int64_t)S::ORBITS * S::NODES * 8;
 };
 
 // One 16-row tile of the result: a warp's unit of work.
@@ -260,14 +263,14 @@ constexpr DenseUnits<Dense<DIM, M, T>::UNITS> dense_units() {
 }
 
 // Parameters of one level's launch.  FP64: a result is its integer x cmul x
-// 2^(vexp + the patch's exponent - its class's exponent), cmul in [2^63, 2^64).
+// 2^(vexp + the patch's exponent - its orbit's exponent), cmul in [2^63, 2^64).
 template <typename T>
 struct DenseJob {
   const T* r;
   T* dst;
   const uint4* table;
   int n, colour;
-  T c;                       // FP32: omega_AS / scale (additive) or 1 / scale
+  T c;                       // omega_AS / scale (additive) or 1 / scale; cells: scale
   unsigned long long cmul;   // FP64: the same as a normalised integer (0: not finite)
   int vexp;                  // and its binary exponent
   uint32_t npatch;
@@ -275,15 +278,17 @@ struct DenseJob {
 };
 
 // ---------------------------------------------------------------- FP64 <-> fixed point
-// v 2^(58 - e + 1022) truncated, for |v| < 2^(e - 1022) (e: biased exponent + 1 bound)
-__device__ __forceinline__ long long fixed_of(double v, int e) {
+// v 2^(60 - e + 1022) truncated, for |v| < 2^(e - 1022) (e: biased exponent + 1
+// bound); mag: its magnitude in units of 2^32
+__device__ __forceinline__ long long fixed_of(double v, int e, unsigned& mag) {
   const int hi = __double2hiint(v);
   const unsigned lo = (unsigned)__double2loint(v);
   const int ex = (hi >> 20) & 0x7FF;
   const unsigned mh = ((unsigned)hi & 0xFFFFFu) | (ex ? 0x100000u : 0u);
-  const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 5;
+  const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 7;
   const int sh = min(e - (ex ? ex : 1), 63);
   const long long x = (long long)(m >> sh);
+  mag = (unsigned)(x >> 32);
   const long long sg = (long long)(hi >> 31);
   return (x ^ sg) - sg;
 }
@@ -294,6 +299,7 @@ __device__ __forceinline__ long long fixed_of(double v, int e) {
 // by 2^100 and bounded by the high word's leading bit.
 struct PatchScale {
   int e;
+  bool subnormal;  // all values: fixed_of is exact
   bool bad;  // an infinity or NaN, or a matrix that is not finite
   bool tiny, any_tiny;
   __device__ __forceinline__ PatchScale() {}
@@ -303,23 +309,93 @@ struct PatchScale {
     any_tiny = __any_sync(0xffffffffu, tiny && mx != 0);  // the FP64 products with 2^100 only where needed
     tiny = tiny && any_tiny;
     e = tiny ? 113 - __clz((int)mx) : max((int)((mx + 0x4000u) >> 20), 1);
+    subnormal = mx < 0x00100000u;
+  }
+  // the largest magnitude, in units of 2^40 (normal)
+  __device__ __forceinline__ unsigned top(unsigned mx) const {
+    return ((mx & 0xFFFFFu) | 0x100000u) >> (e - (int)(mx >> 20) + 1);
   }
   template <int M>
-  __device__ __forceinline__ void fixed(double (&r)[M], long long (&v)[M]) const {
+  __device__ __forceinline__ void fixed(double (&r)[M], long long (&v)[M], unsigned (&mag)[M]) const {
     if (any_tiny) {
 #pragma unroll
       for (int i = 0; i < M; ++i) r[i] = tiny ? r[i] * 0x1p100 : r[i];
     }
 #pragma unroll
-    for (int i = 0; i < M; ++i) v[i] = fixed_of(r[i], e);
+    for (int i = 0; i < M; ++i) v[i] = fixed_of(r[i], e, mag[i]);
   }
 };
 
-// an even / odd combination (of 55 + sh bits) as operand of SL digits
-template <int SL>
-__device__ __forceinline__ long long operand_of(long long v, int sh) {
-  if constexpr (SL == 8) return (long long)((unsigned long long)v << (8 - sh));
-  else return (v + (1ll << (sh - 1))) >> sh;
+// an even / odd combination of up to 2^(3 - sh) values as operand (63 bits and sign)
+__device__ __forceinline__ long long operand_of(long long v, int sh) { return (long long)((unsigned long long)v << sh); }
+
+// The products hold all values of a window to one absolute accuracy (2^-60 of
+// its largest in FP64; the even / odd sums in FP32 to 2^-24 of the largest of
+// the mirror images).  A result that couples to the largest value through
+// small entries only would lose relative accuracy: up to 1e3 (K = 4) and 2e4
+// (K = 8) roundings of |A||x| for one value of 1e6 among N(0,1) ones.  The
+// products of an uneven window are formed again without its spikes -- the
+// values above 2^-10 of the largest --, whose columns are added in FP64
+// (dense_spikes).  Uneven is
+// - a patch with an octant (a cell; the nodes between cells count for both)
+//   whose largest value is below 2^-7 of the patch's: residuals of a solve
+//   keep above 2^-4 in every octant, however small their values at most nodes.
+//   Largest errors above the line, in roundings of |B||r|: K = 3 26, K = 4 430, K = 5 1,500
+//   (N(0,1) values times 1e6 at the outermost corners), the local
+//   V-cycle in FP64 24, 900, 270;
+// - a cell with a mean magnitude below 1/32 of its largest (N(0,1) values: 1/4, in
+//   a corner cell 1/10; x y z 1/8).  Worst found now: K = 3 13, K = 4 42, K = 8 133 roundings of
+//   (|K| x |M| x |M| + ...) |x|; line passes 16, 60, 70 (the 1D matrices' own).
+// A window whose values above 2^-10 of its largest are more than an eighth of
+// its nodes counts as even all the same: they reach every node.  Windows of at
+// most 32 nodes are not split, have no such entries, and are not looked at.
+constexpr int kUnevenExp = 7, kUnevenCell = 32, kSpikeExp = 10;
+
+// bits of |v| in order of magnitude (FP64: the high word)
+__device__ __forceinline__ unsigned magnitude(double v) { return (unsigned)__double2hiint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ unsigned magnitude(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+// above it: a spike of a window whose largest value has the magnitude mx
+template <typename T>
+__device__ __forceinline__ unsigned spike_bound(unsigned mx) {
+  constexpr int MB = sizeof(T) == 8 ? 20 : 23;  // mantissa bits
+  return mx > (unsigned)(kSpikeExp + 1) << MB ? mx - ((unsigned)kSpikeExp << MB) : 1u << MB;
+}
+constexpr unsigned kNoSpikes = 0xFFFFFFFFu;
+
+// The magnitudes of image b of a line into the largest ones of the window's
+// octants, s_oct[side along x][image in the other directions][window]
+template <int DIM, int M>
+constexpr int octants() { return 2 * Lines<DIM, M>::IMAGES; }
+template <int DIM, int M, int P, class F>
+__device__ __forceinline__ void add_octants(const Lines<DIM, M>& ln, int b, F&& mag, unsigned (*s_oct)[P], int pn) {
+  using S = Sectors<DIM, M>;
+  constexpr int IM = Lines<DIM, M>::IMAGES;
+  unsigned lo = 0, hi = 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    if (i < S::E) lo = max(lo, mag(i));
+    if (i >= S::O) hi = max(hi, mag(i));
+  }
+  const bool cy = S::CENTRE && ln.c[0] == S::E - 1, cz = S::CENTRE && DIM == 3 && ln.c[1] == S::E - 1;
+#pragma unroll
+  for (int o = 0; o < IM; ++o) {  // a central line lies on both sides
+    const int x = o ^ b;
+    if ((x & 1) && !(cy && !(b & 1))) continue;
+    if ((x & 2) && !(cz && !(b & 2))) continue;
+    atomicMax(&s_oct[o][pn], lo);
+    atomicMax(&s_oct[IM + o][pn], hi);
+  }
+}
+
+// largest and smallest of a window's octants
+template <int N, int P>
+__device__ __forceinline__ void octant_range(const unsigned (*s_oct)[P], int pn, unsigned& lo, unsigned& hi) {
+  lo = hi = s_oct[0][pn];
+#pragma unroll
+  for (int o = 1; o < N; ++o) {
+    lo = min(lo, s_oct[o][pn]);
+    hi = max(hi, s_oct[o][pn]);
+  }
 }
 
 // y cmul 2^(ve + 64) rounded to nearest (ties away), in integer arithmetic
@@ -364,13 +440,13 @@ __device__ __forceinline__ void ldsm_t(uint32_t (&b)[4], uint32_t addr) {
                : "r"(addr));
 }
 
-constexpr int kNoExp = -(1 << 30);          // class exponent of a matrix that is not finite
+constexpr int kNoExp = -(1 << 30);          // first orbit's exponent of a matrix that is not finite
 constexpr float kMagic = 12582912.0f;       // 1.5 2^23: the accumulator's bits count integers from here
 constexpr int kMagicBits = 0x4B400000;
 
 // FP64 products of one unit: result rows of sector coefficients times the
-// operand rows, in units of 2^-52 of (table integer x operand integer) at the
-// exponent of the row's class.  Two k tiles add at most 16 products of 2^18 to an
+// operand rows, in units of 2^-68 of (table integer x operand integer) at the
+// exponent of the row's orbit.  Two k tiles add at most 16 products of 2^18 to an
 // accumulator (within its exact range of 2^22 around kMagic) before it is
 // emptied into Y.
 template <class D>
@@ -379,7 +455,7 @@ __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __res
                                           int lane) {
   constexpr int SL = D::SL, NT = D::NT, ND = 8;  // ND: digit sums kept, i + j < ND
   const int g = lane >> 2, q = lane & 3;
-  const int* shift = shifts + u.row + g;  // row exponent - its class's
+  const int* shift = shifts + u.row + g;  // row exponent - its orbit's
   const uint4* tp = table + (int64_t)u.frag * 32 + lane;
   const long long* xp = X + (u.prow + 2 * q) * D::XP + g;
   for (int k0 = 0; k0 < u.kt; k0 += 2) {
@@ -423,7 +499,7 @@ __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __res
         a = next;
       }
     }
-    // into Y: partial sums at the row's exponent, at the end rounded to the class's
+    // into Y: partial sums at the row's exponent, at the end rounded to the orbit's
     const bool last = k0 + 2 >= u.kt;
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -502,6 +578,303 @@ static __constant__ const DenseUnits<Dense<PMG_DIM, kCellM, double>::UNITS> c_ce
     dense_units<PMG_DIM, kCellM, double>();
 #endif
 
+// boundary faces of the grid (bits of edge) at node (x, y, z) of a cell
+template <int DIM, int M>
+__device__ __forceinline__ bool on_face(unsigned edge, int x, int y, int z) {
+  return (x == 0 && (edge & 1)) || (x == M - 1 && (edge & 2)) || (y == 0 && (edge & 4)) || (y == M - 1 && (edge & 8)) ||
+         (DIM == 3 && ((z == 0 && (edge & 16)) || (z == M - 1 && (edge & 32))));
+}
+
+// Part of a window's result at node i that the spikes contribute, by the
+// columns of the orbits' first nodes: the operator commutes with the
+// reflections, so the column of a mirror image is the mirrored column.
+template <int DIM, int M, typename T>
+__device__ __forceinline__ double spikes_at(const double* __restrict__ columns, const T* xw,
+                                            const unsigned short* list, int count, int i) {
+  using S = Sectors<DIM, M>;
+  const int ix = i % M, iy = (i / M) % M, iz = i / (M * M);
+  double acc = 0.0;
+#pragma unroll 4
+  for (int l = 0; l < count; ++l) {
+    const int j = list[l], jx = j % M, jy = (j / M) % M, jz = j / (M * M);
+    const bool fx = jx >= S::E, fy = jy >= S::E, fz = jz >= S::E;
+    const int orbit = (fx ? M - 1 - jx : jx) + S::E * ((fy ? M - 1 - jy : jy) + S::E * (fz ? M - 1 - jz : jz));
+    const int node = (fx ? M - 1 - ix : ix) + M * ((fy ? M - 1 - iy : iy) + M * (fz ? M - 1 - iz : iz));
+    acc += __ldg(columns + (int64_t)orbit * S::NODES + node) * (double)xw[j];
+  }
+  return acc;
+}
+
+// list of the nodes with a magnitude above bound, in order (whole block; returns after a barrier)
+template <int NODES, typename T>
+__device__ __forceinline__ int list_spikes(const T* xw, unsigned bound, unsigned short* list, int* s_count) {
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    int count = 0;
+    for (int i = 0; i < NODES; i += 32) {
+      const bool is = i + lane < NODES && magnitude(xw[min(i + lane, NODES - 1)]) > bound;
+      const unsigned mask = __ballot_sync(0xffffffffu, is);
+      if (is) list[count + __popc(mask & ((1u << lane) - 1))] = (unsigned short)(i + lane);
+      count += __popc(mask);
+    }
+    if (lane == 0) *s_count = count;
+  }
+  __syncthreads();
+  return *s_count;
+}
+
+// The spikes of a batch's uneven windows, one window after the other, added to
+// the results (whole block; its dynamic shared memory is free once the block has met).
+template <int DIM, typename T, bool CELL>
+__device__ __noinline__ void dense_spikes(const DenseJob<T>& J, uint32_t batch, const unsigned* s_spike,
+                                          const int64_t* s_base, const int* s_colour, int* s_count) {
+  constexpr int M = CELL ? kCellM : kPatchM;
+  using S = Sectors<DIM, M>;
+  using D = Dense<DIM, M, T>;
+  static_assert(D::SMEM >= S::NODES * ((int)sizeof(T) + 2), "a window and its list fit");
+  extern __shared__ __align__(16) unsigned char smraw[];
+  T* xw = reinterpret_cast<T*>(smraw);
+  unsigned short* list = reinterpret_cast<unsigned short*>(xw + S::NODES);
+  const int N1 = K * J.n + 1;
+  const int64_t N = (int64_t)N1 * N1 * (DIM == 3 ? N1 : 1);
+  const double* columns = reinterpret_cast<const double*>(reinterpret_cast<const char*>(J.table) + D::COLUMNS);
+#pragma unroll 1
+  for (int gp = 0; gp < D::P; ++gp) {
+    if (s_spike[gp] == kNoSpikes) continue;
+    __syncthreads();
+    const int edge = s_colour[gp];
+    const T* r = J.r + s_base[gp];
+    for (int i = threadIdx.x; i < S::NODES; i += blockDim.x) {
+      const int x = i % M, y = (i / M) % M, z = i / (M * M);
+      xw[i] = CELL && on_face<DIM, M>(edge, x, y, z) ? T(0) : r[x + N1 * (y + (DIM == 3 ? N1 * z : 0))];
+    }
+    __syncthreads();
+    const int count = list_spikes<S::NODES>(xw, s_spike[gp], list, s_count);
+    for (int i = threadIdx.x; i < S::NODES; i += blockDim.x) {
+      const int x = i % M, y = (i / M) % M, z = i / (M * M);
+      T* d;
+      if constexpr (CELL) d = J.dst + ((int64_t)batch * D::P + gp) * S::NODES + i;
+      else d = J.dst + (J.colour < 0 ? s_colour[gp] * N : 0) + s_base[gp] + x + N1 * (y + (DIM == 3 ? N1 * z : 0));
+      *d = (T)((double)*d + (double)J.c * spikes_at<DIM, M>(columns, xw, list, count, i));
+    }
+  }
+}
+
+// Operands and products of the windows whose first nodes are at `base` (a lane
+// holds one window): gather, even / odd combinations, results in Y.  Finds the
+// uneven windows (s_spike, s_any); AGAIN: the block's windows without spikes.
+template <int DIM, typename T, bool CELL, bool AGAIN, int NOCT>
+__device__ __forceinline__ void dense_round(const DenseJob<T>& J, int64_t base, bool active, unsigned edge,
+                                            unsigned* s_max, unsigned (*s_oct)[Dense<DIM, CELL ? kCellM : kPatchM, T>::P],
+                                            unsigned* s_spike, int* s_any) {
+  constexpr int M = CELL ? kCellM : kPatchM;
+  using S = Sectors<DIM, M>;
+  using D = Dense<DIM, M, T>;
+  using L = Lines<DIM, M>;
+  constexpr int P = D::P, NSUB = D::NSUB, NW = D::NW;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pn = lane % P, item0 = warp * NSUB + lane / P;
+  constexpr int STEP = NW * NSUB;
+  const int N1 = K * J.n + 1;
+  const T* rp = J.r + base;
+  using XT = std::conditional_t<D::F64, long long, uint16_t>;
+  using YT = std::conditional_t<D::F64, long long, float>;
+  XT* X = reinterpret_cast<XT*>(smraw);
+  YT* Y = reinterpret_cast<YT*>(smraw + D::YOFF);
+  PatchScale sc;  // FP64
+  const int* orbitexp = reinterpret_cast<const int*>(J.table + D::FRAGS) + S::ROWS;
+  if constexpr (D::F64) {
+      double* R = reinterpret_cast<double*>(Y);
+    unsigned mx = 0;
+    for (int l = item0; l < S::NODES / S::M; l += STEP) {
+      const int ly = DIM == 3 ? l % M : l, lz = DIM == 3 ? l / M : 0;
+      const double* q = rp + N1 * (ly + N1 * lz);
+      const bool in = active && !(CELL && (((edge & 4) && ly == 0) || ((edge & 8) && ly == M - 1) ||
+                                           (DIM == 3 && (((edge & 16) && lz == 0) || ((edge & 32) && lz == M - 1)))));
+      double v[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+        v[i] = in && !(CELL && ((i == 0 && (edge & 1)) || (i == M - 1 && (edge & 2)))) ? q[i] : 0.0;
+      if constexpr (AGAIN) {
+#pragma unroll
+        for (int i = 0; i < M; ++i) v[i] = magnitude(v[i]) > s_spike[pn] ? 0.0 : v[i];
+      }
+#pragma unroll
+      for (int i = 0; i < S::M; ++i) {
+        R[(l * S::M + i) * P + pn] = v[i];
+        // the low bit: a value below the high word's range is not zero
+        mx = max(mx, magnitude(v[i]) | (__double2loint(v[i]) != 0));
+      }
+    }
+#pragma unroll
+    for (int o = P; o < 32; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane < P) atomicMax(&s_max[pn], mx);
+    __syncthreads();
+    sc = PatchScale(s_max[pn], J.cmul == 0 || orbitexp[0] == kNoExp);
+  }
+  // even / odd combinations, stored as operands
+  unsigned sum = 0;  // cells: of the magnitudes, in units of 2^40
+  for (int l = item0; l < L::N; l += STEP) {
+    const L ln(l);
+    if constexpr (D::F64) {
+      const double* R = reinterpret_cast<const double*>(Y);
+      long long v[L::IMAGES][M];
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b) {
+        const double* q = R + ln.node(b, M) * P + pn;
+        double r[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) r[i] = ln.has(b) || !S::SPLIT ? q[i * P] : 0.0;
+        unsigned mag[M];
+        sc.template fixed<M>(r, v[b], mag);
+        if constexpr (S::SPLIT && CELL) {
+#pragma unroll
+          for (int i = 0; i < M; ++i) sum += mag[i] >> 8;
+        }
+        if constexpr (NOCT > 1 && !AGAIN) add_octants(ln, b, [&](int i) { return mag[i]; }, s_oct, pn);
+      }
+      reflect<DIM, M>(v);
+      const int sh0 = (S::SPLIT ? 3 - DIM : 3) + ln.centres();  // 2^(d-c) images were summed
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b)
+        if (ln.has(b) || !S::SPLIT)
+          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
+            X[(S::prow(s) + ox + ln.coef(s)) * D::XP + pn] =
+                operand_of(v[b][i], S::CENTRE && i == S::E - 1 ? sh0 + 1 : sh0);
+          });
+    } else {
+      float v[L::IMAGES][M];
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b) {
+        const float* q = rp + ln.node(b, N1);
+        const bool in = active && (ln.has(b) || !S::SPLIT);
+#pragma unroll
+        for (int i = 0; i < M; ++i) v[b][i] = in ? q[i] : 0.f;
+      }
+      if constexpr (NOCT > 1) {
+        if constexpr (AGAIN) {
+#pragma unroll
+          for (int b = 0; b < L::IMAGES; ++b)
+#pragma unroll
+            for (int i = 0; i < M; ++i) v[b][i] = magnitude(v[b][i]) > s_spike[pn] ? 0.f : v[b][i];
+        } else {
+#pragma unroll
+          for (int b = 0; b < L::IMAGES; ++b)
+            add_octants(ln, b, [&](int i) { return magnitude(v[b][i]); }, s_oct, pn);
+        }
+      }
+      reflect<DIM, M>(v);
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b)
+        if (ln.has(b) || !S::SPLIT)
+          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
+            XT* x = X + (S::prow(s) + ox + ln.coef(s)) * D::XP + pn;
+            const uint32_t b1 = __float_as_uint(v[b][i]);
+            const float f2 = v[b][i] - __uint_as_float(b1 & 0xFFFF0000u);
+            const uint32_t b2 = __float_as_uint(f2);
+            const float f3 = f2 - __uint_as_float(b2 & 0xFFFF0000u);
+            x[0] = (uint16_t)(b1 >> 16);
+            x[S::PROWS * D::XP] = (uint16_t)(b2 >> 16);
+            x[2 * S::PROWS * D::XP] = (uint16_t)(__float_as_uint(f3) >> 16);
+          });
+    }
+  }
+  // integers throughout, so that the choice does not depend on the batch
+  if constexpr (S::SPLIT && CELL) {
+    if constexpr (!AGAIN) {
+#pragma unroll
+      for (int o = P; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane < P) atomicAdd(&s_oct[0][pn], sum);
+    }
+  }
+  __syncthreads();
+  if (S::SPLIT && !AGAIN && threadIdx.x < P) {
+    unsigned mx = s_max[pn];
+    bool uneven;
+    if constexpr (CELL) {
+      uneven = !sc.bad && !sc.subnormal &&
+               (unsigned long long)s_oct[0][pn] * kUnevenCell < (unsigned long long)sc.top(mx) * S::NODES;
+    } else {
+      unsigned lo, hi;
+      octant_range<NOCT>(s_oct, pn, lo, hi);
+      if constexpr (D::F64) {
+        uneven = !sc.bad && !sc.subnormal && lo < hi >> kUnevenExp;
+      } else {
+        mx = hi;
+        uneven = hi < 0x7F800000u && hi > (unsigned)(kUnevenExp + 1) << 23 && lo < hi - ((unsigned)kUnevenExp << 23);
+      }
+    }
+    if (uneven) {
+      s_spike[pn] = spike_bound<T>(mx);
+      *s_any = 1;
+    }
+  }
+  if constexpr (D::F64) {
+    for (int u = warp; u < D::UNITS; u += NW) {
+#if PMG_PREC == 0
+      dense_mma<D>(CELL ? c_cell_units.u[CELL ? u : 0] : c_units.u[CELL ? 0 : u], J.table, orbitexp - S::ROWS, X, Y, lane);
+#endif
+    }
+    __syncthreads();
+  } else {
+    float y[D::UPW][D::NT][4];
+#pragma unroll
+    for (int i = 0; i < D::UPW; ++i)
+      if (warp + i * NW < D::UNITS) dense_mma<D>(c_units.u[warp + i * NW], J.table, X, y[i], lane);
+    __syncthreads();  // the results take the operands' place
+    if (S::SPLIT && !AGAIN && *s_any) return;  // not needed
+#pragma unroll
+    for (int i = 0; i < D::UPW; ++i)
+      if (warp + i * NW < D::UNITS) {
+        const DenseUnit& u = c_units.u[warp + i * NW];
+#pragma unroll
+        for (int t = 0; t < D::NT; ++t)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int rr = (lane >> 2) + 8 * h;
+            if (rr < u.valid)
+              *reinterpret_cast<float2*>(Y + (u.row + rr) * D::YP + 8 * t + 2 * (lane & 3)) =
+                  make_float2(y[i][t][2 * h], y[i][t][2 * h + 1]);
+          }
+      }
+    __syncthreads();
+  }
+}
+
+// The second round.  A window with more spikes than an eighth of its nodes
+// keeps them (kNoSpikes): its large values reach every node.
+template <int DIM, typename T, bool CELL, int NOCT>
+__device__ __noinline__ void dense_again(const DenseJob<T>& J, const int64_t* s_base, const int* s_colour,
+                                         unsigned* s_max,
+                                         unsigned (*s_oct)[Dense<DIM, CELL ? kCellM : kPatchM, T>::P],
+                                         unsigned* s_spike, int* s_any) {
+  constexpr int P = Dense<DIM, CELL ? kCellM : kPatchM, T>::P;
+  constexpr int M = CELL ? kCellM : kPatchM, NODES = ipow(M, DIM);
+  const int pn = (threadIdx.x & 31) % P, N1 = K * J.n + 1;
+  if (threadIdx.x < P) s_oct[0][pn] = 0;
+  __syncthreads();
+  const int64_t base = s_base[pn];
+  const unsigned bound = s_spike[pn];
+  if (bound != kNoSpikes) {
+    unsigned count = 0;
+    for (int i = threadIdx.x / P; i < NODES; i += blockDim.x / P) {
+      const int x = i % M, y = (i / M) % M, z = i / (M * M);
+      const T v = J.r[base + x + N1 * (y + (DIM == 3 ? N1 * z : 0))];
+      count += magnitude(v) > bound && !(CELL && on_face<DIM, M>(s_colour[pn], x, y, z));
+    }
+    atomicAdd(&s_oct[0][pn], count);
+  }
+  __syncthreads();
+  if (threadIdx.x < P && s_oct[0][pn] > NODES / 8) s_spike[pn] = kNoSpikes;
+  __syncthreads();
+  if (!__syncthreads_or(s_spike[pn] != kNoSpikes) && sizeof(T) == 8) return;  // the first round's results stand
+  if (threadIdx.x < P) s_max[pn] = 0;
+  __syncthreads();
+  dense_round<DIM, T, CELL, true, NOCT>(J, base < 0 ? 0 : base, base >= 0, CELL ? (unsigned)s_colour[pn] : 0, s_max, s_oct,
+                                        s_spike, s_any);
+}
+
 // The patches of batch `batch` of a level: gather r_j, even / odd
 // combinations, products, and back; omega_AS d_j to the colour's vector
 // (additive) or d_j added to u (multiplicative).  A lane holds one patch (P
@@ -520,7 +893,10 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int64_t s_base[P];
   __shared__ int s_colour[P];
-  __shared__ unsigned s_max[P];
+  constexpr int NOCT = S::SPLIT && !CELL ? octants<DIM, M>() : 1;
+  __shared__ unsigned s_max[P], s_oct[NOCT][P];  // magnitudes: largest; octants', or (cells) the sum
+  __shared__ unsigned s_spike[P];  // magnitude above which a value is a spike
+  __shared__ int s_any, s_count;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int pn = lane % P, item0 = warp * NSUB + lane / P;
   constexpr int STEP = NW * NSUB;
@@ -548,11 +924,14 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     if (DIM == 3) base += (int64_t)N1 * N1 * (K * (v[2] - o) + o);
     if (threadIdx.x < P) {
       s_base[pn] = active ? base : -1;
-      s_colour[pn] = J.colour < 0 ? (v[0] & 1) | ((v[1] & 1) << 1) | (DIM == 3 ? (v[2] & 1) << 2 : 0) : 0;
+      s_colour[pn] = CELL ? (int)edge : J.colour < 0 ? (v[0] & 1) | ((v[1] & 1) << 1) | (DIM == 3 ? (v[2] & 1) << 2 : 0) : 0;
       s_max[pn] = 0;
+#pragma unroll
+      for (int o = 0; o < NOCT; ++o) s_oct[o][pn] = 0;
+      s_spike[pn] = kNoSpikes;
     }
+    if (threadIdx.x == 0) s_any = 0;
   }
-  const T* rp = J.r + base;
   using L = Lines<DIM, M>;
   using XT = std::conditional_t<D::F64, long long, uint16_t>;
   using YT = std::conditional_t<D::F64, long long, float>;
@@ -572,111 +951,14 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
         }
     }
   }
+  __syncthreads();  // the shared arrays
+  dense_round<DIM, T, CELL, false, NOCT>(J, base, active, edge, s_max, s_oct, s_spike, &s_any);
+  if constexpr (S::SPLIT) {
+    if (s_any) dense_again<DIM, T, CELL, NOCT>(J, s_base, s_colour, s_max, s_oct, s_spike, &s_any);
+  }
+  const int* orbitexp = reinterpret_cast<const int*>(J.table + D::FRAGS) + S::ROWS;
   PatchScale sc;  // FP64
-  const int* classexp = reinterpret_cast<const int*>(J.table + D::FRAGS) + S::ROWS;
-  if constexpr (D::F64) {
-    __syncthreads();  // s_max
-    double* R = reinterpret_cast<double*>(Y);
-    unsigned mx = 0;
-    for (int l = item0; l < S::NODES / S::M; l += STEP) {
-      const int ly = DIM == 3 ? l % M : l, lz = DIM == 3 ? l / M : 0;
-      const double* q = rp + N1 * (ly + N1 * lz);
-      const bool in = active && !(CELL && (((edge & 4) && ly == 0) || ((edge & 8) && ly == M - 1) ||
-                                           (DIM == 3 && (((edge & 16) && lz == 0) || ((edge & 32) && lz == M - 1)))));
-      double v[M];
-#pragma unroll
-      for (int i = 0; i < M; ++i)
-        v[i] = in && !(CELL && ((i == 0 && (edge & 1)) || (i == M - 1 && (edge & 2)))) ? q[i] : 0.0;
-#pragma unroll
-      for (int i = 0; i < S::M; ++i) {
-        R[(l * S::M + i) * P + pn] = v[i];
-        // the low bit: a value below the high word's range is not zero
-        mx = max(mx, ((unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu) | (__double2loint(v[i]) != 0));
-      }
-    }
-#pragma unroll
-    for (int o = P; o < 32; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane < P) atomicMax(&s_max[pn], mx);
-    __syncthreads();
-    sc = PatchScale(s_max[pn], J.cmul == 0 || classexp[0] == kNoExp);
-  }
-  // even / odd combinations, stored as operands
-  for (int l = item0; l < L::N; l += STEP) {
-    const L ln(l);
-    if constexpr (D::F64) {
-      const double* R = reinterpret_cast<const double*>(Y);
-      long long v[L::IMAGES][S::M];
-#pragma unroll
-      for (int b = 0; b < L::IMAGES; ++b) {
-        const double* q = R + ln.node(b, S::M) * P + pn;
-        double r[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) r[i] = ln.has(b) || !S::SPLIT ? q[i * P] : 0.0;
-        sc.template fixed<M>(r, v[b]);
-      }
-      reflect<DIM, M>(v);
-      const int sh0 = (S::SPLIT ? DIM + 3 : 3) - ln.centres();  // to 55 bits and sign: 2^(d-c) images were summed
-#pragma unroll
-      for (int b = 0; b < L::IMAGES; ++b)
-        if (ln.has(b) || !S::SPLIT)
-          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
-            X[(S::prow(s) + ox + ln.coef(s)) * D::XP + pn] =
-                operand_of<D::SL>(v[b][i], S::CENTRE && i == S::E - 1 ? sh0 - 1 : sh0);
-          });
-    } else {
-      float v[L::IMAGES][S::M];
-#pragma unroll
-      for (int b = 0; b < L::IMAGES; ++b) {
-        const float* q = rp + ln.node(b, N1);
-        const bool in = active && (ln.has(b) || !S::SPLIT);
-#pragma unroll
-        for (int i = 0; i < S::M; ++i) v[b][i] = in ? q[i] : 0.f;
-      }
-      reflect<DIM, M>(v);
-#pragma unroll
-      for (int b = 0; b < L::IMAGES; ++b)
-        if (ln.has(b) || !S::SPLIT)
-          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
-            XT* x = X + (S::prow(s) + ox + ln.coef(s)) * D::XP + pn;
-            const uint32_t b1 = __float_as_uint(v[b][i]);
-            const float f2 = v[b][i] - __uint_as_float(b1 & 0xFFFF0000u);
-            const uint32_t b2 = __float_as_uint(f2);
-            const float f3 = f2 - __uint_as_float(b2 & 0xFFFF0000u);
-            x[0] = (uint16_t)(b1 >> 16);
-            x[S::PROWS * D::XP] = (uint16_t)(b2 >> 16);
-            x[2 * S::PROWS * D::XP] = (uint16_t)(__float_as_uint(f3) >> 16);
-          });
-    }
-  }
-  __syncthreads();
-  if constexpr (D::F64) {
-    for (int u = warp; u < D::UNITS; u += NW) {
-#if PMG_PREC == 0
-      dense_mma<D>(CELL ? c_cell_units.u[CELL ? u : 0] : c_units.u[CELL ? 0 : u], J.table, classexp - S::ROWS, X, Y, lane);
-#endif
-    }
-  } else {
-    float y[D::UPW][D::NT][4];
-#pragma unroll
-    for (int i = 0; i < D::UPW; ++i)
-      if (warp + i * NW < D::UNITS) dense_mma<D>(c_units.u[warp + i * NW], J.table, X, y[i], lane);
-    __syncthreads();  // the results take the operands' place
-#pragma unroll
-    for (int i = 0; i < D::UPW; ++i)
-      if (warp + i * NW < D::UNITS) {
-        const DenseUnit& u = c_units.u[warp + i * NW];
-#pragma unroll
-        for (int t = 0; t < D::NT; ++t)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int rr = (lane >> 2) + 8 * h;
-            if (rr < u.valid)
-              *reinterpret_cast<float2*>(Y + (u.row + rr) * D::YP + 8 * t + 2 * (lane & 3)) =
-                  make_float2(y[i][t][2 * h], y[i][t][2 * h + 1]);
-          }
-      }
-  }
-  __syncthreads();
+  if constexpr (D::F64) sc = PatchScale(s_max[pn], J.cmul == 0 || orbitexp[0] == kNoExp);
   // back to the nodes
   for (int l = item0; l < L::N; l += STEP) {
     const L ln(l);
@@ -693,12 +975,12 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     for (int b = 0; b < L::IMAGES; ++b)
       if (ln.has(b) || !S::SPLIT) {
         T* z = Z + pn * D::ZP + ln.node(b, S::M);
-        const int ve = D::F64 ? J.vexp + sc.e - (sc.tiny ? 100 : 0) : 0, nc = ln.centres();
-        const int ve0 = D::F64 ? ve - __ldg(classexp + nc) : 0, ve1 = D::F64 ? ve - __ldg(classexp + nc + 1) : 0;
+        const int ve = D::F64 ? J.vexp + sc.e - (sc.tiny ? 100 : 0) : 0;
 #pragma unroll
         for (int i = 0; i < S::M; ++i) {
           if constexpr (D::F64)
-            z[i] = sc.bad ? __longlong_as_double(0x7FF8000000000000ll) : double_of(v[b][i], J.cmul, S::CENTRE && i == S::E - 1 ? ve1 : ve0);
+            z[i] = sc.bad ? __longlong_as_double(0x7FF8000000000000ll)
+                          : double_of(v[b][i], J.cmul, ve - __ldg(orbitexp + S::E * l + (i < S::E ? i : M - 1 - i)));
           else
             z[i] = J.c * v[b][i];
         }
@@ -712,6 +994,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
       const int gp = i / S::NODES;
       o[i] = Z[gp * D::ZP + i - gp * S::NODES];
     }
+    if (S::SPLIT && s_any) dense_spikes<DIM, T, true>(J, batch, s_spike, s_base, s_colour, &s_count);
     return;
   }
   // a warp writes a patch; each lane keeps the offsets of its nodes
@@ -737,6 +1020,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
         if (lane + 32 * j < S::NODES) o[off[j]] += z[32 * j];
     }
   }
+  if (S::SPLIT && s_any) dense_spikes<DIM, T, false>(J, batch, s_spike, s_base, s_colour, &s_count);
 }
 
 template <int DIM, typename T>
@@ -874,13 +1158,15 @@ struct Stage {
   using S = Sectors<DIM, kPatchM>;
   static constexpr int P = D::P;
   static constexpr int64_t XWORDS = (int64_t)S::ROWS * P, YWORDS = XWORDS;  // per batch
-  static constexpr int64_t BYTES = 8 * (XWORDS + YWORDS) + 4 * P;          // and the patches' exponents
+  static constexpr int64_t BYTES = 8 * (XWORDS + YWORDS) + 8 * P;          // and two words per patch
   static constexpr int MAXT = S::tiles(0);
   static constexpr int XSM = 16 * MAXT * D::XP * 8, YSM = S::size(0) * P * 8;  // products: one sector
   static constexpr int MP2 = kPatchM * kPatchM, ZP = (2 * MP2) | 1, ZSM = P * ZP * 8;  // merge: two planes
+  static_assert(ZSM >= 10 * S::NODES, "or a window and its list of spikes");
 };
 
-// exponent word of a patch: bits 0-11 the exponent bound, 12 tiny, 13 bad
+// exponent word of a patch: bits 0-11 the exponent bound, 12 tiny, 13 bad;
+// the words are followed by the patches' spike bounds (kNoSpikes: even)
 struct PatchOrigin {
   int64_t base;
   int colour;
@@ -901,7 +1187,7 @@ __device__ __forceinline__ PatchOrigin patch_origin(const DenseJob<double>& J, u
   return o;
 }
 
-// X [row][P] and the exponent words of batch first + blockIdx.x
+// X [row][P] and the words of batch first + blockIdx.x
 template <int DIM>
 __global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant__ DenseJob<double> J, uint32_t first,
                                                           long long* __restrict__ X, int* __restrict__ words) {
@@ -909,54 +1195,100 @@ __global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant_
   using S = Sectors<DIM, M>;
   using L = Lines<DIM, M>;
   constexpr int P = Stage<DIM>::P;
-  __shared__ unsigned s_max[P];
+  constexpr int NOCT = octants<DIM, M>();
+  __shared__ unsigned s_max[P], s_oct[NOCT][P], s_spike[P];
+  __shared__ int s_any;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pn = lane % P, item0 = warp * (32 / P) + lane / P;
   constexpr int STEP = 8 * (32 / P);
   const int N1 = K * J.n + 1;
   const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + pn);
   const double* rp = J.r + o.base;
-  const int* classexp = reinterpret_cast<const int*>(J.table + Stage<DIM>::D::FRAGS) + S::ROWS;
+  const int* orbitexp = reinterpret_cast<const int*>(J.table + Stage<DIM>::D::FRAGS) + S::ROWS;
   X += blockIdx.x * Stage<DIM>::XWORDS;
-  if (threadIdx.x < P) s_max[threadIdx.x] = 0;
-  __syncthreads();
-  unsigned mx = 0;
-  for (int l = item0; l < M * M; l += STEP) {
-    const double* q = rp + N1 * (l % M + N1 * (l / M));
-    double v[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) v[i] = o.active ? q[i] : 0.0;
-#pragma unroll
-    for (int i = 0; i < M; ++i)
-      mx = max(mx, ((unsigned)__double2hiint(v[i]) & 0x7FFFFFFFu) | (__double2loint(v[i]) != 0));
+  words += blockIdx.x * 2 * P;
+  if (threadIdx.x < P) {
+    s_max[threadIdx.x] = 0;
+    for (int i = 0; i < NOCT; ++i) s_oct[i][threadIdx.x] = 0;
+    s_spike[threadIdx.x] = kNoSpikes;
   }
-#pragma unroll
-  for (int w = P; w < 32; w <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-  if (lane < P) atomicMax(&s_max[pn], mx);
+  if (threadIdx.x == 0) s_any = 0;
   __syncthreads();
-  mx = s_max[pn];
-  const PatchScale sc(mx, J.cmul == 0 || classexp[0] == kNoExp);
-  if (threadIdx.x < P) words[blockIdx.x * P + pn] = sc.e | (sc.tiny ? 1 << 12 : 0) | (sc.bad ? 1 << 13 : 0);
-  for (int l = item0; l < L::N; l += STEP) {
-    const L ln(l);
-    long long v[L::IMAGES][M];
+#pragma unroll 1
+  for (int round = 0;; ++round) {  // as in dense_body
+    const unsigned bound = s_spike[pn];
+    unsigned mx = 0;
+    for (int l = item0; l < M * M; l += STEP) {
+      const double* q = rp + N1 * (l % M + N1 * (l / M));
+      double v[M];
 #pragma unroll
-    for (int b = 0; b < L::IMAGES; ++b) {
-      const double* q = rp + ln.node(b, N1);
-      const bool in = o.active && ln.has(b);
-      double r[M];
+      for (int i = 0; i < M; ++i) v[i] = o.active ? q[i] : 0.0;
 #pragma unroll
-      for (int i = 0; i < M; ++i) r[i] = in ? q[i] : 0.0;
-      sc.template fixed<M>(r, v[b]);
+      for (int i = 0; i < M; ++i) {
+        const unsigned m = magnitude(v[i]);
+        mx = max(mx, m > bound ? 0 : m | (__double2loint(v[i]) != 0));
+      }
     }
-    reflect<DIM, M>(v);
-    const int sh0 = DIM + 3 - ln.centres();
 #pragma unroll
-    for (int b = 0; b < L::IMAGES; ++b)
-      if (ln.has(b))
-        for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
-          X[(S::row(s) + ox + ln.coef(s)) * P + pn] =
-              operand_of<Stage<DIM>::D::SL>(v[b][i], S::CENTRE && i == S::E - 1 ? sh0 - 1 : sh0);
-        });
+    for (int w = P; w < 32; w <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+    if (lane < P) atomicMax(&s_max[pn], mx);
+    __syncthreads();
+    mx = s_max[pn];
+    const PatchScale sc(mx, J.cmul == 0 || orbitexp[0] == kNoExp);
+    for (int l = item0; l < L::N; l += STEP) {
+      const L ln(l);
+      long long v[L::IMAGES][M];
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b) {
+        const double* q = rp + ln.node(b, N1);
+        const bool in = o.active && ln.has(b);
+        double r[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) r[i] = in ? q[i] : 0.0;
+        if (round) {
+#pragma unroll
+          for (int i = 0; i < M; ++i) r[i] = magnitude(r[i]) > bound ? 0.0 : r[i];
+        }
+        unsigned mag[M];
+        sc.template fixed<M>(r, v[b], mag);
+        if (round == 0) add_octants(ln, b, [&](int i) { return mag[i]; }, s_oct, pn);
+      }
+      reflect<DIM, M>(v);
+      const int sh0 = 3 - DIM + ln.centres();
+#pragma unroll
+      for (int b = 0; b < L::IMAGES; ++b)
+        if (ln.has(b))
+          for_coefs<DIM, M>(b, [&](int i, int s, int ox) {
+            X[(S::row(s) + ox + ln.coef(s)) * P + pn] =
+                operand_of(v[b][i], S::CENTRE && i == S::E - 1 ? sh0 + 1 : sh0);
+          });
+    }
+    __syncthreads();
+    if (threadIdx.x < P) {
+      unsigned lo, hi;
+      octant_range<NOCT>(s_oct, pn, lo, hi);
+      if (round == 0 && !sc.bad && !sc.subnormal && lo < hi >> kUnevenExp) {
+        s_spike[pn] = spike_bound<double>(mx);
+        s_any = 1;
+      }
+      s_max[pn] = s_oct[0][pn] = 0;
+      words[pn] = sc.e | (sc.tiny ? 1 << 12 : 0) | (sc.bad ? 1 << 13 : 0);
+      words[P + pn] = (int)s_spike[pn];
+    }
+    __syncthreads();
+    if (round || !s_any) break;
+    if (s_spike[pn] != kNoSpikes) {  // as dense_again
+      unsigned count = 0;
+      for (int i = threadIdx.x / P; i < S::NODES; i += 256 / P)
+        count += magnitude(rp[i % M + N1 * (i / M % M + N1 * (i / (M * M)))]) > s_spike[pn];
+      atomicAdd(&s_oct[0][pn], count);
+    }
+    __syncthreads();
+    if (threadIdx.x < P) {
+      if (s_oct[0][pn] > S::NODES / 8) s_spike[pn] = kNoSpikes;
+      words[P + pn] = (int)s_spike[pn];
+    }
+    __syncthreads();
+    if (!__syncthreads_or(s_spike[pn] != kNoSpikes)) break;
   }
 }
 
@@ -1006,8 +1338,10 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
   double* Z = reinterpret_cast<double*>(smraw);
   const int pn = threadIdx.x % P, cz = blockIdx.y;
   const int N1 = K * J.n + 1;
-  const int* classexp = reinterpret_cast<const int*>(J.table + St::D::FRAGS) + S::ROWS;
-  const int word = words[blockIdx.x * P + pn];
+  const int* orbitexp = reinterpret_cast<const int*>(J.table + St::D::FRAGS) + S::ROWS;
+  __shared__ int s_count;
+  words += blockIdx.x * 2 * P;
+  const int word = words[pn];
   const int ve = J.vexp + (word & 0xFFF) - (word & (1 << 12) ? 100 : 0);
   Y += blockIdx.x * St::YWORDS;
   for (int cy = threadIdx.x / P; cy < S::E; cy += 128 / P) {
@@ -1021,7 +1355,7 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
       });
     }
     reflect<DIM, M>(v);
-    const int nc = ln.centres(), ve0 = ve - __ldg(classexp + nc), ve1 = ve - __ldg(classexp + nc + 1);
+    const int* oe = orbitexp + S::E * (cy + S::E * cz);
 #pragma unroll
     for (int b = 0; b < L::IMAGES; ++b)
       if (ln.has(b)) {
@@ -1029,10 +1363,10 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
 #pragma unroll
         for (int i = 0; i < M; ++i)
           z[i] = word & (1 << 13) ? __longlong_as_double(0x7FF8000000000000ll)
-                                  : double_of(v[b][i], J.cmul, S::CENTRE && i == S::E - 1 ? ve1 : ve0);
+                                  : double_of(v[b][i], J.cmul, ve - __ldg(oe + (i < S::E ? i : M - 1 - i)));
       }
   }
-  __syncthreads();
+  const bool any = __syncthreads_or((unsigned)words[P + pn] != kNoSpikes);
   const int64_t N = (int64_t)N1 * N1 * N1;
   const int planes = cz == S::E - 1 ? 1 : 2;
   for (int gp = threadIdx.x >> 5; gp < P; gp += 4) {
@@ -1043,6 +1377,25 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
       double* d = J.dst + (J.colour < 0 ? o.colour * N : 0) + o.base + ix + N1 * (r + N1 * iz);
       if (J.colour < 0) *d = Z[gp * ZP + i];
       else *d += Z[gp * ZP + i];  // one patch of the colour per node
+    }
+  }
+  if (!any) return;
+  // the spikes' part of this block's planes of the uneven patches
+  const double* columns = reinterpret_cast<const double*>(reinterpret_cast<const char*>(J.table) + St::D::COLUMNS);
+  unsigned short* list = reinterpret_cast<unsigned short*>(Z + S::NODES);
+#pragma unroll 1
+  for (int gp = 0; gp < P; ++gp) {
+    const unsigned bound = (unsigned)words[P + gp];
+    if (bound == kNoSpikes) continue;
+    const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + gp);
+    __syncthreads();
+    for (int i = threadIdx.x; i < S::NODES; i += 128) Z[i] = J.r[o.base + i % M + N1 * (i / M % M + N1 * (i / MP2))];
+    __syncthreads();
+    const int count = list_spikes<S::NODES>(Z, bound, list, &s_count);
+    for (int i = threadIdx.x; i < planes * MP2; i += 128) {
+      const int pl = i >= MP2, q = i - pl * MP2, iz = pl ? M - 1 - cz : cz;
+      J.dst[(J.colour < 0 ? o.colour * N : 0) + o.base + q % M + N1 * (q / M + N1 * iz)] +=
+          J.c * spikes_at<DIM, M>(columns, Z, list, count, q + MP2 * iz);
     }
   }
 }
@@ -1079,13 +1432,14 @@ __global__ void __launch_bounds__(256) patch_point_group_kernel(const __grid_con
 // ---------------------------------------------------------------- the matrix
 // Columns of B at unit scale (the FP64 part serves both precisions): the local
 // solver applied to the unit vectors of the orbits' first nodes, one node per
-// patch of the block; out[column][node].  A further local cycle (Algorithm 2,
-// N_iter > 1) continues from out.  For FP64 products V = dd: the matrix is
+// patch of the block; column[orbit][node], hi + lo.  A further local cycle (Algorithm 2,
+// N_iter > 1) continues from them.  For FP64 products V = dd: the matrix is
 // rounded once, where the local solver in plain FP64 would leave 2-5 times
 // the error of a solve in the products (K = 3: 1.1e-15 against 3.3e-16).
 template <int DIM, typename V>
-__global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__ out, int np, bool first,
-                                                            const double* __restrict__ dinv, PatchParams<double> H) {
+__global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__ hi, double* __restrict__ lo, int np,
+                                                            bool first, const double* __restrict__ dinv,
+                                                            PatchParams<double> H) {
   using S = Sectors<DIM, kPatchM>;
   using PS = PatchShape<DIM>;
   constexpr int SZT = PS::SZT, RT = PS::off_r(PS::L - 1), DT = PS::off_d(PS::L - 1);
@@ -1101,9 +1455,13 @@ __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__
   P.half = H.half;
   P.colour = H.colour;
   const CartGeo<DIM, V> geo{dinv, P.scale, P.inv_scale, P.inv_a0};
+  auto value = [&](int64_t t) {
+    if constexpr (sizeof(V) == 16) return V(hi[t], lo[t]);
+    else return V(hi[t]);
+  };
   pfor<SZT>(pb, [&](int g, int i) {
     pb.at(g)[RT + i] = V(i == Orbit<DIM, kPatchM>(c0 + g).node(0) ? 1.0 : 0.0);
-    if (!first) pb.at(g)[DT + i] = V(out[(int64_t)(c0 + g) * SZT + i]);
+    if (!first) pb.at(g)[DT + i] = value((int64_t)(c0 + g) * SZT + i);
   });
   __syncthreads();
   if constexpr (PS::L > 1) {
@@ -1111,10 +1469,41 @@ __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__
   }
   pvcycle<DIM, PS::L - 1>(pb, geo, P);
   pfor<SZT>(pb, [&](int g, int i) {
-    double& o = out[(int64_t)(c0 + g) * SZT + i];
-    const V d = pb.at(g)[DT + i];
-    o = first ? value_of(d) : value_of(V(o) + d);
+    const int64_t t = (int64_t)(c0 + g) * SZT + i;
+    V d = pb.at(g)[DT + i];
+    if (!first) d = value(t) + d;
+    if constexpr (sizeof(V) == 16) {
+      const double v = value_of(d);
+      lo[t] = (d.hi - v) + d.lo;
+      hi[t] = v;
+    } else {
+      hi[t] = d;
+      lo[t] = 0.0;
+    }
   });
+}
+
+// Columns of the element stiffness matrix of Eq. (3) at unit scale, from the
+// 1D element matrices; as patch_columns_kernel
+template <int DIM>
+__global__ void __launch_bounds__(256) cell_columns_kernel(double* __restrict__ hi, double* __restrict__ lo) {
+  constexpr int M = kCellM;
+  using S = Sectors<DIM, M>;
+  const int t = blockIdx.x * 256 + threadIdx.x;
+  if (t >= S::ORBITS * S::NODES) return;
+  const Orbit<DIM, M> o(t / S::NODES);
+  const int i = t % S::NODES, c[3] = {i % M, (i / M) % M, i / (M * M)};
+  dd acc(0.0);
+#pragma unroll
+  for (int d = 0; d < DIM; ++d) {
+    dd p(1.0);
+#pragma unroll
+    for (int e = 0; e < DIM; ++e) p = c_coef64[(d == e ? LAY.Ke : LAY.Me) + c[e] * M + o.c[e]] * p;
+    acc += p;
+  }
+  const double v = value_of(acc);
+  hi[t] = v;
+  lo[t] = (acc.hi - v) + acc.lo;
 }
 
 // coefficient k of sector s: its orbit
@@ -1125,24 +1514,36 @@ __device__ __forceinline__ Orbit<DIM, M> orbit_of(int s, int k) {
   return Orbit<DIM, M>(k % e0 + S::E * ((k / e0) % e1 + S::E * (k / (e0 * e1))));
 }
 
-// Sector matrices, one warp per row: the entry of row m and coefficient j is
-// the signed sum over the mirror images of m's node of the operator's entry
-// for j's node, over 2^d -- the operand of an orbit with c central
-// coordinates, which has only 2^(d-c) images, counts 2^c times.  Patch: from
-// the columns; cell: from the 1D element matrices (coef: the coefficient
-// block), in pairs of doubles.
-// rowexp: the largest exponent x with entry 2^x below 0.98 2^55 (7 signed
-// digits reach 127/128 of 2^55) and the row's sum of magnitudes times 2^x
-// below 2^57 (8 digits: 2^63, 2^65; results and their even / odd sums stay within 64 bits).  The
+// Entry of row om and coefficient oj of sector s: the signed sum over the
+// mirror images of om's node of the operator's entry for oj's node, over 2^d
+// -- the operand of an orbit with c central coordinates, which has only
+// 2^(d-c) images, counts 2^c times.
+template <int DIM, int M>
+__device__ __forceinline__ dd sector_entry(const double* __restrict__ hi, const double* __restrict__ lo, int s,
+                                           const Orbit<DIM, M>& om, const Orbit<DIM, M>& oj) {
+  using S = Sectors<DIM, M>;
+  const int64_t col = (int64_t)(oj.c[0] + S::E * (oj.c[1] + S::E * oj.c[2])) * S::NODES;
+  dd a(0.0);
+#pragma unroll
+  for (int b = 0; b < S::IMAGES; ++b) {
+    if (S::IMAGES > 1 && !oj.has(b)) continue;
+    const int64_t t = col + om.node(b);
+    const double sg = (__popc(s & b) & 1) ? -1.0 / S::IMAGES : 1.0 / S::IMAGES;
+    a += dd(sg * hi[t], sg * lo[t]);
+  }
+  return a;
+}
+
+// Exponents of the sector matrices, one warp per row.
+// rowexp: the largest exponent x with entry 2^x below 0.98 2^63 (8 signed
+// digits reach 127/128 of 2^63) and the row's sum of magnitudes times 2^x
+// below 2^65 (results and their even / odd sums stay within 64 bits).  The
 // sectors' results for one orbit are summed, so they need a common exponent:
-// minexp, the least one of the rows of a class -- the nodes with the same
-// number of central coordinates, whose coefficients have the same size
-// (kNoExp if an entry is not finite).
-template <int DIM, bool CELL>
-__global__ void __launch_bounds__(128) sector_entries_kernel(const double* __restrict__ columns,
-                                                             double* __restrict__ entries, int* __restrict__ rowexp,
-                                                             int* __restrict__ minexp) {
-  constexpr int M = CELL ? kCellM : kPatchM;
+// minexp, the least one of the orbit's rows (kNoExp in the first if an entry is not finite).
+template <int DIM, int M>
+__global__ void __launch_bounds__(128) sector_exponents_kernel(const double* __restrict__ hi,
+                                                               const double* __restrict__ lo, int* __restrict__ rowexp,
+                                                               int* __restrict__ minexp) {
   using S = Sectors<DIM, M>;
   const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= S::ROWS) return;
@@ -1150,46 +1551,11 @@ __global__ void __launch_bounds__(128) sector_entries_kernel(const double* __res
   while (s + 1 < S::NS && row >= S::row(s + 1)) ++s;
   const int m = row - S::row(s), sz = S::size(s);
   const Orbit<DIM, M> om = orbit_of<DIM, M>(s, m);
-  double* out = entries + S::entry(s) + (int64_t)m * sz;
   double top = 0.0, sum = 0.0;
   for (int k = lane; k < sz; k += 32) {
-    const Orbit<DIM, M> oj = orbit_of<DIM, M>(s, k);
-    double a;
-    if constexpr (CELL) {
-      const double* C = coef<double>();
-      dd f[2][3];  // 1D mass and stiffness between the two coefficients, per direction
-#pragma unroll
-      for (int d = 0; d < DIM; ++d)
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-          const double* T1 = C + (w ? LAY.Ke : LAY.Me) + oj.c[d];
-          const double r = T1[om.c[d] * M], q = T1[(M - 1 - om.c[d]) * M];
-          const bool centre = S::CENTRE && oj.c[d] == S::E - 1;  // one image in this direction
-          f[w][d] = !S::SPLIT ? dd(r) : centre ? dd(0.5 * r) : 0.5 * (dd(r) + dd(((s >> d) & 1) ? -q : q));
-        }
-      dd acc(0.0);
-#pragma unroll
-      for (int d = 0; d < DIM; ++d) {
-        dd p = f[d == 0][0];
-#pragma unroll
-        for (int e = 1; e < DIM; ++e) p = p * f[d == e][e];
-        acc += p;
-      }
-      a = value_of(acc);
-    } else {
-      const double* col = columns + (int64_t)(oj.c[0] + S::E * (oj.c[1] + S::E * oj.c[2])) * S::NODES;
-      a = 0.0;
-#pragma unroll
-      for (int b = 0; b < S::IMAGES; ++b) {
-        if (S::IMAGES > 1 && !oj.has(b)) continue;
-        const double v = col[om.node(b)];
-        a += (__popc(s & b) & 1) ? -v : v;
-      }
-      a /= S::IMAGES;
-    }
-    out[k] = a;
-    top = fmax(top, fabs(a));
-    sum += fabs(a);
+    const double a = fabs(value_of(sector_entry<DIM, M>(hi, lo, s, om, orbit_of<DIM, M>(s, k))));
+    top = fmax(top, a);
+    sum += a;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -1197,58 +1563,58 @@ __global__ void __launch_bounds__(128) sector_entries_kernel(const double* __res
     sum += __shfl_xor_sync(0xffffffffu, sum, o);
   }
   if (lane) return;
-  constexpr int SL = Dense<DIM, M, double>::SL;
   int te = 0, se = 0;
   if (frexp(top, &te) > 0.98) ++te;
   frexp(sum, &se);
-  const int x = sum == 0.0 ? 1000 : min(8 * SL - 1 - te, 8 * SL + 1 - se);
+  const int x = sum == 0.0 ? 1000 : min(63 - te, 65 - se);
   rowexp[row] = x;
-  atomicMin(minexp + om.centres(), x);
+  atomicMin(minexp + om.c[0] + S::E * (om.c[1] + S::E * om.c[2]), x);
   if (!isfinite(sum)) atomicMin(minexp, kNoExp);
 }
 
 // Fragments of the first operand of mma.m16n8k16, per 16 x 16 tile and part:
 // lane l holds rows l / 4 and l / 4 + 8, columns 2 (l % 4) and + 8.  FP64:
 // 8-bit signed digits of entry 2^(the row's exponent, at most 15 above its
-// class's); FP32: three BF16 parts, rounded.
-template <int DIM, typename T, bool CELL>
-__global__ void __launch_bounds__(256) sector_table_kernel(const double* __restrict__ entries,
+// orbit's); FP32: three BF16 parts, rounded.
+template <int DIM, typename T, int M>
+__global__ void __launch_bounds__(256) sector_table_kernel(const double* __restrict__ hi, const double* __restrict__ lo,
                                                            const int* __restrict__ rowexp,
                                                            const int* __restrict__ minexp,
                                                            uint32_t* __restrict__ table) {
-  constexpr int M = CELL ? kCellM : kPatchM;
   using S = Sectors<DIM, M>;
   using D = Dense<DIM, M, T>;
   constexpr int SL = D::SL;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int* tail = reinterpret_cast<int*>(table + (int64_t)D::FRAGS * 4);
+  if (sizeof(T) == 8 && t < S::ORBITS) tail[S::ROWS + t] = minexp[t];
   if (t >= (int64_t)S::TILES * 32 * 4) return;
   const int reg = (int)(t & 3), lane = (int)(t >> 2) & 31, tile = (int)(t >> 7);
   int s = 0;
   while (s + 1 < S::NS && tile >= S::tile(s + 1)) ++s;
   const int nt = S::tiles(s), sz = S::size(s), mt = (tile - S::tile(s)) / nt, kt = (tile - S::tile(s)) % nt;
   const int m = 16 * mt + (lane >> 2) + 8 * (reg & 1), k0 = 16 * kt + 2 * (lane & 3) + 8 * (reg >> 1);
+  const Orbit<DIM, M> om = orbit_of<DIM, M>(s, m < sz ? m : 0);
   int re = 0;
   if (sizeof(T) == 8 && m < sz) {
-    const int exp = minexp[orbit_of<DIM, M>(s, m).centres()];
+    const int exp = minexp[om.c[0] + S::E * (om.c[1] + S::E * om.c[2])];
     re = min(rowexp[S::row(s) + m], exp + 15);
-    int* tail = reinterpret_cast<int*>(table + (int64_t)D::FRAGS * 4);
     if (kt == 0 && (lane & 3) == 0 && reg < 2) tail[S::row(s) + m] = re - exp;
-    if (tile == 0 && lane == 0 && reg == 0)
-      for (int i = 0; i < 4; ++i) tail[S::ROWS + i] = minexp[i];
   }
   uint32_t part[SL] = {};
   for (int h = 0; h < 2; ++h) {
     const int k = k0 + h;
-    const double a = m < sz && k < sz ? entries[S::entry(s) + (int64_t)m * sz + k] : 0.0;
+    const Orbit<DIM, M> oj = orbit_of<DIM, M>(s, k < sz ? k : 0);
+    const dd a = m < sz && k < sz ? sector_entry<DIM, M>(hi, lo, s, om, oj) : dd(0.0);
     if constexpr (sizeof(T) == 8) {
-      const unsigned long long v = (unsigned long long)__double2ll_rn(scalbn(a, re)) + D::BIAS;
+      const long long w = __double2ll_rn(scalbn(a.hi, re)) + __double2ll_rn(scalbn(a.lo, re));
+      const unsigned long long v = (unsigned long long)w + D::BIAS;
       for (int i = 0; i < SL; ++i) {
         const int digit = (int)((v >> (8 * (SL - 1 - i))) & 0xFF) - 128;
         part[i] |= (uint32_t)__half_as_ushort(__int2half_rn(digit)) << (16 * h);
       }
     } else {
       // FP32 operands are plain sums over the images
-      double rest = a * (1 << orbit_of<DIM, M>(s, k < sz ? k : 0).centres());
+      double rest = value_of(a) * (1 << oj.centres());
       for (int i = 0; i < SL; ++i) {
         const __nv_bfloat16 p = __double2bfloat16(rest);
         rest -= (double)__bfloat162float(p);

@@ -228,7 +228,8 @@ int make_plan(const pmg_config* cfg, Plan& P) {
       if (P.stage_batches > 0) P.stage = bump(cur, km->patch_stage_bytes(P.stage_batches));
     }
     if (cb > 0) P.ctable = bump(cur, cb);
-    if (tb > 0 || cb > 0) P.tscratch = bump(cur, k64->patch_scratch_bytes(P.dim));
+    if (tb > 0 || cb > 0)
+      P.tscratch = bump(cur, std::max(tb > 0 ? k64->patch_scratch_bytes(P.dim) : 0, k64->cell_scratch_bytes(P.dim)));
   }
   if (cfg->geometry == PMG_GEOM_DISTORTED) P.verts = bump(cur, ipow64(nf + 1, P.dim) * P.dim * 8);
   if (P.deformed) P.cellbuf = bump(cur, ipow64(nf, P.dim) * ipow64(P.K + 1, P.dim) * 8);
@@ -907,7 +908,7 @@ void pinned_scalars_put(double* p) {
   g_pin_free.push_back(p);
 }
 
-// Sector matrices of the Cartesian local solver (kernels_patch.cuh): entries
+// Sector matrices of the Cartesian local solver (kernels_patch.cuh): columns
 // from the FP64 part at unit scale, then the table of the MG precision.
 int setup_patch_table(pmg_ctx* c) {
   double* scratch = (double*)at(c, c->plan.tscratch);
@@ -925,8 +926,8 @@ int setup_patch_table(pmg_ctx* c) {
   P.inv_a0 = 1.0 / (c->dim * 2.0 * std::pow(2.0 / 3.0, c->dim - 1));
   P.half = c->cfg.local_half;
   P.colour = -1;
-  PMG_CUDA(c->kt[PMG_FP64]->patch_entries(c->dim, P, c->cfg.local_cycles, c->mgprec, c->dtab64, scratch,
-                                            c->stream));
+  PMG_CUDA(c->kt[PMG_FP64]->patch_entries(c->dim, P, c->cfg.local_cycles, c->mgprec, c->dtab64,
+                                            c->km()->patch_columns(c->dim, c->mgprec, c->table), scratch, c->stream));
   PMG_CUDA(c->km()->patch_table(c->dim, c->mgprec, scratch, c->table, c->stream));
   return PMG_OK;
 }

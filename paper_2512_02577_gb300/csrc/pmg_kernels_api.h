@@ -135,22 +135,25 @@ struct KernelTable {
   cudaError_t (*h_restrict_group)(int dim, int prec, int count, const TransferSolveJob* jobs, cudaStream_t s);
   // Cartesian patches as products with the local solver's sector matrices:
   // device bytes of the part's table (0: the part sum-factorises, or K = 1) and
-  // of the FP64 scratch of its set-up; the set-up on the degree's FP64 part
-  // (the local solver of n_iter cycles at unit scale, for products in precision
-  // prec), then the table on the part itself
+  // of the FP64 scratch of its set-up; the columns of the local solver, which
+  // end the table, and their set-up on the degree's FP64 part (n_iter cycles at
+  // unit scale, for products in precision prec); then the rest of the table on
+  // the part itself
   int64_t (*patch_table_bytes)(int dim, int prec);
   int64_t (*patch_scratch_bytes)(int dim);
+  double* (*patch_columns)(int dim, int prec, void* table);
   cudaError_t (*patch_entries)(int dim, const PatchParamsHost& H, int n_iter, int prec, const double* dinv,
-                               double* scratch, cudaStream_t s);
-  cudaError_t (*patch_table)(int dim, int prec, const double* scratch, void* table, cudaStream_t s);
+                               double* columns, double* scratch, cudaStream_t s);
+  cudaError_t (*patch_table)(int dim, int prec, double* scratch, void* table, cudaStream_t s);
   // staged parts (FP64 K = 6, 7 in 3D): bytes of the buffers for a number of
   // batches, the batches to provide for a finest level of n cells (else 0)
   int64_t (*patch_stage_bytes)(int64_t batches);
   int64_t (*patch_stage_batches)(int n);
   // FP64 Cartesian apply as products with the cell's sector matrices (FP64
-  // part): bytes of their table (0: line passes only), its set-up (scratch as
-  // above), y = A x or b - A x; cells: n^d (K+1)^d doubles of scratch
+  // part): bytes of their table (0: line passes only) and of its set-up's
+  // scratch, the set-up, y = A x or b - A x; cells: n^d (K+1)^d doubles of scratch
   int64_t (*cell_table_bytes)(int dim);
+  int64_t (*cell_scratch_bytes)(int dim);
   cudaError_t (*cell_table)(int dim, double* scratch, void* table, cudaStream_t s);
   cudaError_t (*cell_apply)(int dim, const double* x, double* y, const double* b, double* cells, const void* table,
                             int n, double scale, cudaStream_t s);
