@@ -1187,10 +1187,19 @@ __device__ __forceinline__ PatchOrigin patch_origin(const DenseJob<double>& J, u
   return o;
 }
 
-// X [row][P] and the words of batch first + blockIdx.x
+// A run of batches of one level: batch first + b of the job in place b of the buffers
+struct StageJob {
+  DenseJob<double> J;
+  uint32_t first;
+  long long* X;
+  long long* Y;
+  int* words;
+};
+
+// X [row][P] and the words of batch first + b
 template <int DIM>
-__global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant__ DenseJob<double> J, uint32_t first,
-                                                          long long* __restrict__ X, int* __restrict__ words) {
+__device__ __forceinline__ void patch_split(const StageJob& G, uint32_t b) {
+  const DenseJob<double>& J = G.J;
   constexpr int M = kPatchM;
   using S = Sectors<DIM, M>;
   using L = Lines<DIM, M>;
@@ -1201,11 +1210,11 @@ __global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant_
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pn = lane % P, item0 = warp * (32 / P) + lane / P;
   constexpr int STEP = 8 * (32 / P);
   const int N1 = K * J.n + 1;
-  const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + pn);
+  const PatchOrigin o = patch_origin<DIM>(J, (G.first + b) * P + pn);
   const double* rp = J.r + o.base;
   const int* orbitexp = reinterpret_cast<const int*>(J.table + Stage<DIM>::D::FRAGS) + S::ROWS;
-  X += blockIdx.x * Stage<DIM>::XWORDS;
-  words += blockIdx.x * 2 * P;
+  long long* X = G.X + b * Stage<DIM>::XWORDS;
+  int* words = G.words + b * 2 * P;
   if (threadIdx.x < P) {
     s_max[threadIdx.x] = 0;
     for (int i = 0; i < NOCT; ++i) s_oct[i][threadIdx.x] = 0;
@@ -1292,11 +1301,9 @@ __global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant_
   }
 }
 
-// products of sector blockIdx.y for batch blockIdx.x
+// products of sector s for batch first + b
 template <int DIM>
-__global__ void __launch_bounds__(256, 2) patch_product_kernel(const uint4* __restrict__ table,
-                                                               const long long* __restrict__ X,
-                                                               long long* __restrict__ Y) {
+__device__ __forceinline__ void patch_product(const StageJob& G, uint32_t b, int s) {
   using St = Stage<DIM>;
   using D = typename St::D;
   using S = typename St::S;
@@ -1304,8 +1311,9 @@ __global__ void __launch_bounds__(256, 2) patch_product_kernel(const uint4* __re
   extern __shared__ __align__(16) unsigned char smraw[];
   long long* xs = reinterpret_cast<long long*>(smraw);
   long long* ys = reinterpret_cast<long long*>(smraw + St::XSM);
-  const int s = blockIdx.y, size = S::size(s), tiles = S::tiles(s), row = S::row(s);
-  const long long* x = X + blockIdx.x * St::XWORDS + (int64_t)row * P;
+  const int size = S::size(s), tiles = S::tiles(s), row = S::row(s);
+  const uint4* table = G.J.table;
+  const long long* x = G.X + b * St::XWORDS + (int64_t)row * P;
   for (int i = threadIdx.x; i < 16 * tiles * P; i += 256)
     xs[i / P * D::XP + i % P] = i < size * P ? x[i] : 0;
   __syncthreads();
@@ -1320,15 +1328,14 @@ __global__ void __launch_bounds__(256, 2) patch_product_kernel(const uint4* __re
     dense_mma<D>(u, table, shifts, xs, ys, threadIdx.x & 31);
   }
   __syncthreads();
-  long long* y = Y + blockIdx.x * St::YWORDS + (int64_t)row * P;
+  long long* y = G.Y + b * St::YWORDS + (int64_t)row * P;
   for (int i = threadIdx.x; i < size * P; i += 256) y[i] = ys[i];
 }
 
-// nodes of the planes z = blockIdx.y and its mirror image, batch first + blockIdx.x
+// nodes of the planes z = cz and its mirror image, batch first + b
 template <int DIM>
-__global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant__ DenseJob<double> J, uint32_t first,
-                                                          const long long* __restrict__ Y,
-                                                          const int* __restrict__ words) {
+__device__ __forceinline__ void patch_merge(const StageJob& G, uint32_t b, int cz) {
+  const DenseJob<double>& J = G.J;
   constexpr int M = kPatchM;
   using St = Stage<DIM>;
   using S = typename St::S;
@@ -1336,14 +1343,14 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
   constexpr int P = St::P, MP2 = St::MP2, ZP = St::ZP;
   extern __shared__ __align__(16) unsigned char smraw[];
   double* Z = reinterpret_cast<double*>(smraw);
-  const int pn = threadIdx.x % P, cz = blockIdx.y;
+  const int pn = threadIdx.x % P;
   const int N1 = K * J.n + 1;
   const int* orbitexp = reinterpret_cast<const int*>(J.table + St::D::FRAGS) + S::ROWS;
   __shared__ int s_count;
-  words += blockIdx.x * 2 * P;
+  const int* words = G.words + b * 2 * P;
   const int word = words[pn];
   const int ve = J.vexp + (word & 0xFFF) - (word & (1 << 12) ? 100 : 0);
-  Y += blockIdx.x * St::YWORDS;
+  const long long* Y = G.Y + b * St::YWORDS;
   for (int cy = threadIdx.x / P; cy < S::E; cy += 128 / P) {
     const L ln(cy + S::E * cz);
     long long v[L::IMAGES][M];
@@ -1370,7 +1377,7 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
   const int64_t N = (int64_t)N1 * N1 * N1;
   const int planes = cz == S::E - 1 ? 1 : 2;
   for (int gp = threadIdx.x >> 5; gp < P; gp += 4) {
-    const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + gp);
+    const PatchOrigin o = patch_origin<DIM>(J, (G.first + b) * P + gp);
     if (!o.active) break;
     for (int i = threadIdx.x & 31; i < planes * MP2; i += 32) {
       const int pl = i >= MP2, r = (i - pl * MP2) / M, ix = i - pl * MP2 - r * M, iz = pl ? M - 1 - cz : cz;
@@ -1387,7 +1394,7 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
   for (int gp = 0; gp < P; ++gp) {
     const unsigned bound = (unsigned)words[P + gp];
     if (bound == kNoSpikes) continue;
-    const PatchOrigin o = patch_origin<DIM>(J, (first + blockIdx.x) * P + gp);
+    const PatchOrigin o = patch_origin<DIM>(J, (G.first + b) * P + gp);
     __syncthreads();
     for (int i = threadIdx.x; i < S::NODES; i += 128) Z[i] = J.r[o.base + i % M + N1 * (i / M % M + N1 * (i / MP2))];
     __syncthreads();
@@ -1398,6 +1405,35 @@ __global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant_
           J.c * spikes_at<DIM, M>(columns, Z, list, count, q + MP2 * iz);
     }
   }
+}
+
+// one run, and the runs of several levels (blockIdx.x numbers the batches)
+template <int DIM>
+__global__ void __launch_bounds__(256) patch_split_kernel(const __grid_constant__ StageJob G) {
+  patch_split<DIM>(G, blockIdx.x);
+}
+template <int DIM>
+__global__ void __launch_bounds__(256) patch_split_group_kernel(const __grid_constant__ GroupOf<StageJob> G) {
+  const int j = group_find(G, blockIdx.x);
+  patch_split<DIM>(G.job[j], blockIdx.x - (uint32_t)G.start[j]);
+}
+template <int DIM>
+__global__ void __launch_bounds__(256, 2) patch_product_kernel(const __grid_constant__ StageJob G) {
+  patch_product<DIM>(G, blockIdx.x, blockIdx.y);
+}
+template <int DIM>
+__global__ void __launch_bounds__(256, 2) patch_product_group_kernel(const __grid_constant__ GroupOf<StageJob> G) {
+  const int j = group_find(G, blockIdx.x);
+  patch_product<DIM>(G.job[j], blockIdx.x - (uint32_t)G.start[j], blockIdx.y);
+}
+template <int DIM>
+__global__ void __launch_bounds__(128) patch_merge_kernel(const __grid_constant__ StageJob G) {
+  patch_merge<DIM>(G, blockIdx.x, blockIdx.y);
+}
+template <int DIM>
+__global__ void __launch_bounds__(128) patch_merge_group_kernel(const __grid_constant__ GroupOf<StageJob> G) {
+  const int j = group_find(G, blockIdx.x);
+  patch_merge<DIM>(G.job[j], blockIdx.x - (uint32_t)G.start[j], blockIdx.y);
 }
 
 // K = 1: the patch is its vertex, the local solve one multiplication by
