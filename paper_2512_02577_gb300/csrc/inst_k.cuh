@@ -197,13 +197,17 @@ template <int DIM>
 static cudaError_t stage_launch(const GroupOf<StageJob>& G, cudaStream_t st) {
   using St = Stage<DIM>;
   const unsigned nb = (unsigned)G.start[G.count];
+  // while the blocks are less than two per SM, a sector's row tiles in up to
+  // three parts of 8, a tile per warp (half cycle, K = 7 at 4^3 cells, sweep: 155 us
+  // with one part, 110 with three, 127 by sum factorisation)
+  const unsigned z = std::max(1u, std::min((St::MAXT + 7u) / 8u, 304u / (nb * St::S::NS)));
   if (G.count == 1) {
     patch_split_kernel<DIM><<<nb, 256, 0, st>>>(G.job[0]);
-    patch_product_kernel<DIM><<<dim3(nb, St::S::NS), 256, St::XSM + St::YSM, st>>>(G.job[0]);
+    patch_product_kernel<DIM><<<dim3(nb, St::S::NS, z), 256, St::XSM + St::YSM, st>>>(G.job[0]);
     patch_merge_kernel<DIM><<<dim3(nb, St::S::E), 128, St::ZSM, st>>>(G.job[0]);
   } else {
     patch_split_group_kernel<DIM><<<nb, 256, 0, st>>>(G);
-    patch_product_group_kernel<DIM><<<dim3(nb, St::S::NS), 256, St::XSM + St::YSM, st>>>(G);
+    patch_product_group_kernel<DIM><<<dim3(nb, St::S::NS, z), 256, St::XSM + St::YSM, st>>>(G);
     patch_merge_group_kernel<DIM><<<dim3(nb, St::S::E), 128, St::ZSM, st>>>(G);
   }
   g_launches += 3;

@@ -186,10 +186,15 @@ __device__ __forceinline__ void for_coefs(int b, F&& f) {
 // ---------------------------------------------------------------- block shape
 // P windows per block (the n extent of the products), NW warps: the fastest of
 // P = 16, 32 and NW = 2..16 in FP32 (K = 4 at 32^3: 0.055 ms, 0.061 with P =
-// 32, 0.067 with 4 or 16 warps; K = 2 at 100^3: 0.157 ms, 0.25 with 8 warps).  3D patches of
-// K >= 6 keep the sum-factorised kernel: their operands fill an SM's shared
-// memory with 8-16 patches, and the matrix is streamed from L2 for so few
-// columns (K = 6 FP32 at 33^3 cells: 0.67 ms against 0.49 ms).
+// 32, 0.067 with 4 or 16 warps; K = 2 at 100^3: 0.157 ms, 0.25 with 8 warps).
+// 16 warps where one or two blocks fill an SM's shared memory (K = 5 patches, cells of
+// K = 7, 8): a launch of few blocks is one block's latency, half the row tiles per
+// warp shorten it (8 and 16 warps: FP32 K = 5 at 8^3 cells, sweep 33.8 and 31.1 us,
+// multiplicative 255 and 231; FP64 apply K = 8 71.8 and 67.1), and large
+// ones are as fast.  3D FP32 patches of K >= 6 and FP64 ones of K = 8 keep the
+// sum-factorised kernel: their operands fill an SM's shared memory with 8-16
+// patches, and the matrix is streamed from L2 for so few columns (K = 6 FP32 at
+// 33^3 cells: 0.67 ms against 0.49 ms).
 template <int DIM, int M, typename T>
 struct Dense {
   using S = Sectors<DIM, M>;
@@ -200,7 +205,7 @@ struct Dense {
   static constexpr int NT = P / 8;                              // 8-column tiles
   static constexpr int NSUB = 32 / P;                           // lines a warp handles at once
   static constexpr int UNITS = S::PROWS / 16;                   // 16-row tiles of the result
-  static constexpr int NW = UNITS >= 16 ? 8 : (UNITS > 2 ? 4 : 2);
+  static constexpr int NW = UNITS >= 32 ? 16 : UNITS >= 16 ? 8 : (UNITS > 2 ? 4 : 2);
   static constexpr int UPW = (UNITS + NW - 1) / NW;             // units per warp
   // Operands: FP64 fixed-point values [row][XP], FP32 the three parts as
   // planes of BF16 [part][row][XP]; the pitch spreads the rows over the banks.
@@ -1323,7 +1328,8 @@ __device__ __forceinline__ void patch_split(const StageJob& G, uint32_t b) {
   }
 }
 
-// products of sector s for batch first + b
+// products of sector s for batch first + b; the sector's row tiles in
+// gridDim.z parts (stage_launch)
 template <int DIM>
 __device__ __forceinline__ void patch_product(const StageJob& G, uint32_t b, int s) {
   using St = Stage<DIM>;
@@ -1340,7 +1346,8 @@ __device__ __forceinline__ void patch_product(const StageJob& G, uint32_t b, int
     xs[i / P * D::XP + i % P] = i < size * P ? x[i] : 0;
   __syncthreads();
   const int* shifts = reinterpret_cast<const int*>(table + D::FRAGS) + row;
-  for (int m = threadIdx.x >> 5; m < tiles; m += 8) {
+  const int m0 = (int)(blockIdx.z * tiles / gridDim.z), m1 = (int)((blockIdx.z + 1) * tiles / gridDim.z);
+  for (int m = m0 + (threadIdx.x >> 5); m < m1; m += 8) {
     DenseUnit u;
     u.prow = 0;
     u.kt = (short)tiles;
@@ -1351,7 +1358,7 @@ __device__ __forceinline__ void patch_product(const StageJob& G, uint32_t b, int
   }
   __syncthreads();
   long long* y = G.Y + b * St::YWORDS + (int64_t)row * P;
-  for (int i = threadIdx.x; i < size * P; i += 256) y[i] = ys[i];
+  for (int i = 16 * m0 * P + threadIdx.x; i < min(16 * m1, size) * P; i += 256) y[i] = ys[i];
 }
 
 // nodes of the planes z = cz and its mirror image, batch first + b
