@@ -80,7 +80,7 @@ enum pmg_outer {
  * local solves, §3.2).  Both give bitwise the same results.  The layout,
  * patches_per_block, patch_threads and patch_persistent shape the
  * sum-factorised patch kernels: deformed and distorted meshes, and Cartesian
- * 3D FP32 of degree >= 6 and FP64 of degree 8.  The other Cartesian patches are
+ * 2D FP32 of degree 2, 3D FP32 of degree >= 6 and FP64 of degree 8.  The other Cartesian patches are
  * solved by products with the local solver's matrix, which have one block
  * shape: there the values are checked and reported, without effect. */
 enum pmg_patch_layout {

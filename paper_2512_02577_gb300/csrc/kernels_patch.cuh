@@ -228,7 +228,12 @@ struct Dense {
     const int bs = 227 * 1024 / (SMEM + 1536), br = 65536 / (32 * NW * (F64 ? 128 : 64)), b = bs < br ? bs : br;
     return b < 1 ? 1 : (b > 8 ? 8 : b);
   }
-  static constexpr bool ok() { return K >= 2 && M <= (DIM == 2 ? 15 : 9) && SMEM <= kMaxDynSmem; }
+  // patches of this part are products; not 2D K = 2 in FP32, whose 9 nodes fill
+  // half a tile and are bound by their gather and scatter (700^2 cells: sweep 80
+  // us, 66 by sum factorisation; multiplicative 178 and 129)
+  static constexpr bool ok() {
+    return K >= 2 && M <= (DIM == 2 ? 15 : 9) && SMEM <= kMaxDynSmem && !(DIM == 2 && K == 2 && !F64);
+  }
   // table: 16-byte fragments, then (FP64) per row its exponent above its
   // orbit's, and the exponents of the orbits' results (kNoExp in the first: a
   // matrix that is not finite), then the columns of the orbits' first nodes
