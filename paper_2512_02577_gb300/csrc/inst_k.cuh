@@ -739,11 +739,20 @@ static DenseJob<double> cell_job(const double* x, double* cells, const void* tab
   return J;
 }
 
+// Levels whose cells are multiplied; on the others the line passes are faster:
+// up to 8^3 cells of K = 8 (32 blocks, one per SM for its 216 KB, 62-67 us; 57-58
+// us by lines; at 12^3 81 and 187)
+template <int DIM>
+static bool cells_pay(int n) { return !(DIM == 3 && K == 8) || n > 8; }
+
+// t: scratch of cart_apply; t[0] also holds n^d (K+1)^d doubles
 template <int DIM, typename T>
-static cudaError_t cell_apply_t(const double* x, double* y, const double* b, double* cells, const void* table, int n,
+static cudaError_t cell_apply_t(const double* x, double* y, const double* b, double* const* t, const void* table, int n,
                                 double scale, cudaStream_t st) {
   if constexpr (kCellDense) {
+    if (!cells_pay<DIM>(n)) return cart_apply_t<DIM, double>(x, y, b, t[0], t[1], t[2], t[3], n, scale, st);
     using D = CellDense<DIM>;
+    double* cells = t[0];
     const DenseJob<double> J = cell_job<DIM>(x, cells, table, n, scale);
     cell_dense_kernel<DIM><<<(J.npatch + D::P - 1) / D::P, 32 * D::NW, D::SMEM, st>>>(J);
     const int64_t N = ipow64(K * n + 1, DIM);
@@ -754,10 +763,10 @@ static cudaError_t cell_apply_t(const double* x, double* y, const double* b, dou
   return cudaErrorInvalidValue;
 }
 
-static cudaError_t cell_apply(int dim, const double* x, double* y, const double* b, double* cells, const void* table,
+static cudaError_t cell_apply(int dim, const double* x, double* y, const double* b, double* const* t, const void* table,
                               int n, double scale, cudaStream_t st) {
   if (dim != DP) return cudaErrorInvalidValue;
-  return cell_apply_t<DP, TP>(x, y, b, cells, table, n, scale, st);
+  return cell_apply_t<DP, TP>(x, y, b, t, table, n, scale, st);
 }
 
 template <int DIM, typename T>
@@ -766,17 +775,28 @@ static cudaError_t cell_apply_group_t(int count, const ApplyJob* jobs, cudaStrea
     using D = CellDense<DIM>;
     GroupOf<DenseJob<double>> G;
     GroupOf<CellSumJob<DIM>> H;
-    G.count = H.count = count;
     G.start[0] = H.start[0] = 0;
-    for (int j = 0; j < count; ++j) {
-      const ApplyJob& a = jobs[j];
-      G.job[j] = cell_job<DIM>((const double*)a.x, (double*)a.t[0], a.table, a.n, a.scale);
-      G.start[j + 1] = G.start[j] + (G.job[j].npatch + D::P - 1) / D::P;
-      H.job[j] = CellSumJob<DIM>{(const double*)a.t[0], (const double*)a.b, (double*)a.y, a.n, FastDiv(K * a.n + 1)};
-      H.start[j + 1] = H.start[j] + ipow64(K * a.n + 1, DIM);
+    ApplyJob lines[kMaxGroup];  // the members whose level takes the line passes
+    int m = 0, nl = 0;
+    for (int i = 0; i < count; ++i) {
+      const ApplyJob& a = jobs[i];
+      if (!cells_pay<DIM>(a.n)) {
+        lines[nl++] = a;
+        continue;
+      }
+      G.job[m] = cell_job<DIM>((const double*)a.x, (double*)a.t[0], a.table, a.n, a.scale);
+      G.start[m + 1] = G.start[m] + (G.job[m].npatch + D::P - 1) / D::P;
+      H.job[m] = CellSumJob<DIM>{(const double*)a.t[0], (const double*)a.b, (double*)a.y, a.n, FastDiv(K * a.n + 1)};
+      H.start[m + 1] = H.start[m] + ipow64(K * a.n + 1, DIM);
+      ++m;
     }
-    cell_dense_group_kernel<DIM><<<(unsigned)G.start[count], 32 * D::NW, D::SMEM, st>>>(G);
-    cell_sum_group_kernel<DIM><<<(unsigned)((H.start[count] + 255) / 256), 256, 0, st>>>(H);
+    G.count = H.count = m;
+    if (nl > 0) {
+      cudaError_t e = cart_apply_group_t<DIM, double>(nl, lines, st);
+      if (e != cudaSuccess || m == 0) return e;
+    }
+    cell_dense_group_kernel<DIM><<<(unsigned)G.start[m], 32 * D::NW, D::SMEM, st>>>(G);
+    cell_sum_group_kernel<DIM><<<(unsigned)((H.start[m] + 255) / 256), 256, 0, st>>>(H);
     g_launches += 2;
     return cudaGetLastError();
   }

@@ -308,7 +308,7 @@ int level_apply(pmg_ctx* c, int level, int prec, const void* u, void* r, const v
                                prec == c->mgprec ? c->def_cpb : 0, c->stream);
   } else if (prec == PMG_FP64 && c->ctable) {
     // the four scratch vectors hold the cells' results: (K+1)^d n^d <= 4 (K n + 1)^d for K >= 2
-    e = c->kt[PMG_FP64]->cell_apply(c->dim, (const double*)u, (double*)r, (const double*)b, c->t64[0], c->ctable, L.n,
+    e = c->kt[PMG_FP64]->cell_apply(c->dim, (const double*)u, (double*)r, (const double*)b, c->t64, c->ctable, L.n,
                                     L.scale, c->stream);
   } else {
     void** t = prec == PMG_FP64 ? (void**)c->t64 : c->t_mg;

@@ -151,11 +151,12 @@ struct KernelTable {
   int64_t (*patch_stage_batches)(int n);
   // FP64 Cartesian apply as products with the cell's sector matrices (FP64
   // part): bytes of their table (0: line passes only) and of its set-up's
-  // scratch, the set-up, y = A x or b - A x; cells: n^d (K+1)^d doubles of scratch
+  // scratch, the set-up, y = A x or b - A x, by lines on levels too small for
+  // them; t: scratch of cart_apply, t[0] with room for n^d (K+1)^d doubles
   int64_t (*cell_table_bytes)(int dim);
   int64_t (*cell_scratch_bytes)(int dim);
   cudaError_t (*cell_table)(int dim, double* scratch, void* table, cudaStream_t s);
-  cudaError_t (*cell_apply)(int dim, const double* x, double* y, const double* b, double* cells, const void* table,
+  cudaError_t (*cell_apply)(int dim, const double* x, double* y, const double* b, double* const* t, const void* table,
                             int n, double scale, cudaStream_t s);
   cudaError_t (*cell_apply_group)(int dim, int count, const ApplyJob* jobs, cudaStream_t s);
 };
