@@ -228,8 +228,10 @@ int make_plan(const pmg_config* cfg, Plan& P) {
       if (P.stage_batches > 0) P.stage = bump(cur, km->patch_stage_bytes(P.stage_batches));
     }
     if (cb > 0) P.ctable = bump(cur, cb);
-    if (tb > 0 || cb > 0)
-      P.tscratch = bump(cur, std::max(tb > 0 ? k64->patch_scratch_bytes(P.dim) : 0, k64->cell_scratch_bytes(P.dim)));
+    // the set-up's scratch: where the scratch and CG vectors (one behind the
+    // other, free until the first operation) hold it, in them
+    const int64_t scratch = std::max(tb > 0 ? k64->patch_scratch_bytes(P.dim) : 0, k64->cell_scratch_bytes(P.dim));
+    if (tb > 0 || cb > 0) P.tscratch = P.cg[5] + NF * 8 - P.t64[0] >= scratch ? P.t64[0] : bump(cur, scratch);
   }
   if (cfg->geometry == PMG_GEOM_DISTORTED) P.verts = bump(cur, ipow64(nf + 1, P.dim) * P.dim * 8);
   if (P.deformed) P.cellbuf = bump(cur, ipow64(nf, P.dim) * ipow64(P.K + 1, P.dim) * 8);
