@@ -419,13 +419,12 @@ int pmg_server_stats(const pmg_server* server, int64_t* used_bytes, int* residen
  * vectors) is a file-scope device array of 4 x PMG_NOALLOC_MAX_DOFS doubles
  * (64 MiB) that every GPU loading the library holds until exit.  The first
  * call on a device (and the first for each degree) resolves that array's
- * address and loads the degree's 1D matrices into constant memory (once per
- * degree and dimension), which
+ * address and loads the degree's kernels (once per degree and dimension), which
  * synchronises: make it before any stream capture.  All calls share the
  * array; calls that overlap on the GPU race on it.  Grids above
  * PMG_NOALLOC_MAX_DOFS are rejected with PMG_ERR_UNSUPPORTED.  x, y and the
  * stream must belong to the calling thread's current device: the scratch
- * array, the constant-memory upload and the launch all use that device. */
+ * array, the kernels and the launch all use that device. */
 int pmg_apply_cartesian_noalloc(int dim, int n_cells, int degree, const double* x, double* y, void* stream);
 
 #ifdef __cplusplus

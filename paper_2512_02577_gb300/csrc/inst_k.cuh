@@ -30,15 +30,6 @@ static int64_t ipow64(int64_t b, int e) { return e == 0 ? 1 : b * ipow64(b, e - 
 
 static bool mine(int dim, int prec) { return dim == DP && prec == PMG_PREC; }
 
-static cudaError_t upload(const double* coef) {
-  const int n = LAY.total;
-  float tmp[kMaxCoef];
-  for (int i = 0; i < n; ++i) tmp[i] = (float)coef[i];
-  cudaError_t e = cudaMemcpyToSymbol(c_coef64, coef, sizeof(double) * n);
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyToSymbol(c_coef32, tmp, sizeof(float) * n);
-}
-
 template <int DIM, typename T>
 static cudaError_t cart_apply_t(const T* x, T* y, const T* b, T* t0, T* t1, T* t2, T* t3, int n, T s,
                                 cudaStream_t st) {
@@ -1033,7 +1024,6 @@ const KernelTable* PMG_TABLE_FN() {
       PMG_DIM,
       PMG_PREC,
       PMG_KNS::prepare,
-      PMG_KNS::upload,
       PMG_KNS::cart_apply,
       PMG_KNS::patch_cart,
       PMG_KNS::patch_gather,

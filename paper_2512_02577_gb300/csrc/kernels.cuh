@@ -5,8 +5,8 @@
 // Layout on the device: every level vector is the full (K n + 1)^DIM nodal
 // grid, x fastest; boundary entries are zero.  The per-degree 1D matrices
 // (reference mass/stiffness, patch matrices, p-transfers, h-prolongation
-// tables, Gauss tables) live in __constant__ memory of this translation unit,
-// in float64 and float32 copies (coef_layout in pmg_common.cuh).
+// tables, Gauss tables) are compile-time tables of this translation unit, in
+// float64 and float32 (coef_layout in pmg_common.cuh).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -23,14 +23,10 @@ namespace PMG_KNS {
 constexpr int K = PMG_K;
 constexpr CoefLayout LAY = coef_layout(K);
 
-static __constant__ double c_coef64[kMaxCoef];
-static __constant__ float c_coef32[kMaxCoef];
-
-// The same coefficient block as compile-time tables (generated at build time
-// from the host set-up, coef_tables.h).  Every contraction whose indices are
-// known after unrolling reads these: the compiler folds the entries into the
-// arithmetic instead of loading them for every line.  Reads with run-time
-// indices (the h-transfer passes) use the constant-memory copy above.
+// The degree's coefficient block as compile-time tables (generated at build
+// time from the host set-up, coef_tables.h).  Every contraction whose indices
+// are known after unrolling folds the entries into the arithmetic instead of
+// loading them for every line.
 #define PMG_TAB_(prec, k) PMG_COEF##prec##_K##k
 #define PMG_TAB(prec, k) PMG_TAB_(prec, k)
 static __device__ constexpr double c_tab64[] = PMG_TAB(64, PMG_K);
@@ -43,13 +39,6 @@ static inline int grid_for(int64_t work, int block) {
   if (g < 1) g = 1;
   return (int)g;
 }
-
-template <typename T>
-__device__ __forceinline__ const T* coef();
-template <>
-__device__ __forceinline__ const double* coef<double>() { return c_coef64; }
-template <>
-__device__ __forceinline__ const float* coef<float>() { return c_coef32; }
 
 template <typename T>
 __device__ __forceinline__ const T* ctab();
@@ -1409,7 +1398,7 @@ __global__ void __launch_bounds__(256) patch_gather_group(const __grid_constant_
 // A thread owns the nodes of one coarse cell on one grid line along AX (2K
 // fine nodes, or K coarse ones; one more item per line for its last node), so
 // the 1D embedding is a compile-time table folded into the arithmetic, its
-// zeros dropped.  One thread per node read the table from constant memory at
+// zeros dropped.  One thread per node used to read the table from constant memory at
 // lane-dependent addresses and divided for every node (one V-cycle's transfers,
 // FP32 48^3 Q5: 0.347 ms before, 0.167 now).
 // ex, ey, ez: extents of the OUTPUT array; item order: x fastest (AX = 0: the

@@ -1580,7 +1580,7 @@ __global__ void __launch_bounds__(256) cell_columns_kernel(double* __restrict__ 
   for (int d = 0; d < DIM; ++d) {
     dd p(1.0);
 #pragma unroll
-    for (int e = 0; e < DIM; ++e) p = c_coef64[(d == e ? LAY.Ke : LAY.Me) + c[e] * M + o.c[e]] * p;
+    for (int e = 0; e < DIM; ++e) p = c_tab64[(d == e ? LAY.Ke : LAY.Me) + c[e] * M + o.c[e]] * p;
     acc += p;
   }
   const double v = value_of(acc);

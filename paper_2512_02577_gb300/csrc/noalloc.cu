@@ -38,7 +38,7 @@ static __device__ __align__(256) double g_apply_scratch[4 * kMaxDofs];
 struct DeviceState {
   bool ready = false;
   double* scratch = nullptr;  // device address of g_apply_scratch on this device
-  bool coef[9][2] = {};  // by degree and dimension
+  bool loaded[9][2] = {};  // by degree and dimension
 };
 
 constexpr int kMaxDevices = 64;
@@ -83,7 +83,7 @@ extern "C" int pmg_apply_cartesian_noalloc(int dim, int n_cells, int degree, con
   double* scratch = nullptr;
   {
     // first call on this device (and first call for this degree): resolve the
-    // scratch address and load the degree's 1D matrices into constant memory
+    // scratch address and load the degree's kernels
     std::lock_guard<std::mutex> g(g_mu);
     DeviceState& s = g_state[dev];
     if (!s.ready) {
@@ -93,12 +93,10 @@ extern "C" int pmg_apply_cartesian_noalloc(int dim, int n_cells, int degree, con
       s.scratch = (double*)ptr;
       s.ready = true;
     }
-    if (!s.coef[degree][dim - 2]) {
-      const std::vector<double>& coef = pmg::host::coefficients(degree);
+    if (!s.loaded[degree][dim - 2]) {
       e = kt->prepare();
-      if (e == cudaSuccess) e = kt->upload(coef.data());
-      if (e != cudaSuccess) return fail(PMG_ERR_CUDA, std::string("coefficient upload: ") + cudaGetErrorString(e));
-      s.coef[degree][dim - 2] = true;
+      if (e != cudaSuccess) return fail(PMG_ERR_CUDA, std::string("kernel set-up: ") + cudaGetErrorString(e));
+      s.loaded[degree][dim - 2] = true;
     }
     scratch = s.scratch;
   }

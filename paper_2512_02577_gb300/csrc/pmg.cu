@@ -983,8 +983,8 @@ int setup_context(pmg_ctx* c) {
   c->cellbuf = at(c, P.cellbuf);
   c->verts = (double*)at(c, P.verts);
 
-  // coefficients and kernel attributes: once per device and kernel part
-  // (module state that every context of the part shares)
+  // kernel attributes: once per device and kernel part (module state that
+  // every context of the part shares)
   const std::vector<double>& coef = host::coefficients(c->K);
   {
     static std::mutex mu;
@@ -995,7 +995,6 @@ int setup_context(pmg_ctx* c) {
     for (const KernelTable* t : c->kt) {
       if (ready.count({dev, t})) continue;
       PMG_CUDA(t->prepare());
-      PMG_CUDA(t->upload(coef.data()));
       ready.insert({dev, t});
     }
   }

@@ -2,7 +2,7 @@
 // p-multigrid vertex-patch library: the degree hierarchy of the local
 // p-multigrid (§2.2: 1, 3, 7, ... capped at the target degree), patch sizes,
 // structural zeros of the 1D patch and transfer matrices, and the layout of
-// the per-degree coefficient block that lives in __constant__ memory.
+// the per-degree coefficient block (compile-time tables in the kernels).
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>

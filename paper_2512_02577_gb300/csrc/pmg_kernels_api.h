@@ -4,8 +4,6 @@
 // enqueues on the given stream and returns the launch's cudaError_t, and
 // rejects (cudaErrorInvalidValue) a (dim, prec) that is not its part's.
 // Precision flag: 0 = double, 1 = float (element type of every vector).
-// Each part has its own constant-memory copy of the degree's coefficients:
-// upload() fills that copy.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -73,7 +71,6 @@ struct KernelTable {
   int dim;
   int prec;
   cudaError_t (*prepare)();
-  cudaError_t (*upload)(const double* coef);
   // y = A x (b == nullptr) or y = b - A x; Cartesian; t0..t3: scratch of N
   cudaError_t (*cart_apply)(int dim, int prec, const void* x, void* y, const void* b, void* t0, void* t1,
                             void* t2, void* t3, int n, double scale, cudaStream_t s);
