@@ -40,7 +40,7 @@ ORACLE_N = 4          # bounded CPU sample: same degree and dimension, 4^3 cells
 FP32_PEAK_TFLOPS = 78.5  # measured FP32 FMA (128 lanes x 152 SMs x 2 x ~2.0 GHz)
 # DRAM bytes (read + write) of one FP64 patch launch at 32^3 Q4, from one ncu
 # capture of that launch; to be re-taken whenever patch_dense_kernel changes.
-PATCH64_TRAFFIC_BYTES = 117700000
+PATCH64_TRAFFIC_BYTES = 117404416
 
 
 # ----------------------------------------------------------------- flop model
@@ -60,7 +60,7 @@ def p_hierarchy(k):
 
 def product_flops(d, k):
     """Tensor-core operations of one FP64 Cartesian patch solve as the patch
-    kernel executes it (K <= 5): 34 digit products of the 16 x 16 tiles of the
+    kernel executes it (K <= 5): 36 digit products of the 16 x 16 tiles of the
     sector matrices (k or k - 1 rows per direction).  Counts an FMA as 2."""
     tiles = 0
     for s in range(2 ** d):
@@ -68,7 +68,7 @@ def product_flops(d, k):
         for a in range(d):
             rows *= k - ((s >> a) & 1)
         tiles += ((rows + 15) // 16) ** 2
-    return 34 * tiles * 16 * 16 * 2
+    return 36 * tiles * 16 * 16 * 2
 
 
 def patch_flops(d, k, n_iter=1):

@@ -104,7 +104,7 @@ enum pmg_outer_apply {
                                        pair of floats (about 48 significant bits, relative error of A x within
                                        a few 1e-14 of |A| |x|) on the FP32 pipes -- on GB300 several times
                                        faster than the FP64 pipes (Cartesian FP64 applies of degree >= 2 take
-                                       the tensor cores: 32^3 Q4 0.112 ms, float-float 0.093 ms); the
+                                       the tensor cores: 32^3 Q4 0.118 ms, float-float 0.094 ms); the
                                        coarse-matrix assembly stays in FP64.
                                        Cartesian meshes; deformed and distorted ones in 3D with degree <= 3
                                        and geom_precision PMG_FP32 (else PMG_ERR_UNSUPPORTED) */
@@ -334,7 +334,8 @@ int pmg_default_damping(int dim, int degree, double* omega_patch, double* omega_
 
 /* Instrumentation: mean device times (ms, CUDA events on the context's
  * stream) of the three phases of one smoothing step on `level`, over `reps`
- * repetitions after one warm-up, on the level's own vectors: ms[0] residual
+ * repetitions after one warm-up, on the level's own vectors (starting from u = 0
+ * and a constant b): ms[0] residual
  * r = b - A u, ms[1] the patch launch (every local solve), ms[2] the gather
  * u += sum_j Pi_j^T d_j.  Overwrites the level's work vectors. */
 int pmg_smoother_phase_times(pmg_ctx* ctx, int level, int reps, double* ms);

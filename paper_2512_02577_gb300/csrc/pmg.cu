@@ -1552,6 +1552,10 @@ int pmg_smoother_phase_times(pmg_ctx* c, int level, int reps, double* ms) {
   if (int rc = check_smooth_level(c, level)) return rc;
   if (reps < 1) return fail(PMG_ERR_ARG, "reps < 1");
   LevelData& L = c->lv[level];
+  // what the level's vectors hold decides how many windows are uneven (kernels_patch.cuh): u = 0, b constant
+  const size_t es = c->mg32 ? 4 : 8;
+  PMG_CUDA(cudaMemsetAsync(L.u, 0, es * L.N, c->stream));
+  PMG_CUDA(cudaMemsetAsync(L.b, 0x3F, es * L.N, c->stream));
   cudaEvent_t ev[4];
   for (auto& e : ev) PMG_CUDA(cudaEventCreate(&e));
   double acc[3] = {0, 0, 0};
