@@ -609,8 +609,8 @@ static cudaError_t patch_columns_t(const PatchParamsHost& H, int n_iter, const d
   const int smem = np * PatchShape<DIM>::ELEMS * (int)sizeof(V);
   if (smem > kMaxDynSmem) return cudaErrorInvalidConfiguration;
   for (int it = 0; it < n_iter; ++it)
-    patch_columns_kernel<DIM, V><<<(S::ORBITS + np - 1) / np, threads, smem, st>>>(columns, scratch, np, it == 0, dinv,
-                                                                                   to_params<double>(H));
+    patch_columns_kernel<DIM, V><<<(S::ORBITS + np - 1) / np, threads, smem, st>>>(
+        columns, scratch, sector_exponents<S>(scratch), np, it == 0, dinv, to_params<double>(H));
   g_launches += n_iter;
   return cudaGetLastError();
 }
@@ -620,9 +620,7 @@ template <int DIM, int M>
 static cudaError_t sector_exponents_t(const double* columns, double* scratch, cudaStream_t st) {
   using S = Sectors<DIM, M>;
   int* exps = sector_exponents<S>(scratch);
-  cudaError_t e = cudaMemsetAsync(exps, 0x7F, 4 * S::ORBITS, st);
-  if (e != cudaSuccess) return e;
-  sector_exponents_kernel<DIM, M><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, scratch, exps + S::ORBITS, exps);
+  sector_exponents_kernel<DIM, M><<<(S::ROWS + 3) / 4, 128, 0, st>>>(columns, exps + S::ORBITS, exps);
   g_launches += 1;
   return cudaGetLastError();
 }
@@ -646,12 +644,13 @@ static cudaError_t patch_entries_t(const PatchParamsHost& H, int n_iter, bool fp
   if constexpr (sizeof(T) == 8 && K > 1) {
     cudaError_t e = cudaErrorInvalidValue;  // no such product part
     if (fp64) {
-      if constexpr (kProducts64) e = patch_columns_t<DIM, dd>(H, n_iter, dinv, columns, scratch, st);
+      if constexpr (kProducts64) {
+        e = patch_columns_t<DIM, dd>(H, n_iter, dinv, columns, scratch, st);
+        if (e == cudaSuccess) e = sector_exponents_t<DIM, kPatchM>(columns, scratch, st);
+      }
     } else {
       if constexpr (kProducts32) e = patch_columns_t<DIM, double>(H, n_iter, dinv, columns, scratch, st);
     }
-    if constexpr (kProducts64 || kProducts32)
-      if (e == cudaSuccess) e = sector_exponents_t<DIM, kPatchM>(columns, scratch, st);
     return e;
   }
   return cudaErrorInvalidValue;
@@ -699,7 +698,8 @@ static cudaError_t cell_table_t(double* scratch, void* table, cudaStream_t st) {
   if constexpr (kCellDense) {
     using S = Sectors<DIM, kCellM>;
     double* columns = (double*)((char*)table + CellDense<DIM>::COLUMNS);
-    cell_columns_kernel<DIM><<<(S::ORBITS * S::NODES + 255) / 256, 256, 0, st>>>(columns, scratch);
+    cell_columns_kernel<DIM><<<(S::ORBITS * S::NODES + 255) / 256, 256, 0, st>>>(columns, scratch,
+                                                                               sector_exponents<S>(scratch));
     g_launches += 1;
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = sector_exponents_t<DIM, kCellM>(columns, scratch, st);

@@ -32,12 +32,12 @@
 // three BF16 parts of each value (8 bits each, exact), the six products of
 // weight 2^-16 and above.
 //
-// Patch launch of one sweep, before and now (GB300): FP64 K = 4 at 32^3 cells
-// 2.344 and 0.195 ms (tensor pipe 35% of its cycles, issue slots 40%: the
-// digit conversions and the 64-bit gather and scatter); FP64 K = 5 at 24^3
-// 2.12 and 0.36 ms; FP32 K = 4 at 32^3 0.135 and 0.055 ms (shared-memory and
-// L1 wavefronts: 80% of their rate), K = 5 at 40^3 0.473 and 0.319 ms, K = 3
-// at 67^3 0.328 and 0.203 ms, K = 2 at 100^3 0.283 and 0.162 ms.
+// Patch launch of one sweep, by sum factorisation and now (GB300): FP64 K = 4
+// at 32^3 cells 2.343 and 0.229 ms (tensor pipe 30% of its cycles, issue slots
+// 46%: the digit conversions and the 64-bit gather and scatter); FP64 K = 5 at
+// 24^3 2.12 and 0.36 ms; FP32 K = 4 at 32^3 0.135 and 0.057 ms (shared-memory
+// and L1 wavefronts: 69% of their rate), K = 5 at 40^3 0.473 and 0.316 ms, K =
+// 3 at 67^3 0.327 and 0.192 ms, K = 2 at 100^3 0.283 and 0.157 ms.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -674,7 +674,7 @@ __device__ __noinline__ void dense_spikes(const DenseJob<T>& J, uint32_t batch, 
 // holds one window): gather, even / odd combinations, results in Y.  Finds the
 // uneven windows (s_spike, s_any); AGAIN: the block's windows without spikes.
 template <int DIM, typename T, bool CELL, bool AGAIN, int NOCT>
-__device__ __forceinline__ void dense_round(const DenseJob<T>& J, int64_t base, bool active, unsigned edge,
+__device__ __forceinline__ void dense_pass(const DenseJob<T>& J, int64_t base, bool active, unsigned edge,
                                             unsigned* s_max, unsigned (*s_oct)[Dense<DIM, CELL ? kCellM : kPatchM, T>::P],
                                             unsigned* s_spike, int* s_any) {
   constexpr int M = CELL ? kCellM : kPatchM;
@@ -852,7 +852,7 @@ __device__ __forceinline__ void dense_round(const DenseJob<T>& J, int64_t base, 
   }
 }
 
-// The second round.  A window with more spikes than an eighth of its nodes
+// The second pass.  A window with more spikes than an eighth of its nodes
 // keeps them (kNoSpikes): its large values reach every node.
 template <int DIM, typename T, bool CELL, int NOCT>
 __device__ __noinline__ void dense_again(const DenseJob<T>& J, const int64_t* s_base, const int* s_colour,
@@ -878,10 +878,10 @@ __device__ __noinline__ void dense_again(const DenseJob<T>& J, const int64_t* s_
   __syncthreads();
   if (threadIdx.x < P && s_oct[0][pn] > NODES / 8) s_spike[pn] = kNoSpikes;
   __syncthreads();
-  if (!__syncthreads_or(s_spike[pn] != kNoSpikes) && sizeof(T) == 8) return;  // the first round's results stand
+  if (!__syncthreads_or(s_spike[pn] != kNoSpikes) && sizeof(T) == 8) return;  // the first pass's results stand
   if (threadIdx.x < P) s_max[pn] = 0;
   __syncthreads();
-  dense_round<DIM, T, CELL, true, NOCT>(J, base < 0 ? 0 : base, base >= 0, CELL ? (unsigned)s_colour[pn] : 0, s_max, s_oct,
+  dense_pass<DIM, T, CELL, true, NOCT>(J, base < 0 ? 0 : base, base >= 0, CELL ? (unsigned)s_colour[pn] : 0, s_max, s_oct,
                                         s_spike, s_any);
 }
 
@@ -962,7 +962,7 @@ __device__ __forceinline__ void dense_body(const DenseJob<T>& J, uint32_t batch)
     }
   }
   __syncthreads();  // the shared arrays
-  dense_round<DIM, T, CELL, false, NOCT>(J, base, active, edge, s_max, s_oct, s_spike, &s_any);
+  dense_pass<DIM, T, CELL, false, NOCT>(J, base, active, edge, s_max, s_oct, s_spike, &s_any);
   if constexpr (S::SPLIT) {
     if (s_any) dense_again<DIM, T, CELL, NOCT>(J, s_base, s_colour, s_max, s_oct, s_spike, &s_any);
   }
@@ -1077,9 +1077,9 @@ __global__ void __launch_bounds__(32 * PatchDense<DIM, T>::NW, PatchDense<DIM, T
 // FP64 operator apply on Cartesian meshes: cell results, one block of dst per
 // cell, then cell_sum per node.  The line passes (cart_pass) are bound by the
 // FP64 pipe; here it only sums the one to 2^d cells of a node.  One apply,
-// before and now: 3D K = 4 at 32^3 cells 0.231 and 0.112 ms, K = 2 at 100^3
-// 0.62 and 0.52, K = 3 at 67^3 0.72 and 0.43, K = 6 at 33^3 1.01 and 0.35,
-// K = 8 at 25^3 1.23 and 0.57; 2D K = 8 at 300^2 0.51 and 0.18.
+// by line passes and now: 3D K = 4 at 32^3 cells 0.231 and 0.118 ms, K = 2 at
+// 100^3 0.62 and 0.53, K = 3 at 67^3 0.72 and 0.45, K = 6 at 33^3 1.01 and
+// 0.36, K = 8 at 25^3 1.23 and 0.53; 2D K = 8 at 300^2 0.51 and 0.19.
 template <int DIM>
 __global__ void __launch_bounds__(32 * CellDense<DIM>::NW, CellDense<DIM>::MINB())
     cell_dense_kernel(const __grid_constant__ DenseJob<double> J) {
@@ -1178,9 +1178,9 @@ __global__ void __launch_bounds__(256) cell_sum_group_kernel(const __grid_consta
 // in L2: patch_split (gather to fixed point, even / odd combinations), one
 // block per batch and sector for the products, patch_merge (back to the
 // nodes), one block per batch and pair of mirrored z planes.  Patch
-// launch, sum factorisation before and now: K = 7 at 28^3 cells 11.8 and 3.65
-// ms, at 12^3 1.02 and 0.35, at 4^3 0.123 and 0.106; K = 6 at 32^3 9.80 and
-// 2.76 ms (the matrix, 4-10 MB, is streamed from L2 for every 16 patches).
+// launch, sum factorisation before and now: K = 7 at 28^3 cells 11.8 and 3.91
+// ms, at 12^3 1.02 and 0.32, at 4^3 0.123 and 0.071; K = 6 at 32^3 9.75 and
+// 2.78 ms (the matrix, 4-10 MB, is streamed from L2 for every 16 patches).
 constexpr bool kStaged = PMG_PREC == 0 && PMG_DIM == 3 && (K == 6 || K == 7);
 constexpr int kStageBatches = 76;  // 8 sectors each: two waves of two blocks per SM
 
@@ -1255,7 +1255,7 @@ __device__ __forceinline__ void patch_split(const StageJob& G, uint32_t b) {
   if (threadIdx.x == 0) s_any = 0;
   __syncthreads();
 #pragma unroll 1
-  for (int round = 0;; ++round) {  // as in dense_body
+  for (int pass = 0;; ++pass) {  // as in dense_body
     const unsigned bound = s_spike[pn];
     unsigned mx = 0;
     for (int l = item0; l < M * M; l += STEP) {
@@ -1285,13 +1285,13 @@ __device__ __forceinline__ void patch_split(const StageJob& G, uint32_t b) {
         double r[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) r[i] = in ? q[i] : 0.0;
-        if (round) {
+        if (pass) {
 #pragma unroll
           for (int i = 0; i < M; ++i) r[i] = magnitude(r[i]) > bound ? 0.0 : r[i];
         }
         unsigned mag[M];
         sc.template fixed<M>(r, v[b], mag);
-        if (round == 0) add_octants(ln, b, [&](int i) { return mag[i]; }, s_oct, pn);
+        if (pass == 0) add_octants(ln, b, [&](int i) { return mag[i]; }, s_oct, pn);
       }
       reflect<DIM, M>(v);
       const int sh0 = 3 - DIM + ln.centres();
@@ -1307,7 +1307,7 @@ __device__ __forceinline__ void patch_split(const StageJob& G, uint32_t b) {
     if (threadIdx.x < P) {
       unsigned lo, hi;
       octant_range<NOCT>(s_oct, pn, lo, hi);
-      if (round == 0 && !sc.bad && !sc.subnormal && lo < hi >> kUnevenExp) {
+      if (pass == 0 && !sc.bad && !sc.subnormal && lo < hi >> kUnevenExp) {
         s_spike[pn] = spike_bound<double>(mx);
         s_any = 1;
       }
@@ -1316,7 +1316,7 @@ __device__ __forceinline__ void patch_split(const StageJob& G, uint32_t b) {
       words[P + pn] = (int)s_spike[pn];
     }
     __syncthreads();
-    if (round || !s_any) break;
+    if (pass || !s_any) break;
     if (s_spike[pn] != kNoSpikes) {  // as dense_again
       unsigned count = 0;
       for (int i = threadIdx.x / P; i < S::NODES; i += 256 / P)
@@ -1514,15 +1514,20 @@ __global__ void __launch_bounds__(256) patch_point_group_kernel(const __grid_con
 // ---------------------------------------------------------------- the matrix
 // Columns of B at unit scale (the FP64 part serves both precisions): the local
 // solver applied to the unit vectors of the orbits' first nodes, one node per
-// patch of the block; column[orbit][node], hi + lo.  A further local cycle (Algorithm 2,
-// N_iter > 1) continues from them.  For FP64 products V = dd: the matrix is
-// rounded once, where the local solver in plain FP64 would leave 2-5 times
-// the error of a solve in the products (K = 3: 1.1e-15 against 3.3e-16).
+// patch of the block; column[orbit][node], hi + lo (lo only with V = dd).  A
+// further local cycle (Algorithm 2, N_iter > 1) continues from them.  For FP64
+// products V = dd: the matrix is rounded once, where the local solver in plain
+// FP64 would leave 2-5 times the error of a solve in the products (K = 3:
+// 1.1e-15 against 3.3e-16).  orbitexp: set to kNoOrbit for sector_exponents_kernel.
+constexpr int kNoOrbit = 1 << 30;
+
 template <int DIM, typename V>
-__global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__ hi, double* __restrict__ lo, int np,
-                                                            bool first, const double* __restrict__ dinv,
-                                                            PatchParams<double> H) {
+__global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__ hi, double* __restrict__ lo,
+                                                            int* __restrict__ orbitexp, int np, bool first,
+                                                            const double* __restrict__ dinv, PatchParams<double> H) {
   using S = Sectors<DIM, kPatchM>;
+  if (sizeof(V) == 16 && blockIdx.x == 0)
+    for (int i = threadIdx.x; i < S::ORBITS; i += blockDim.x) orbitexp[i] = kNoOrbit;
   using PS = PatchShape<DIM>;
   constexpr int SZT = PS::SZT, RT = PS::off_r(PS::L - 1), DT = PS::off_d(PS::L - 1);
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -1560,7 +1565,6 @@ __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__
       hi[t] = v;
     } else {
       hi[t] = d;
-      lo[t] = 0.0;
     }
   });
 }
@@ -1568,10 +1572,12 @@ __global__ void __launch_bounds__(256) patch_columns_kernel(double* __restrict__
 // Columns of the element stiffness matrix of Eq. (3) at unit scale, from the
 // 1D element matrices; as patch_columns_kernel
 template <int DIM>
-__global__ void __launch_bounds__(256) cell_columns_kernel(double* __restrict__ hi, double* __restrict__ lo) {
+__global__ void __launch_bounds__(256) cell_columns_kernel(double* __restrict__ hi, double* __restrict__ lo,
+                                                           int* __restrict__ orbitexp) {
   constexpr int M = kCellM;
   using S = Sectors<DIM, M>;
   const int t = blockIdx.x * 256 + threadIdx.x;
+  if (t < S::ORBITS) orbitexp[t] = kNoOrbit;
   if (t >= S::ORBITS * S::NODES) return;
   const Orbit<DIM, M> o(t / S::NODES);
   const int i = t % S::NODES, c[3] = {i % M, (i / M) % M, i / (M * M)};
@@ -1600,18 +1606,20 @@ __device__ __forceinline__ Orbit<DIM, M> orbit_of(int s, int k) {
 // mirror images of om's node of the operator's entry for oj's node, over 2^d
 // -- the operand of an orbit with c central coordinates, which has only
 // 2^(d-c) images, counts 2^c times.
-template <int DIM, int M>
-__device__ __forceinline__ dd sector_entry(const double* __restrict__ hi, const double* __restrict__ lo, int s,
-                                           const Orbit<DIM, M>& om, const Orbit<DIM, M>& oj) {
+// V = dd, or double without lo.
+template <typename V, int DIM, int M>
+__device__ __forceinline__ V sector_entry(const double* __restrict__ hi, const double* __restrict__ lo, int s,
+                                          const Orbit<DIM, M>& om, const Orbit<DIM, M>& oj) {
   using S = Sectors<DIM, M>;
   const int64_t col = (int64_t)(oj.c[0] + S::E * (oj.c[1] + S::E * oj.c[2])) * S::NODES;
-  dd a(0.0);
+  V a(0.0);
 #pragma unroll
   for (int b = 0; b < S::IMAGES; ++b) {
     if (S::IMAGES > 1 && !oj.has(b)) continue;
     const int64_t t = col + om.node(b);
     const double sg = (__popc(s & b) & 1) ? -1.0 / S::IMAGES : 1.0 / S::IMAGES;
-    a += dd(sg * hi[t], sg * lo[t]);
+    if constexpr (sizeof(V) == 16) a += V(sg * hi[t], sg * lo[t]);
+    else a += sg * hi[t];
   }
   return a;
 }
@@ -1624,8 +1632,7 @@ __device__ __forceinline__ dd sector_entry(const double* __restrict__ hi, const 
 // minexp, the least one of the orbit's rows (kNoExp in the first if an entry is not finite).
 template <int DIM, int M>
 __global__ void __launch_bounds__(128) sector_exponents_kernel(const double* __restrict__ hi,
-                                                               const double* __restrict__ lo, int* __restrict__ rowexp,
-                                                               int* __restrict__ minexp) {
+                                                               int* __restrict__ rowexp, int* __restrict__ minexp) {
   using S = Sectors<DIM, M>;
   const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= S::ROWS) return;
@@ -1635,7 +1642,7 @@ __global__ void __launch_bounds__(128) sector_exponents_kernel(const double* __r
   const Orbit<DIM, M> om = orbit_of<DIM, M>(s, m);
   double top = 0.0, sum = 0.0;
   for (int k = lane; k < sz; k += 32) {
-    const double a = fabs(value_of(sector_entry<DIM, M>(hi, lo, s, om, orbit_of<DIM, M>(s, k))));
+    const double a = fabs(sector_entry<double, DIM, M>(hi, nullptr, s, om, orbit_of<DIM, M>(s, k)));
     top = fmax(top, a);
     sum += a;
   }
@@ -1686,7 +1693,8 @@ __global__ void __launch_bounds__(256) sector_table_kernel(const double* __restr
   for (int h = 0; h < 2; ++h) {
     const int k = k0 + h;
     const Orbit<DIM, M> oj = orbit_of<DIM, M>(s, k < sz ? k : 0);
-    const dd a = m < sz && k < sz ? sector_entry<DIM, M>(hi, lo, s, om, oj) : dd(0.0);
+    using V = std::conditional_t<sizeof(T) == 8, dd, double>;
+    const V a = m < sz && k < sz ? sector_entry<V, DIM, M>(hi, lo, s, om, oj) : V(0.0);
     if constexpr (sizeof(T) == 8) {
       const long long w = __double2ll_rn(scalbn(a.hi, re)) + __double2ll_rn(scalbn(a.lo, re));
       const unsigned long long v = (unsigned long long)w + D::BIAS;
@@ -1696,7 +1704,7 @@ __global__ void __launch_bounds__(256) sector_table_kernel(const double* __restr
       }
     } else {
       // FP32 operands are plain sums over the images
-      double rest = value_of(a) * (1 << oj.centres());
+      double rest = a * (1 << oj.centres());
       for (int i = 0; i < SL; ++i) {
         const __nv_bfloat16 p = __double2bfloat16(rest);
         rest -= (double)__bfloat162float(p);
