@@ -97,7 +97,7 @@ enum pmg_patch_layout {
 enum pmg_outer_apply {
   PMG_OUTER_APPLY_FP64 = 0,         /* IEEE double vectors (default).  Cartesian, degree >= 2 (2D: >= 3): exact
                                        products of the cells' values in 60-bit fixed point with the element
-                                       matrix; the error at every node is within about 30 (k + 1) roundings of
+                                       matrix; the error at every node is within 27 (k + 2) roundings of
                                        (|K|x|M|x|M| + ...) |x| (1D matrices, rounded themselves), whatever the
                                        range of x.  An infinity or NaN makes every result of its cells NaN */
   PMG_OUTER_APPLY_FLOAT_FLOAT = 1   /* FP64 vectors in and out, every product and sum carried as an unevaluated

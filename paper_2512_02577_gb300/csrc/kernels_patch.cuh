@@ -24,7 +24,7 @@
 // integers, keeping the 36 digit pairs i + j <= 7 (0-based).  The matrices are
 // formed in pairs of doubles, their results have one exponent per orbit of
 // mirrored nodes.  Windows whose values differ too much for one exponent:
-// kUneven below.  No FP64 instruction is executed but for subnormal windows
+// kUnevenExp below.  No FP64 instruction is executed but for subnormal windows
 // and results and for spikes.  Largest error of one local solve of a patch in
 // units of 2^-53 |B||r|, N(0,1) residuals, by sum factorisation and now: 3D K = 3 3.1,
 // 2.4; K = 4 3.5, 3.5; K = 5 3.7, 1.9; 2D K = 7 5.8, 3.4; K = 8 7.7, 5.6; with one
@@ -456,9 +456,9 @@ constexpr int kMagicBits = 0x4B400000;
 
 // FP64 products of one unit: result rows of sector coefficients times the
 // operand rows, in units of 2^-68 of (table integer x operand integer) at the
-// exponent of the row's orbit.  Two k tiles add at most 16 products of 2^18 to an
-// accumulator (within its exact range of 2^22 around kMagic) before it is
-// emptied into Y.
+// exponent of the row's orbit.  Two k tiles add at most 8 digit pairs of 32
+// products below 2^14 to an accumulator (its exact range is 2^22 around kMagic;
+// the first digits stay within 127) before it is emptied into Y.
 template <class D>
 __device__ __forceinline__ void dense_mma(const DenseUnit& u, const uint4* __restrict__ table,
                                           const int* __restrict__ shifts, const long long* X, long long* Y,
